@@ -393,10 +393,10 @@ ROKS_API roks_status roks_forces(roks_ctx* ctx, const void* psi, int64_t ld, dou
 /* Launch shapes in use (the autotuner's choices when roks_options.autotune
  * was set, else the defaults): the number of band groups of the density's
  * x-stage transform (2, 4 or 8; default 4) and the schedule of the
- * tensor-core A^H B products: 2 is a stream-K schedule over one wave of
- * one CTA per SM (each CTA an equal run of the (tile, K stage) units, the
- * tiles' partial sums added in K order; the default), 5 and 8 split K over
- * 2.5 or 4 waves.  candidate_ms: the timed candidates in that order (ms
+ * tensor-core A^H B products, a stream-K schedule whose (tile, K stage) units
+ * are cut into equal runs, one per CTA, the tiles' partial sums added in K
+ * order: 2 is one run per SM (the default), 5 and 8 cut 2.5 or 4 runs per
+ * SM.  candidate_ms: the timed candidates in that order (ms
  * per launch; 0 when not timed).  Host struct, filled before the call
  * returns. */
 typedef struct {

@@ -428,14 +428,14 @@ size_t gemm_cn_work(int M, int N, int K) {
 
 template <typename T>
 void gemm_cn(int M, int N, int K, const c2<T>* A, int64_t lda, const c2<T>* B, int64_t ldb, double2* C, int ldc,
-             double2* work, size_t work_elems, cudaStream_t st) {
+             double2* work, size_t work_elems, cudaStream_t st, const TcImage* ia, const TcImage* ib) {
     if (M <= 0 || N <= 0) return;
     const int max_chunks = (int)(work_elems / ((size_t)M * N));
     if constexpr (sizeof(T) == 4) {
         // mixed path: large blocks on the tcgen05 tensor cores, the rest on
         // the TMA-streamed SIMT kernel
         if (gemm_cn_tcg(M, N, K, reinterpret_cast<const float2*>(A), lda, reinterpret_cast<const float2*>(B), ldb, C,
-                        ldc, work, work_elems * sizeof(double2), st))
+                        ldc, work, work_elems * sizeof(double2), ia, ib, st))
             return;
         if (gemm_cn_stream(M, N, K, reinterpret_cast<const float2*>(A), lda, reinterpret_cast<const float2*>(B), ldb,
                            C, ldc, work, work_elems, st))
@@ -588,13 +588,13 @@ void launch_nn(int M, int N, int K, int ty, int nt, const c2<T>* A, int64_t lda,
 
 template <typename T>
 void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B, int ldb, c2<T>* C, int64_t ldc,
-             double alpha, double beta, void* bwork, cudaStream_t st, size_t bwork_bytes) {
+             double alpha, double beta, void* bwork, cudaStream_t st, size_t bwork_bytes, const TcImage* ia) {
     if (M <= 0 || N <= 0) return;
     if constexpr (sizeof(T) == 4) {
         if (bwork_bytes > 0 &&
             gemm_nn_tcg(M, N, K, reinterpret_cast<const float2*>(A), lda, B, ldb,
                         beta != 0.0 ? reinterpret_cast<const float2*>(C) : nullptr, ldc, reinterpret_cast<float2*>(C),
-                        ldc, (float)alpha, (float)beta, bwork, bwork_bytes, st))
+                        ldc, (float)alpha, (float)beta, bwork, bwork_bytes, ia, st))
             return;
     }
     // column tiles of at most 64: RN = ceil(tile / 8) columns per thread, TY <= 8 warps
@@ -629,13 +629,13 @@ void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B,
 template <typename T>
 void gemm_nn_io(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B, int ldb, const c2<T>* Cin,
                 int64_t ldcin, c2<T>* Cout, int64_t ldc, double alpha, double beta, void* bwork, cudaStream_t st,
-                size_t bwork_bytes) {
+                size_t bwork_bytes, const TcImage* ia) {
     if (M <= 0 || N <= 0) return;
     if constexpr (sizeof(T) == 4) {
         if (bwork_bytes > 0 &&
             gemm_nn_tcg(M, N, K, reinterpret_cast<const float2*>(A), lda, B, ldb, reinterpret_cast<const float2*>(Cin),
                         ldcin, reinterpret_cast<float2*>(Cout), ldc, (float)alpha, (float)beta, bwork, bwork_bytes,
-                        st))
+                        ia, st))
             return;
         if (gemm_nn_stream(M, N, K, reinterpret_cast<const float2*>(A), lda, B, ldb, bwork,
                            reinterpret_cast<const float2*>(Cin), ldcin, reinterpret_cast<float2*>(Cout), ldc,
@@ -649,18 +649,19 @@ void gemm_nn_io(int M, int N, int K, const c2<T>* A, int64_t lda, const double2*
 }
 
 template void gemm_nn_io<float>(int, int, int, const float2*, int64_t, const double2*, int, const float2*, int64_t,
-                                float2*, int64_t, double, double, void*, cudaStream_t, size_t);
+                                float2*, int64_t, double, double, void*, cudaStream_t, size_t, const TcImage*);
 template void gemm_nn_io<double>(int, int, int, const double2*, int64_t, const double2*, int, const double2*,
-                                 int64_t, double2*, int64_t, double, double, void*, cudaStream_t, size_t);
+                                 int64_t, double2*, int64_t, double, double, void*, cudaStream_t, size_t,
+                                 const TcImage*);
 
 template void gemm_cn<float>(int, int, int, const float2*, int64_t, const float2*, int64_t, double2*, int,
-                             double2*, size_t, cudaStream_t);
+                             double2*, size_t, cudaStream_t, const TcImage*, const TcImage*);
 template void gemm_cn<double>(int, int, int, const double2*, int64_t, const double2*, int64_t, double2*, int,
-                              double2*, size_t, cudaStream_t);
+                              double2*, size_t, cudaStream_t, const TcImage*, const TcImage*);
 template void gemm_nn<float>(int, int, int, const float2*, int64_t, const double2*, int, float2*, int64_t, double,
-                             double, void*, cudaStream_t, size_t);
+                             double, void*, cudaStream_t, size_t, const TcImage*);
 template void gemm_nn<double>(int, int, int, const double2*, int64_t, const double2*, int, double2*, int64_t,
-                              double, double, void*, cudaStream_t, size_t);
+                              double, double, void*, cudaStream_t, size_t, const TcImage*);
 
 // ------------------------------------------------------------------ small FP64 matrices
 // One warp per output element; the lanes split K and reduce with shuffles.

@@ -501,9 +501,16 @@ void set_smem(F* f, size_t bytes) {
 
 }  // namespace
 
-bool tensor_map_2d(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows,
-                   int box_cols, bool swizzle128) {
-    return encode_block(map, ptr, rows, cols, ld, box_rows, box_cols, swizzle128);
+// Tiled map of 64-bit words, dims[0] contiguous, strides (bytes) of the others
+bool tensor_map_words(CUtensorMap* map, const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides,
+                      const uint32_t* box) {
+    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+    if (!fn) return false;
+    const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, rank, const_cast<void*>(ptr),
+              reinterpret_cast<const cuuint64_t*>(dims), reinterpret_cast<const cuuint64_t*>(strides), box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool stream_enabled() {

@@ -1,52 +1,51 @@
 // k_tcgemm.cu -- complex FP32 contractions of the large blocks (hundreds of
 // bands, thousands of projectors) on the 5th-generation tensor cores
-// (tcgen05, kind::tf32), mixed-precision path:
+// (tcgen05, kind::f16), mixed-precision path:
 //
 //   CN:  C (M x N, FP64 out) = A^H B,          A: K x M, B: K x N (K: plane waves)
 //   NN:  Cout (M x N) = alpha A B + beta Cin,   A: M x K tall, B: K x N small (FP64)
 //
-// Real formulation.  Complex vectors are stored as interleaved (re, im)
-// pairs, so a complex dot product is a real one over 2K numbers taken as
-// stored from one operand (a'), against a rearranged copy of the other:
-//   CN  Re = a'.(br, bi),   Im = a'.(bi, -br)      (a' = conj taken by the pairing)
-//   NN  Re = a'.(br, -bi),  Im = a'.(bi, br)
-// The MMA's N side holds 64 complex columns as 128 rows: the 64 rows that
-// give the real parts, then the 64 that give the imaginary parts; one MMA of
-// M = 128, N = 128 yields both.
+// Precision (three FP16 products per FP32 product).  Every column x of an
+// operand is scaled by a power of two that puts its largest element into
+// [2^14, 2^15), then split as x = hi + lo, hi = fp16(x), lo = fp16(x - hi):
+// 22 significant bits for every element above 2^-29 of its column's largest
+// one, and an absolute error of 2^-40 of that largest one below.  A product
+// is lo.hi + hi.lo + hi.hi.  That is the accuracy of a TF32 split (the same
+// 11-bit significands) at twice the MMA rate and half the operand bytes.
+// The tensor cores' FP32 accumulation truncates, which biases long sums of
+// like-signed terms, so every stage (32 complex K) goes into a fresh
+// tensor-memory accumulator, the small cross terms first, and the drain warps
+// add the stage's result into FP32 sums in registers (round to nearest).
 //
-// Precision (three TF32 products per FP32 product): each operand value x is
-// split as x = hi + lo, hi = tf32(x), lo = tf32(x - hi), and each product is
-// lo.hi + hi.lo + hi.hi.  The tensor cores' FP32 accumulation truncates
-// instead of rounding, which biases long sums of like-signed terms (norms,
-// overlaps, diagonal-dominated rotations).  So every stage (32 reals: four
-// K-steps of 8) goes into a fresh tensor-memory accumulator, in the order
-// of the eight small cross terms first and the four hi.hi products last:
-// only those four additions meet a large partial sum (a bias near 1e-7 of
-// the stage's sum at most), and the drain warps add the stage's result into
-// FP32 sums in registers (round to nearest).  Four accumulators of 128
-// columns rotate, so the MMAs of the next stages run while the previous
-// ones drain.  (A drain per K-step was measured a third slower on the
-// mgo-120 products.)
+// Images.  A block X (rows x cols, column major) is split once per use, by
+// k_tcg_split, into an image in global memory that the MMAs can read as it
+// is: for each chunk q of 8 rows, part p (hi, lo) and plane (re, im), all
+// the column groups g of 8, each a 128-byte core matrix of 8 columns x 8
+// rows (16 bytes per column):
+//   byte ((4 q + 2 p + plane) G + g) 128 + 16 (col % 8) + 2 (row % 8).
+// The planes are kept apart, so a complex product is four real ones whose
+// operands the MMA descriptors choose, the minus sign being the instruction
+// descriptor's negate bit; one image serves as the A or the B of A^H B
+// (contraction over the rows: K-major operands) and as the A of A B
+// (contraction over the columns: MN-major).  It has the size of X itself.
+// A kernel that converts operands on their way through shared memory (the
+// TF32 form this replaces) repeats the conversion for every tile and spent
+// its time in the hand-over between conversion and MMA.
 //
-// One CTA per SM (200 KB of shared memory, all 512 tensor-memory columns),
-// 18 warps:
-//   warp 0      producer: 2-D tensor copies of the raw FP32 operand slices
-//               into three raw stages; NN: bulk copies of the pre-split B;
-//   warp 1      one thread issues the MMAs;
-//   warps 2-17  workers.  In iteration i a worker converts its share of
-//               stage i (split into TF32 hi and lo, build the N-side rows,
-//               store K-major core matrices of 8 rows x 16 bytes, no
-//               swizzle, into one of two operand stages) and then drains its
-//               block of stage i - 2's accumulator: the lane quadrant
-//               warp % 4 and 16 complex columns.  The lag of two cannot
-//               deadlock: converting stage i waits for the MMAs of stage
-//               i - 2, which need the drain of stage i - 6 (iteration i - 4)
-//               and the conversion of stage i - 2 (iteration i - 2), and
-//               draining stage i - 2 waits for those same MMAs.
+// One CTA per SM (192 KB of shared memory in three stages, all 512
+// tensor-memory columns), three warpgroups:
+//   warp 0      producer: one tensor copy per operand and stage;
+//   warp 1      one thread issues the 24 MMAs of a stage (M = 128, N = tn,
+//               K = 16) into one of two accumulators, 128 columns for the
+//               real parts and 128 for the imaginary parts;
+//   warps 4-11  drain: lane quadrant warp % 4, 64 complex columns each (128
+//               sums a thread: the first warpgroup gives them registers).
 // Every wait is bounded (the context's wait cap); a wait that gives up sets
 // a device flag and the CTA winds down: copies and MMAs in flight are waited
 // for with the default bound before the tensor memory is freed.
+#include <cooperative_groups.h>
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cstdint>
@@ -57,55 +56,26 @@
 
 namespace roks {
 
-// 2-D tensor map of a column-major complex FP32 block (k_stream.cu)
-bool tensor_map_2d(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows,
-                   int box_cols, bool swizzle128);
+// tiled map of 64-bit words (k_stream.cu)
+bool tensor_map_words(CUtensorMap* map, const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides,
+                      const uint32_t* box);
 
 static __device__ int g_tcg_timeout;
 
 namespace {
 
-constexpr int GB_M = 128;      // tile rows (tensor-memory lanes)
-constexpr int GB_NC = 64;      // complex columns of a tile
-constexpr int GB_NR = 128;     // N-side rows of a tile (real parts, then imaginary parts)
-constexpr int GB_KC = 16;      // complex K per stage
-constexpr int GB_KR = 32;      // real K per stage (four MMA K-steps of 8)
-constexpr int GB_RAW = 3;      // raw stages
-constexpr int GB_CONV = 2;     // operand stages
-constexpr int GB_ACC = 4;      // tensor-memory accumulators
-constexpr int GB_WORKERS = 16;    // worker warps
-constexpr int GB_THREADS = (2 + GB_WORKERS) * 32;
-constexpr uint32_t GB_PART = GB_M * GB_KR * 4;   // one split part (hi or lo) of a 128-row operand: 16 KB
-constexpr uint32_t GB_SLOT = 4 * GB_PART;        // A hi | A lo | B hi | B lo
-constexpr uint32_t GB_RAWA = GB_M * GB_KC * 8;   // 16 KB
-constexpr uint32_t GB_RAWB = GB_NC * GB_KC * 8;  // 8 KB (CN)
-constexpr uint32_t GB_TCOLS = GB_ACC * GB_NR;    // 512 columns
+constexpr int GB_M = 128;     // tile rows (tensor-memory lanes)
+constexpr int GB_NT = 128;    // most complex columns of a tile
+constexpr int GB_KC = 32;     // complex K per stage
+constexpr int GB_ST = 3;      // stages
+constexpr int GB_ACC = 2;     // accumulators (256 tensor-memory columns each)
+constexpr int GB_DRAIN = 8;   // drain warps
+constexpr int GB_THREADS = (4 + GB_DRAIN) * 32;
+constexpr uint32_t GB_ABYTES = GB_M * GB_KC * 8;      // 32 KB
+constexpr uint32_t GB_SLOT = 2 * GB_ABYTES;           // A, then B (tn x KC x 8 bytes)
+constexpr uint32_t GB_TCOLS = 512;
 constexpr uint32_t GB_DEFAULT_WAIT = 1u << 26;
-
-// byte offset of real element kr of row r in a K-major operand tile of
-// 32 reals per row: core matrix (r / 8, kr / 4) of 128 bytes, row r % 8 at
-// 16 (r % 8), element kr % 4 at 4 (kr % 4)
-__device__ __forceinline__ uint32_t cofs(int r, int kr) {
-    return (uint32_t)((((r >> 3) * (GB_KR / 4) + (kr >> 2)) << 7) + ((r & 7) << 4) + ((kr & 3) << 2));
-}
-
-__device__ __forceinline__ void split4(const float4 v, float4& hi, float4& lo) {
-    hi.x = tc::to_tf32(v.x);
-    hi.y = tc::to_tf32(v.y);
-    hi.z = tc::to_tf32(v.z);
-    hi.w = tc::to_tf32(v.w);
-    lo.x = tc::to_tf32(v.x - hi.x);
-    lo.y = tc::to_tf32(v.y - hi.y);
-    lo.z = tc::to_tf32(v.z - hi.z);
-    lo.w = tc::to_tf32(v.w - hi.w);
-}
-
-__device__ __forceinline__ void put_split(unsigned char* hi_base, uint32_t off, const float4 v) {
-    float4 h, l;
-    split4(v, h, l);
-    *reinterpret_cast<float4*>(hi_base + off) = h;
-    *reinterpret_cast<float4*>(hi_base + GB_PART + off) = l;
-}
+constexpr size_t GB_SMEM = (size_t)GB_ST * GB_SLOT + 1024;
 
 // Bounded wait on a phase; gives up after `cap` polls, or early once another
 // role of the CTA has given up (checked every 1024 polls).
@@ -130,87 +100,51 @@ __device__ __forceinline__ void give_up(volatile int* failed) {
     g_tcg_timeout = 1;
 }
 
-// Shared-memory plan of a variant: operand slots (A hi | A lo | B hi | B lo)
-// and raw stages.  APRE: A arrives pre-split (k_tcg_asplit), copied by the
-// producer straight into the slot, so the slots can be three deep; the tall
-// product P Y takes it (B is pre-split as well: no raw stage, no conversion,
-// the worker warps only drain).  The plan also covers A^H B with a pre-split
-// A (raw stages of B alone), which gemm_cn_tcg does not launch: it measured
-// slower than converting both operands in the kernel.
-template <bool NN, bool APRE>
-struct GbPlan {
-    static constexpr int SLOTS = APRE ? 3 : GB_CONV;
-    static constexpr uint32_t RAWA = APRE ? 0u : GB_RAWA;       // raw A bytes per stage
-    static constexpr uint32_t RAWB = NN ? 0u : GB_RAWB;         // raw B bytes per stage
-    static constexpr uint32_t RAWS = RAWA + RAWB;                // bytes of one raw stage
-    static constexpr bool RAW = RAWA + RAWB > 0;                // a TMA raw stage per K stage
-    static constexpr bool CONVERT = RAW;                        // workers convert raw operands
-    static constexpr bool BULK = NN || APRE;                    // bulk copies into the slot
-    static constexpr uint32_t BULK_BYTES = (NN ? 2 * GB_PART : 0u) + (APRE ? 2 * GB_PART : 0u);
-    static constexpr size_t SMEM = (size_t)SLOTS * GB_SLOT + (RAW ? (size_t)GB_RAW * RAWS : 0) + 1024;
-    static constexpr int LAG = CONVERT ? 2 : 0;                 // drain of stage i - LAG in iteration i
-};
+// 2^e as a float, e in [-126, 127]
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
-// CTA-loop schedules (the kernel's SK instance), one CTA per SM:
-// * A^H B, stream-K: CTA c takes units units * c / ctas .. units * (c + 1) /
-//   ctas - 1 of the (tile, stage) sequence, stage fastest (tile t: M tile
-//   t % fast, N tile t / fast), and writes the partial sums of each tile it
-//   touches to its segment slot c * maxseg + (t - its first tile);
+// CTA-loop schedules, at most one CTA per SM:
+// * A^H B, stream-K: CTA c takes the units c len .. (c + 1) len - 1 of the
+//   (tile, stage) sequence, stage fastest (tile t: M tile t % fast, N tile t /
+//   fast), and writes the partial sums of each tile it touches to its segment
+//   slot c * maxseg + (t - its first tile);
 // * A B, persistent: units = tiles, CTA c takes the whole tiles c, c + ctas,
 //   ... (tile t: N tile t % fast, M tile t / fast), its pipeline running on
 //   across them, and writes each tile's result as it completes.
-// ctas = 0: one tile (and one K range) per CTA of a 3-D grid.
 struct SkPlan {
-    int64_t units = 0;
+    int64_t units = 0, len = 0;
     int ctas = 0, maxseg = 0, fast = 0;
+    int tn = 0;   // complex columns of a tile (a multiple of 16)
 };
 
-template <bool NN, bool APRE, bool SK = false>
+template <bool NN>
 __global__ void __launch_bounds__(GB_THREADS, 1)
-    k_tcgemm(int M, int N, int stages_per_cta, int total_stages, SkPlan sk, const __grid_constant__ CUtensorMap tmA,
-             const __grid_constant__ CUtensorMap tmB, const unsigned char* __restrict__ bsplit,
-             const unsigned char* __restrict__ asplit, float2* __restrict__ part, const float2* Cin, int64_t ldcin,
-             float2* Cout, int64_t ldc, float alpha, float beta, uint32_t wcap) {
-    using PL = GbPlan<NN, APRE>;
-    constexpr int SL = PL::SLOTS;
+    k_tcgemm(int M, int N, int total_stages, SkPlan sk, const __grid_constant__ CUtensorMap tmA,
+             const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exB, float2* __restrict__ part,
+             const float2* Cin, int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, uint32_t wcap) {
     extern __shared__ __align__(1024) unsigned char gb_smem[];
-    __shared__ __align__(8) uint64_t raw_full[GB_RAW], raw_empty[GB_RAW], conv_full[SL], conv_empty[SL], b_full[SL],
-        acc_full[GB_ACC], acc_empty[GB_ACC], mma_done;
+    __shared__ __align__(8) uint64_t full[GB_ST], empty[GB_ST], acc_full[GB_ACC], acc_empty[GB_ACC], mma_done;
     __shared__ uint32_t tmem_base;
     __shared__ volatile int failed;
-    unsigned char* base = gb_smem + ((1024u - (tc::smem_u32(gb_smem) & 1023u)) & 1023u);
-    unsigned char* conv = base;                                // SL operand slots
-    unsigned char* raw = base + (size_t)SL * GB_SLOT;          // GB_RAW raw stages (1024-byte aligned)
+    unsigned char* ring = gb_smem + ((1024u - (tc::smem_u32(gb_smem) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // CN: grid (M tiles, N tiles, K splits).  NN: grid (N tiles, M tiles),
-    // so that the CTAs sharing one tile of the tall A run side by side and A
-    // comes from DRAM about once (M fastest re-read it once per N tile)
-    const int mi = NN ? blockIdx.y : blockIdx.x, ni = NN ? blockIdx.x : blockIdx.y;
-    const int m0 = mi * GB_M, n0 = ni * GB_NC;
-    const int s0 = NN ? 0 : blockIdx.z * stages_per_cta;
-    const int64_t u0 = (SK && !NN) ? sk.units * blockIdx.x / sk.ctas : 0;
-    // CTA loop: the first tile and stage (the loops then step them); after a
-    // tile's last stage the next tile is t + tstep
-    const int t_first = SK ? (NN ? (int)blockIdx.x : (int)(u0 / total_stages)) : 0;
-    const int s_first = (SK && !NN) ? (int)(u0 - (int64_t)t_first * total_stages) : 0;
-    const int tstep = (SK && NN) ? sk.ctas : 1;
-    const int ns = NN ? (SK ? (int)((sk.units - blockIdx.x + sk.ctas - 1) / sk.ctas) * total_stages : total_stages)
-                      : (SK ? (int)(sk.units * (blockIdx.x + 1) / sk.ctas - u0)
-                            : max(0, min(total_stages, s0 + stages_per_cta) - s0));
+    const int64_t u0 = NN ? 0 : sk.len * blockIdx.x;
+    // the first tile and stage (the loops then step them); after a tile's
+    // last stage the next tile is t + tstep
+    const int t_first = NN ? (int)blockIdx.x : (int)(u0 / total_stages);
+    const int s_first = NN ? 0 : (int)(u0 - (int64_t)t_first * total_stages);
+    const int tstep = NN ? sk.ctas : 1;
+    const int ns = NN ? (int)((sk.units - blockIdx.x + sk.ctas - 1) / sk.ctas) * total_stages
+                      : (int)(min(sk.units, u0 + sk.len) - u0);
 
     if (tid == 0) {
-        for (int s = 0; s < GB_RAW; ++s) {
-            tc::mbar_init(&raw_full[s], 1);
-            tc::mbar_init(&raw_empty[s], GB_WORKERS);
-        }
-        for (int s = 0; s < SL; ++s) {
-            tc::mbar_init(&conv_full[s], GB_WORKERS);
-            tc::mbar_init(&conv_empty[s], 1);
-            tc::mbar_init(&b_full[s], 1);
+        for (int s = 0; s < GB_ST; ++s) {
+            tc::mbar_init(&full[s], 1);
+            tc::mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < GB_ACC; ++s) {
             tc::mbar_init(&acc_full[s], 1);
-            tc::mbar_init(&acc_empty[s], GB_WORKERS);
+            tc::mbar_init(&acc_empty[s], GB_DRAIN);
         }
         tc::mbar_init(&mma_done, 1);
         failed = 0;
@@ -221,250 +155,192 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_base;
+    const uint32_t wb = (uint32_t)sk.tn * 16u;   // bytes of one (q, part, plane) row of the B tile
 
-    if (warp == 0) {
+    // 384 threads x 168 registers at launch = 128 x 56 + 256 x 224
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------ producer
-        if (lane == 0) {
-            int issued = 0, bissued = 0;
-            int t_cur = t_first, s_cur = s_first;
+        if (warp == 0 && lane == 0) {
+            int issued = 0, t_cur = t_first, s_cur = s_first;
             for (int i = 0; i < ns; ++i) {
-                // this stage's tile (M tile ma, N tile nb_) and K stage ks_
-                int ma = mi, nb_ = ni, ks_ = s0 + i;
-                if (SK) {
-                    ma = NN ? t_cur / sk.fast : t_cur % sk.fast;
-                    nb_ = NN ? t_cur % sk.fast : t_cur / sk.fast;
-                    ks_ = s_cur;
-                    if (++s_cur == total_stages) {
-                        s_cur = 0;
-                        t_cur += tstep;
-                    }
+                const int ma = NN ? t_cur / sk.fast : t_cur % sk.fast;
+                const int nb_ = NN ? t_cur % sk.fast : t_cur / sk.fast;
+                const int ks = s_cur;
+                if (++s_cur == total_stages) {
+                    s_cur = 0;
+                    t_cur += tstep;
                 }
-                if (PL::RAW) {
-                    const int rs = i % GB_RAW;
-                    if (i >= GB_RAW && !gwait(&raw_empty[rs], (uint32_t)((i / GB_RAW - 1) & 1), wcap, &failed)) {
-                        give_up(&failed);
-                        break;
-                    }
-                    unsigned char* ra = raw + (size_t)rs * PL::RAWS;
-                    const int k0 = ks_ * GB_KC, am = ma * GB_M, bn = nb_ * GB_NC;
-                    if (NN) {
-                        tc::mbar_arrive_expect_tx(&raw_full[rs], GB_RAWA);
-                        tc::tma_2d(ra, &tmA, am, k0, &raw_full[rs]);
-                    } else {
-                        tc::mbar_arrive_expect_tx(&raw_full[rs], PL::RAWA + PL::RAWB);
-                        if (!APRE) tc::tma_2d(ra, &tmA, k0, am, &raw_full[rs]);
-                        tc::tma_2d(ra + PL::RAWA, &tmB, k0, bn, &raw_full[rs]);
-                    }
-                    issued = i + 1;
+                const int sl = i % GB_ST;
+                if (i >= GB_ST && !gwait(&empty[sl], (uint32_t)((i / GB_ST - 1) & 1), wcap, &failed)) {
+                    give_up(&failed);
+                    break;
                 }
-                if (PL::BULK) {
-                    // pre-split operands go straight into the operand slot
-                    const int cs = i % SL;
-                    if (i >= SL && !gwait(&conv_empty[cs], (uint32_t)((i / SL - 1) & 1), wcap, &failed)) {
-                        give_up(&failed);
-                        break;
-                    }
-                    unsigned char* sl = conv + (size_t)cs * GB_SLOT;
-                    tc::mbar_arrive_expect_tx(&b_full[cs], PL::BULK_BYTES);
-                    if (APRE)
-                        tc::bulk_g2s(sl, asplit + ((size_t)ma * total_stages + ks_) * (2 * GB_PART),
-                                     2 * GB_PART, &b_full[cs]);
-                    if (NN)
-                        tc::bulk_g2s(sl + 2 * GB_PART,
-                                     bsplit + ((size_t)nb_ * total_stages + ks_) * (2 * GB_PART), 2 * GB_PART,
-                                     &b_full[cs]);
-                    bissued = i + 1;
-                }
+                unsigned char* a = ring + (size_t)sl * GB_SLOT;
+                tc::mbar_arrive_expect_tx(&full[sl], GB_ABYTES + 16u * wb);
+                // A: CN 16 groups x 4 chunks of rows, NN 16 chunks x 4 groups
+                if (NN) tc::tma_4d(a, &tmA, ma * 16, ks * 4, 0, &full[sl]);
+                else tc::tma_2d(a, &tmA, ma * 256, ks * 16, &full[sl]);
+                tc::tma_2d(a + GB_ABYTES, &tmB, nb_ * sk.tn * 2, ks * 16, &full[sl]);
+                issued = i + 1;
             }
             // copies still in flight complete before the CTA may exit
-            for (int i = issued > GB_RAW ? issued - GB_RAW : 0; i < issued; ++i)
-                gwait(&raw_full[i % GB_RAW], (uint32_t)((i / GB_RAW) & 1), GB_DEFAULT_WAIT, &failed);
-            for (int i = bissued > SL ? bissued - SL : 0; i < bissued; ++i)
-                gwait(&b_full[i % SL], (uint32_t)((i / SL) & 1), GB_DEFAULT_WAIT, &failed);
+            for (int i = issued > GB_ST ? issued - GB_ST : 0; i < issued; ++i)
+                gwait(&full[i % GB_ST], (uint32_t)((i / GB_ST) & 1), GB_DEFAULT_WAIT, &failed);
         }
-        __syncwarp();
-    } else if (warp == 1) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_tf32(GB_M, GB_NR);
-            constexpr uint32_t LBO = 128, SBO = (GB_KR / 4) * 128;
+        if (warp == 1 && lane == 0) {
+            // A: K-major over [chunk 8192][part 4096][plane 2048][group 128], or
+            // MN-major over [part 16384][plane 8192][group 2048][chunk 128];
+            // B: K-major over [chunk 4 wb][part 2 wb][plane wb][group 128]
+            const uint32_t idesc = tc::idesc_f16(GB_M, sk.tn) | (NN ? tc::IDESC_A_MN : 0u);
+            const uint64_t da0 = NN ? tc::make_desc(0, 2048, 128) : tc::make_desc(0, 8192, 128);
+            const uint64_t db0 = tc::make_desc(0, 4 * wb, 128);
+            constexpr uint32_t a_part = NN ? 16384 : 4096, a_plane = NN ? 8192 : 2048, a_k = NN ? 4096 : 16384;
             bool ok = true;
-            int u = 0;
             for (int i = 0; i < ns && ok; ++i) {
-                const int cs = i % SL;
-                const uint32_t par = (uint32_t)((i / SL) & 1);
-                if ((PL::CONVERT && !gwait(&conv_full[cs], par, wcap, &failed)) ||
-                    (PL::BULK && !gwait(&b_full[cs], par, wcap, &failed))) {
+                const int sl = i % GB_ST, b = i % GB_ACC;
+                if (!gwait(&full[sl], (uint32_t)((i / GB_ST) & 1), wcap, &failed) ||
+                    (i >= GB_ACC && !gwait(&acc_empty[b], (uint32_t)((i / GB_ACC - 1) & 1), wcap, &failed))) {
                     ok = false;
                     break;
                 }
                 tc::fence_after_sync();
-                const uint32_t sa = tc::smem_u32(conv + (size_t)cs * GB_SLOT);
-                // one accumulator per stage
-                const int b = u % GB_ACC;
-                if (u >= GB_ACC && !gwait(&acc_empty[b], (uint32_t)((u / GB_ACC - 1) & 1), wcap, &failed)) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t d = tmem + (uint32_t)(b * GB_NR);
-                // small cross terms of the four K-steps first (8 reals = two K chunks of 128 bytes) ...
-                for (int kk = 0; kk < GB_KR / 8; ++kk) {
-                    const uint32_t ko = (uint32_t)kk * 256u;
-                    tc::mma_tf32(d, tc::make_desc(sa + GB_PART + ko, LBO, SBO),
-                                 tc::make_desc(sa + 2 * GB_PART + ko, LBO, SBO), idesc, kk > 0 ? 1u : 0u);
-                    tc::mma_tf32(d, tc::make_desc(sa + ko, LBO, SBO), tc::make_desc(sa + 3 * GB_PART + ko, LBO, SBO),
-                                 idesc, 1u);
-                }
-                // ... then the hi.hi products
-                for (int kk = 0; kk < GB_KR / 8; ++kk) {
-                    const uint32_t ko = (uint32_t)kk * 256u;
-                    tc::mma_tf32(d, tc::make_desc(sa + ko, LBO, SBO), tc::make_desc(sa + 2 * GB_PART + ko, LBO, SBO),
-                                 idesc, 1u);
+                const uint32_t sa = tc::smem_u32(ring + (size_t)sl * GB_SLOT), sb = sa + GB_ABYTES;
+                const uint32_t d = tmem + (uint32_t)(b * 256);
+                // D(out) += A(part pa, plane xa) B(part pb, plane xb) over the stage's two K-steps of 16
+                auto mm = [&](int out, int pa, int xa, int pb, int xb, bool neg, uint32_t first) {
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk)
+                        tc::mma_f16(d + 128u * out, da0 + ((sa + pa * a_part + xa * a_plane + kk * a_k) >> 4),
+                                    db0 + ((sb + pb * 2 * wb + xb * wb + kk * 8 * wb) >> 4),
+                                    neg ? (idesc | tc::IDESC_NEG_A) : idesc, (first && kk == 0) ? 0u : 1u);
+                };
+                // the small cross terms first, then the hi.hi products, which alone
+                // meet a large partial sum.  CN: re = Ar.Br + Ai.Bi, im = Ar.Bi -
+                // Ai.Br; NN: re = Ar.Br - Ai.Bi, im = Ar.Bi + Ai.Br.  The last
+                // products are those with Br: in A B, where B is near a real
+                // multiple of the identity or has a real diagonal, its large
+                // elements are then truncated least often
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const bool n0 = !NN && o == 1, n1 = NN && o == 0;   // the terms with Br, with Bi
+                    mm(o, 1, 1 - o, 0, 1, n1, 1u);
+                    mm(o, 0, 1 - o, 1, 1, n1, 0u);
+                    mm(o, 1, o, 0, 0, n0, 0u);
+                    mm(o, 0, o, 1, 0, n0, 0u);
+                    mm(o, 0, 1 - o, 0, 1, n1, 0u);
+                    mm(o, 0, o, 0, 0, n0, 0u);
                 }
                 tc::commit(&acc_full[b]);
-                ++u;
-                tc::commit(&conv_empty[cs]);   // the operand slot is free once these MMAs complete
+                tc::commit(&empty[sl]);   // the slot is free once these MMAs complete
             }
             if (!ok) give_up(&failed);
             // every MMA issued completes before the tensor memory is freed
             tc::commit(&mma_done);
             gwait(&mma_done, 0u, GB_DEFAULT_WAIT, &failed);
         }
-        __syncwarp();
+        __syncwarp();   // the role's lane rejoins its warp
     } else {
-        // ------------------------------------------------ workers: conversion, then drain
-        const int wt = tid - 64;                // 0 .. 32 GB_WORKERS - 1
-        const int q = warp & 3;                 // lane quadrant
-        const int cg = (warp - 2) >> 2;         // complex columns 16 cg .. 16 cg + 15
-        const int r = 32 * q + lane;            // tile row of the drain
-        const int rr = wt & 127, c0 = wt >> 7;  // conversion of A: row rr, chunks c0 and c0 + 4
-        float re[16], im[16];
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        // ------------------------------------------------ drain
+        const int q = warp & 3;               // lane quadrant
+        const int cg = 64 * ((warp - 4) >> 2);   // complex columns cg .. cg + 63
+        const int r = 32 * q + lane;          // tile row
+        // What the truncating additions of a stage take from its sum, given
+        // back: A^H B's long sums of like sign lose 2.3e-7 of their size
+        // (measured on the norms of 11,075 plane waves; four additions of
+        // half a unit in the last place each, and those inside an MMA), nearly
+        // 2^-22.  The products with the small B of A B lose no measurable part.
+        constexpr float gain = NN ? 1.f : 1.f + 0x1p-22f;
+        float2 re[32], im[32];                // column pairs
 #pragma unroll
-        for (int j = 0; j < 16; ++j) re[j] = im[j] = 0.f;
+        for (int j = 0; j < 32; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
         bool ok = true;
-        // CTA loop: stages left in the current tile's segment, its index,
-        // and its tile
-        int left = total_stages - s_first, seg = 0, t_drain = t_first;
-        // A B: this thread's row and 16 columns of the tile at (mo, no),
-        // times alpha, plus beta Cin
-        auto write_nn = [&](int mo, int no) {
-            const int m = mo + r;
-            if (m >= M) return;
+        int left = total_stages - s_first, seg = 0, t_cur = t_first;
+        for (int i = 0; i < ns; ++i) {
+            const int b = i % GB_ACC;
+            if (!warp_wait(&acc_full[b], (uint32_t)((i / GB_ACC) & 1), wcap, &failed)) {
+                ok = false;
+                break;
+            }
+            tc::fence_after_sync();
+            const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * 256 + cg);
+            if (NN && beta != 0.f && left == total_stages && (lane & 15) == 0) {
+                // a tile's first stage: its Cin on the way to L2
+                const int no = (t_cur % sk.fast) * sk.tn + cg, m = (t_cur / sk.fast) * GB_M + r;
+                const int nc = min(sk.tn - cg, N - no);
+                for (int j = 0; j < nc && m < M; ++j)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(Cin + (int64_t)(no + j) * ldcin + m));
+            }
+            if (cg < sk.tn) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int n = no + 16 * cg + j;
-                if (n < N) {
-                    float2 o = make_float2(alpha * re[j], alpha * im[j]);
-                    if (beta != 0.f) {
-                        const float2 ci = Cin[(int64_t)n * ldcin + m];
-                        o.x = fmaf(beta, ci.x, o.x);
-                        o.y = fmaf(beta, ci.y, o.y);
+                for (int c = 0; c < 4; ++c) {
+                    float v[16], w[16];
+                    tc::tmem_ld16_nowait(ta + 16 * c, v);
+                    tc::tmem_ld16_nowait(ta + 128 + 16 * c, w);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float2 g2 = make_float2(gain, gain);
+                        re[8 * c + j] = __ffma2_rn(make_float2(v[2 * j], v[2 * j + 1]), g2, re[8 * c + j]);
+                        im[8 * c + j] = __ffma2_rn(make_float2(w[2 * j], w[2 * j + 1]), g2, im[8 * c + j]);
                     }
-                    Cout[(int64_t)n * ldc + m] = o;
                 }
             }
-        };
-        for (int i = 0; i < ns + PL::LAG; ++i) {
-            if (PL::CONVERT && i < ns) {
-                const int rs = i % GB_RAW, cs = i % SL;
-                if (!warp_wait(&raw_full[rs], (uint32_t)((i / GB_RAW) & 1), wcap, &failed) ||
-                    (i >= SL && !warp_wait(&conv_empty[cs], (uint32_t)((i / SL - 1) & 1), wcap, &failed))) {
-                    ok = false;
-                    break;
-                }
-                const unsigned char* ra = raw + (size_t)rs * PL::RAWS;
-                unsigned char* sl = conv + (size_t)cs * GB_SLOT;
-                if (!NN) {
-                    if (!APRE) {
-                        // A row rr (column rr of A): 16 complex in eight 16-byte chunks,
-                        // stored by the copy with the 128-byte swizzle
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&acc_empty[b]);
+            // the last stage of a tile in this CTA's run: its sums go out (NN:
+            // the result; CN: the partial sums to the segment slot) and restart
+            if (--left == 0 || i == ns - 1) {
+                if (NN) {
+                    const int m = (t_cur / sk.fast) * GB_M + r;
+                    const int no = (t_cur % sk.fast) * sk.tn + cg;
+                    const int nc = min(sk.tn - cg, N - no);   // this warp's columns
+                    if (m < M) {
+                        // 32 columns at a time, every load before the first store
+                        // (Cin may be Cout, so the compiler keeps their order: one
+                        // load in flight per thread took 25 us a tile)
 #pragma unroll
-                        for (int h2 = 0; h2 < 2; ++h2) {
-                            const int ch = c0 + 4 * h2;
-                            const float4 v =
-                                *reinterpret_cast<const float4*>(ra + rr * 128 + ((ch ^ (rr & 7)) << 4));
-                            put_split(sl, cofs(rr, 4 * ch), v);
+                        for (int c = 0; c < 2; ++c) {
+                            float2 ci[32];
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) {
+                                const int jj = 32 * c + j;
+                                ci[j] = make_float2(0.f, 0.f);
+                                if (beta != 0.f && jj < nc) ci[j] = Cin[(int64_t)(no + jj) * ldcin + m];
+                            }
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) {
+                                const int jj = 32 * c + j;
+                                if (jj < nc) {
+                                    const float2 x = re[jj >> 1], y = im[jj >> 1];
+                                    const float sc = alpha * pow2f(-exB[no + jj]);
+                                    const float2 o = (j & 1) ? make_float2(sc * x.y, sc * y.y)
+                                                             : make_float2(sc * x.x, sc * y.x);
+                                    Cout[(int64_t)(no + jj) * ldc + m] =
+                                        make_float2(fmaf(beta, ci[j].x, o.x), fmaf(beta, ci[j].y, o.y));
+                                }
+                            }
                         }
                     }
-                    // B column j, chunk ch: the real-part row (re, im) and the
-                    // imaginary-part row (im, -re)
-                    const int j = wt & 63, ch = wt >> 6;
-                    const float4 v =
-                        *reinterpret_cast<const float4*>(ra + PL::RAWA + j * 128 + ((ch ^ (j & 7)) << 4));
-                    put_split(sl + 2 * GB_PART, cofs(j, 4 * ch), v);
-                    put_split(sl + 2 * GB_PART, cofs(GB_NC + j, 4 * ch), make_float4(v.y, -v.x, v.w, -v.z));
                 } else {
-                    // A row rr (plane wave m0 + rr): the raw slice is [k][m], 1 KB per k
+                    float2* Pp = part + (((int64_t)blockIdx.x * sk.maxseg + seg) * sk.tn + cg) * GB_M + r;
 #pragma unroll
-                    for (int h2 = 0; h2 < 2; ++h2) {
-                        const int ch = c0 + 4 * h2;
-                        const float2 a0 = *reinterpret_cast<const float2*>(ra + (2 * ch) * 1024 + rr * 8);
-                        const float2 a1 = *reinterpret_cast<const float2*>(ra + (2 * ch + 1) * 1024 + rr * 8);
-                        put_split(sl, cofs(rr, 4 * ch), make_float4(a0.x, a0.y, a1.x, a1.y));
-                    }
+                    for (int j = 0; j < 64; ++j)
+                        if (cg + j < sk.tn)
+                            Pp[(int64_t)j * GB_M] = (j & 1) ? make_float2(re[j >> 1].y, im[j >> 1].y)
+                                                            : make_float2(re[j >> 1].x, im[j >> 1].x);
                 }
-                tc::fence_async_smem();   // generic-proxy stores become visible to the tensor cores
-                __syncwarp();
-                if (lane == 0) {
-                    tc::mbar_arrive(&raw_empty[rs]);
-                    tc::mbar_arrive(&conv_full[cs]);
-                }
-            }
-            const int dsg = i - PL::LAG;
-            if (dsg >= 0) {
-                const int b = dsg % GB_ACC;
-                if (!warp_wait(&acc_full[b], (uint32_t)((dsg / GB_ACC) & 1), wcap, &failed)) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * GB_NR + 16 * cg);
-                float v[16], w[16];
-                tc::tmem_ld16_nowait(ta, v);
-                tc::tmem_ld16_nowait(ta + GB_NC, w);
-                tc::tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    re[j] += v[j];
-                    im[j] += w[j];
-                }
-                tc::fence_before_sync();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&acc_empty[b]);
-                if (SK) {
-                    // the last stage of a tile in this CTA's run: its sums
-                    // go out (A B: the result; A^H B: the partial sums to
-                    // the segment slot), and the sums restart
-                    if (--left == 0 || dsg == ns - 1) {
-                        if (NN) {
-                            write_nn((t_drain / sk.fast) * GB_M, (t_drain % sk.fast) * GB_NC);
-                        } else {
-                            float2* Pp = part + ((int64_t)blockIdx.x * sk.maxseg + seg) * GB_NC * GB_M;
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) Pp[(int64_t)(16 * cg + j) * GB_M + r] = make_float2(re[j], im[j]);
-                        }
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) re[j] = im[j] = 0.f;
-                        ++seg;
-                        t_drain += tstep;
-                        left = total_stages;
-                    }
-                }
+                for (int j = 0; j < 32; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
+                ++seg;
+                t_cur += tstep;
+                left = total_stages;
             }
         }
         if (!ok) give_up(&failed);
-        if (ok && !SK) {
-            if (NN) {
-                write_nn(m0, n0);
-            } else {
-                const int tile = blockIdx.x + blockIdx.y * gridDim.x;
-                const int tiles = gridDim.x * gridDim.y;
-                float2* P = part + ((int64_t)blockIdx.z * tiles + tile) * GB_NC * GB_M;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) P[(int64_t)(16 * cg + j) * GB_M + r] = make_float2(re[j], im[j]);
-            }
-        }
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -474,114 +350,196 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
     }
 }
 
-// A pre-split for the tall product A B, once per operand that does not
-// change (the projector matrix): for each (128-row tile t, stage s of 16
-// complex K) a block of hi (16 KB) then lo (16 KB) in the operand-slot
-// layout, element (r, kr) = real part kr & 1 of A(128 t + r, 16 s + kr / 2)
-// (A is M x K, column major).  Zero beyond M and K.
-__global__ void k_tcg_asplit(int M, int K, const float2* __restrict__ A, int64_t lda, int nst, int mt,
-                             unsigned char* __restrict__ out) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)mt * nst * GB_M * 8;
-    if (idx >= total) return;
-    const int ch = (int)(idx % 8);
-    const int rr = (int)((idx / 8) % GB_M);
-    const int s = (int)((idx / (8 * GB_M)) % nst);
-    const int t = (int)(idx / (8 * GB_M * nst));
-    const int m = t * GB_M + rr;
-    float v[4];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int k = s * GB_KC + 2 * ch + e;
-        float2 a = make_float2(0.f, 0.f);
-        if (k < K && m < M) a = A[(int64_t)k * lda + m];
-        v[2 * e] = a.x;
-        v[2 * e + 1] = a.y;
-    }
-    unsigned char* blk = out + ((size_t)t * nst + s) * (2 * GB_PART);
-    float4 hi, lo;
-    split4(make_float4(v[0], v[1], v[2], v[3]), hi, lo);
-    *reinterpret_cast<float4*>(blk + cofs(rr, 4 * ch)) = hi;
-    *reinterpret_cast<float4*>(blk + GB_PART + cofs(rr, 4 * ch)) = lo;
-}
+// ------------------------------------------------------------------ operand images
+// Column group g = blockIdx.y, its chunks of 8 rows shared out over the
+// cluster's CTAs (blockIdx.x): the columns' largest finite elements first
+// (reduced over the cluster), then the split.  Lane = chunk % 4 + 4 (column
+// % 8): a warp reads 256 contiguous bytes of each column and writes whole
+// 128-byte core matrices.  The second read of the block mostly comes from L2.
+// D: the element type (float2, or double2 for the small B of A B); exA: the
+// exponents of the A image it multiplies, taken out of B's rows; VEC: 16-byte
+// loads of float2 (the column bases are 16-byte aligned).
+constexpr int SP_THREADS = 256;
+constexpr int SP_CL = 8;
 
-// B (K x N complex FP64, ldb) -> the NN kernel's N-side operand: for each
-// (64-column tile t, stage s) a block of hi (16 KB) then lo (16 KB), rows
-// j < 64 (re, -im) and 64 + j (im, re) of column 64 t + j, K-major core
-// matrices; zero beyond K and N.
-__global__ void k_tcg_bsplit(int K, int N, const double2* __restrict__ B, int ldb, int nst, int nt,
-                             unsigned char* __restrict__ out) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)nt * nst * GB_NR * 8;
-    if (idx >= total) return;
-    const int ch = (int)(idx % 8);
-    const int r = (int)((idx / 8) % GB_NR);
-    const int s = (int)((idx / (8 * GB_NR)) % nst);
-    const int t = (int)(idx / (8 * GB_NR * nst));
-    const int n = t * GB_NC + (r % GB_NC);
-    float v[4];
+template <typename D, bool VEC>
+__device__ __forceinline__ void split_load(const D* __restrict__ col, int r0, int R, const int* __restrict__ exA,
+                                           float2 (&x)[8]) {
+    if constexpr (VEC) {
+        if (r0 + 8 <= R) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int k = s * GB_KC + 2 * ch + e;
-        double2 b = make_double2(0.0, 0.0);
-        if (k < K && n < N) b = B[(int64_t)n * ldb + k];
-        if (r < GB_NC) {
-            v[2 * e] = (float)b.x;
-            v[2 * e + 1] = -(float)b.y;
-        } else {
-            v[2 * e] = (float)b.y;
-            v[2 * e + 1] = (float)b.x;
+            for (int k = 0; k < 4; ++k) {
+                const float4 v = *reinterpret_cast<const float4*>(col + r0 + 2 * k);
+                x[2 * k] = make_float2(v.x, v.y);
+                x[2 * k + 1] = make_float2(v.z, v.w);
+            }
+            return;
         }
     }
-    unsigned char* blk = out + ((size_t)t * nst + s) * (2 * GB_PART);
-    const uint32_t off = (uint32_t)((((r >> 3) * (GB_KR / 4) + ch) << 7) + ((r & 7) << 4));
-    float4 hi, lo;
-    split4(make_float4(v[0], v[1], v[2], v[3]), hi, lo);
-    *reinterpret_cast<float4*>(blk + off) = hi;
-    *reinterpret_cast<float4*>(blk + GB_PART + off) = lo;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        x[k] = make_float2(0.f, 0.f);
+        if (r0 + k < R) {
+            const D v = col[r0 + k];
+            x[k] = make_float2((float)v.x, (float)v.y);
+            if (exA) {
+                const float s = pow2f(-exA[r0 + k]);
+                x[k].x *= s;
+                x[k].y *= s;
+            }
+        }
+    }
 }
 
-// C (M x N, FP64, ldc) = sum over the K splits of the CN partials, in split
-// order (FP64 sums).
-__global__ void k_tcg_reduce(int M, int N, int mt, int tiles, int ks, const float2* __restrict__ part,
-                             double2* __restrict__ C, int ldc) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)M * N) return;
-    const int m = (int)(idx % M), n = (int)(idx / M);
-    const int tile = (m / GB_M) + (n / GB_NC) * mt;
-    const int64_t off = ((int64_t)tile * GB_NC + (n % GB_NC)) * GB_M + (m % GB_M);
-    double sr = 0.0, si = 0.0;
-    for (int z = 0; z < ks; ++z) {
-        const float2 p = part[(int64_t)z * tiles * GB_NC * GB_M + off];
-        sr += (double)p.x;
-        si += (double)p.y;
+template <typename D, bool VEC>
+__global__ void __launch_bounds__(SP_THREADS) k_tcg_split(int R, int V, const D* __restrict__ X, int64_t ld, int Q,
+                                                          int G, const int* __restrict__ exA,
+                                                          unsigned char* __restrict__ img, int* __restrict__ ex) {
+    namespace cg = cooperative_groups;
+    __shared__ float red[SP_THREADS / 32][8];
+    __shared__ float mine[8], top[8];
+    cg::cluster_group cl = cg::this_cluster();
+    const int ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int g = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int vl = lane >> 2, v = 8 * g + vl;
+    const int per = (Q + ncl - 1) / ncl;
+    const int q1 = min(Q, (rank + 1) * per);
+    const D* col = X + (int64_t)(v < V ? v : 0) * ld;
+    const int R_ = v < V ? R : 0;   // columns past the end: zeros
+    float m = 0.f;
+    for (int q = rank * per + 4 * warp + (lane & 3); q < q1; q += SP_THREADS / 8) {
+        float2 x[8];
+        split_load<D, VEC>(col, 8 * q, R_, exA, x);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float a = fmaxf(fabsf(x[k].x), fabsf(x[k].y));
+            if (a <= 3.4028234e38f) {   // finite (an infinity must not scale the others away)
+                m = fmaxf(m, a);
+            } else {
+                if (fabsf(x[k].x) <= 3.4028234e38f) m = fmaxf(m, fabsf(x[k].x));
+                if (fabsf(x[k].y) <= 3.4028234e38f) m = fmaxf(m, fabsf(x[k].y));
+            }
+        }
     }
-    C[(int64_t)n * ldc + m] = make_double2(sr, si);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    if ((lane & 3) == 0) red[warp][vl] = m;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        float t = 0.f;
+        for (int w = 0; w < SP_THREADS / 32; ++w) t = fmaxf(t, red[w][threadIdx.x]);
+        mine[threadIdx.x] = t;
+    }
+    cl.sync();
+    if (threadIdx.x < 8) {
+        float t = 0.f;
+        for (int k = 0; k < ncl; ++k) t = fmaxf(t, cl.map_shared_rank(mine, k)[threadIdx.x]);
+        top[threadIdx.x] = t;
+    }
+    cl.sync();
+    // the exponent that puts the largest element into [2^14, 2^15)
+    const float t = top[vl];
+    int e = 0;
+    if (t > 0.f) e = min(126, 14 - ilogbf(t));
+    const float s = pow2f(e);
+    if (rank == 0 && threadIdx.x < 32 && (lane & 3) == 0) ex[v] = e;
+    for (int q = rank * per + 4 * warp + (lane & 3); q < q1; q += SP_THREADS / 8) {
+        float2 x[8];
+        split_load<D, VEC>(col, 8 * q, R_, exA, x);
+        uint4 o[4];   // hi re, hi im, lo re, lo im
+        __half2* h = reinterpret_cast<__half2*>(o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 a = make_float2(s * x[2 * k].x, s * x[2 * k + 1].x);   // two real parts
+            const float2 b = make_float2(s * x[2 * k].y, s * x[2 * k + 1].y);
+            const __half2 ha = __float22half2_rn(a), hb = __float22half2_rn(b);
+            const float2 fa = __half22float2(ha), fb = __half22float2(hb);
+            h[k] = ha;
+            h[4 + k] = hb;
+            h[8 + k] = __float22half2_rn(make_float2(a.x - fa.x, a.y - fa.y));
+            h[12 + k] = __float22half2_rn(make_float2(b.x - fb.x, b.y - fb.y));
+        }
+        unsigned char* dst = img + ((int64_t)4 * q * G + g) * 128 + 16 * vl;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) *reinterpret_cast<uint4*>(dst + (int64_t)k * G * 128) = o[k];
+    }
 }
 
-// The stream-K partials of tile t: the CTAs whose unit runs meet the tile's
-// units t T .. (t + 1) T - 1, in CTA (that is K) order, summed in FP64.
-__global__ void k_tcg_reduce_sk(int M, int N, int mt, int T, SkPlan sk, const float2* __restrict__ part,
-                                double2* __restrict__ C, int ldc) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)M * N) return;
-    const int m = (int)(idx % M), n = (int)(idx / M);
-    const int t = (m / GB_M) + (n / GB_NC) * mt;
-    const int64_t off = (int64_t)(n % GB_NC) * GB_M + (m % GB_M);
-    const int64_t ta = (int64_t)t * T, tb = ta + T;
-    int c = (int)(ta * sk.ctas / sk.units) - 1;
-    if (c < 0) c = 0;
-    double sr = 0.0, si = 0.0;
-    for (; c < sk.ctas; ++c) {
-        const int64_t a = sk.units * c / sk.ctas, b = sk.units * (c + 1) / sk.ctas;
-        if (a >= tb) break;
-        if (b <= ta || a == b) continue;   // no unit of the tile (or none at all)
-        const int seg = t - (int)(a / T);
-        const float2 p = part[((int64_t)c * sk.maxseg + seg) * GB_NC * GB_M + off];
-        sr += (double)p.x;
-        si += (double)p.y;
+template <typename D, bool VEC>
+bool launch_split(int R, int V, const D* X, int64_t ld, const int* exA, const TcImage& im, cudaStream_t st) {
+    const int Q = (R + 7) / 8, G = (V + 7) / 8;
+    cudaLaunchConfig_t cfg = {};
+    // a CTA's share of a column group is at least four rounds of its warps
+    int ncl = 1;
+    while (ncl < SP_CL && Q > 2 * ncl * SP_THREADS / 8) ncl *= 2;
+    cfg.gridDim = dim3(ncl, G, 1);
+    cfg.blockDim = dim3(SP_THREADS, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ncl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    roks::count_launch();
+    return cudaLaunchKernelEx(&cfg, k_tcg_split<D, VEC>, R, V, X, ld, Q, G, exA,
+                              static_cast<unsigned char*>(im.data), im.ex) == cudaSuccess;
+}
+
+// ------------------------------------------------------------------ partial sums
+// C (M x N, FP64) of tile t: the segments of the CTAs whose runs meet the
+// tile's units t T .. (t + 1) T - 1.  A warp covers 32 rows of one column; RG
+// warps of a block take every RG-th CTA of the tile, the block's other warps
+// further columns.  Compensated FP32 sums (FP64 arithmetic is slow on this
+// part), combined in warp order; the operands' scales come out at the end.
+// The order is fixed.
+template <int RG>
+__global__ void __launch_bounds__(256) k_tcg_reduce_sk(int M, int N, int mt, int T, SkPlan sk,
+                                                       const int* __restrict__ exA, const int* __restrict__ exB,
+                                                       const float2* __restrict__ part, double2* __restrict__ C,
+                                                       int ldc) {
+    constexpr int NW = 8 / RG;   // columns of a block
+    __shared__ float4 red[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wg = w % RG;
+    const int m = blockIdx.x * 32 + lane, n = blockIdx.y * NW + w / RG;
+    float sx = 0.f, cx = 0.f, sy = 0.f, cy = 0.f;
+    auto add = [](float& s, float& e, float v) {
+        const float u = s + v, bp = u - s;
+        e += (s - (u - bp)) + (v - bp);
+        s = u;
+    };
+    if (n < N) {
+        const int t = (blockIdx.x * 32) / GB_M + (n / sk.tn) * mt;
+        const int64_t off = (int64_t)(n % sk.tn) * GB_M + (m % GB_M);
+        const int64_t ta = (int64_t)t * T;
+        const int c0 = (int)(ta / sk.len), c1 = (int)((ta + T - 1) / sk.len);
+#pragma unroll 4
+        for (int c = c0 + wg; c <= c1; c += RG) {
+            // a run that starts before the tile has it further on
+            const int seg = c == c0 ? t - (int)(c0 * sk.len / T) : 0;
+            const float2 p = part[((int64_t)c * sk.maxseg + seg) * sk.tn * GB_M + off];
+            add(sx, cx, p.x);
+            add(sy, cy, p.y);
+        }
     }
-    C[(int64_t)n * ldc + m] = make_double2(sr, si);
+    if constexpr (RG > 1) {
+        red[w][lane] = make_float4(sx, cx, sy, cy);
+        __syncthreads();
+        if (wg > 0) return;
+        for (int k = 1; k < RG; ++k) {
+            const float4 v = red[w + k][lane];
+            add(sx, cx, v.x);
+            add(sy, cy, v.z);
+            cx += v.y;
+            cy += v.w;
+        }
+    }
+    if (m >= M || n >= N) return;
+    const double sc = __hiloint2double((1023 - exA[m] - exB[n]) << 20, 0);
+    C[(int64_t)n * ldc + m] =
+        make_double2(sc * ((double)sx + (double)cx), sc * ((double)sy + (double)cy));
 }
 
 int sm_count() {
@@ -599,68 +557,77 @@ int sm_count() {
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
-template <bool NN, bool APRE, bool SK = false>
+template <bool NN>
 void set_attr() {
     static bool done = false;
     if (!done) {
-        cudaFuncSetAttribute(k_tcgemm<NN, APRE, SK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)GbPlan<NN, APRE>::SMEM);
+        cudaFuncSetAttribute(k_tcgemm<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GB_SMEM);
         done = true;
     }
 }
 
-// Operands split once (tcg_presplit): looked up by address, leading
-// dimension and shape, so that a call on another matrix never takes them.
-struct PreSplit {
-    const void* A;
-    int64_t lda;
-    int M, K;
-    const unsigned char* split;
-};
-constexpr int kMaxPreSplit = 32;
-PreSplit g_pre[kMaxPreSplit];
-int g_npre = 0;
+int stages(int k) { return (k + GB_KC - 1) / GB_KC; }
+int tile_cols(int N, int nt) { return ((N + nt - 1) / nt + 15) / 16 * 16; }
 
-const unsigned char* find_presplit(const void* A, int64_t lda, int M, int K) {
-    static int on = -1;
-    if (on < 0) {
-        // ROKS_TC_PRESPLIT=0 converts every operand in the kernel (for comparisons)
-        const char* e = std::getenv("ROKS_TC_PRESPLIT");
-        on = (e && e[0] == '0') ? 0 : 1;
-    }
-    if (!on) return nullptr;
-    for (int i = 0; i < g_npre; ++i) {
-        const PreSplit& p = g_pre[i];
-        if (p.A == A && p.lda == lda && p.M == M && p.K == K) return p.split;
-    }
-    return nullptr;
-}
-
-// Schedule of A^H B (tcg_set_waves): 2 (the default) is the stream-K
-// schedule over one wave of one CTA per SM; 5 and 8 split K into 2.5 or 4
-// waves.  Stream-K removes the partial last wave of the split (P^H Psi at
-// mgo-120: 385 CTAs ran as 3 waves of 148): 1.45 -> 1.23 ms.
+// Runs of A^H B's unit sequence, in half waves of one CTA per SM
+// (tcg_set_waves): 2, one run per SM, is the default; the autotuner also
+// times 5 and 8, more and shorter runs.
 int g_waves_x2 = 2;
 
-// K splits of a CN product: about g_waves_x2 / 2 waves of CTAs
-// waves_x2 = 2: the stream-K schedule over one wave (one CTA per SM)
-SkPlan cn_stream_k(int mt, int nt, int total) {
+// A^H B: the fewest N tiles of equal width; runs of no fewer than four stages
+// (a run that short is mostly pipeline fill, and every CTA leaves a partial
+// tile to add)
+SkPlan cn_plan(int M, int N, int K, int waves_x2) {
     SkPlan p;
-    if (g_waves_x2 != 2) return p;
-    p.ctas = sm_count();
+    const int mt = (M + GB_M - 1) / GB_M, nt = (N + GB_NT - 1) / GB_NT, T = stages(K);
+    p.tn = tile_cols(N, nt);
     p.fast = mt;
-    p.units = (int64_t)mt * nt * total;
-    const int64_t len = (p.units + p.ctas - 1) / p.ctas;
-    p.maxseg = (int)((len + total - 1) / total) + 1;
+    p.units = (int64_t)mt * nt * T;
+    p.ctas = (int)std::min<int64_t>(sm_count() * waves_x2 / 2, std::max<int64_t>(1, p.units / 4));
+    p.len = (p.units + p.ctas - 1) / p.ctas;
+    p.ctas = (int)((p.units + p.len - 1) / p.len);
+    p.maxseg = (int)((p.len + T - 1) / T) + 1;
     return p;
 }
 
-int cn_splits(int tiles, int total) {
-    int ks = (g_waves_x2 * sm_count() / 2 + tiles - 1) / tiles;
-    if (ks > total) ks = total;
-    if (ks < 1) ks = 1;
-    const int per = (total + ks - 1) / ks;
-    return (total + per - 1) / per;
+// A B: the number of N tiles with the least time of the busiest CTA (its
+// tiles times the tile width, the A operand's share counting as 32 columns)
+SkPlan nn_plan(int M, int N) {
+    SkPlan best;
+    double best_cost = 1e300;
+    const int mt = (M + GB_M - 1) / GB_M, n0 = (N + GB_NT - 1) / GB_NT;
+    for (int nt = n0; nt < n0 + 4 && 16 * (nt - 1) < N; ++nt) {
+        SkPlan p;
+        p.tn = tile_cols(N, nt);
+        p.fast = nt;
+        p.units = (int64_t)mt * nt;
+        p.ctas = (int)std::min<int64_t>(sm_count(), p.units);
+        const double cost = (double)((p.units + p.ctas - 1) / p.ctas) * (p.tn + 32);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = p;
+        }
+    }
+    return best;
+}
+
+size_t cn_part_bytes(const SkPlan& p) {
+    return ((size_t)p.ctas * p.maxseg * p.tn * GB_M * sizeof(float2) + 255) / 256 * 256;
+}
+
+// tensor maps over an image: rows of 16 G 64-bit words, one per (chunk, part, plane) ...
+bool image_map(CUtensorMap* map, const TcImage& im, int box_words, int box_rows) {
+    const uint64_t Q = (im.rows + 7) / 8, G = (im.cols + 7) / 8;
+    const uint64_t dims[2] = {16 * G, 4 * Q}, strides[1] = {128 * G};
+    const uint32_t box[2] = {(uint32_t)box_words, (uint32_t)box_rows};
+    return tensor_map_words(map, im.data, 2, dims, strides, box);
+}
+// ... or core matrices by (chunk, group, part and plane), for boxes of 16 chunks x 4 groups
+bool image_map_mn(CUtensorMap* map, const TcImage& im) {
+    const uint64_t Q = (im.rows + 7) / 8, G = (im.cols + 7) / 8;
+    const uint64_t dims[4] = {16, Q, G, 4}, strides[3] = {512 * G, 128, 128 * G};
+    const uint32_t box[4] = {16, 16, 4, 4};
+    return tensor_map_words(map, im.data, 4, dims, strides, box);
 }
 
 }  // namespace
@@ -676,56 +643,50 @@ bool tcg_enabled() {
     return on == 1;
 }
 
-void tcg_set_waves(int waves_x2) { g_waves_x2 = waves_x2 >= 1 ? waves_x2 : 2; }
+// ROKS_TC_PRESPLIT=0 makes every operand's image at each call (for comparisons)
+bool tcg_keep_images() {
+    static int on = -1;
+    if (on < 0) {
+        const char* e = std::getenv("ROKS_TC_PRESPLIT");
+        on = (e && e[0] == '0') ? 0 : 1;
+    }
+    return on == 1;
+}
 
 bool tcg_cn_takes(int M, int N, int K) { return tcg_enabled() && M >= 128 && N >= 64 && K >= 1024; }
 bool tcg_nn_takes(int M, int N, int K) { return tcg_enabled() && M >= 4096 && N >= 64 && K >= 64; }
 
+size_t tcg_image_bytes(int rows, int cols) {
+    const size_t Q = (rows + 7) / 8, G = (cols + 7) / 8;
+    return 512 * Q * G + (32 * G + 255) / 256 * 256;
+}
+
+TcImage tcg_image_at(void* buf, int rows, int cols) {
+    TcImage im;
+    const size_t Q = (rows + 7) / 8, G = (cols + 7) / 8;
+    im.data = buf;
+    im.ex = reinterpret_cast<int*>(static_cast<unsigned char*>(buf) + 512 * Q * G);
+    im.rows = rows;
+    im.cols = cols;
+    return im;
+}
+
+bool tcg_split(const TcImage& im, const float2* X, int64_t ld, cudaStream_t st) {
+    const bool vec = !(ld & 1) && aligned(X, 16);
+    return vec ? launch_split<float2, true>(im.rows, im.cols, X, ld, nullptr, im, st)
+               : launch_split<float2, false>(im.rows, im.cols, X, ld, nullptr, im, st);
+}
+
+void tcg_set_waves(int waves_x2) { g_waves_x2 = waves_x2 >= 1 ? waves_x2 : 2; }
+
 size_t tcg_cn_work_bytes(int M, int N, int K) {
-    // the larger of the split-K and the stream-K partials (the autotuner
-    // may take either after the buffer is sized)
-    const int mt = (M + GB_M - 1) / GB_M, nt = (N + GB_NC - 1) / GB_NC, total = (K + GB_KC - 1) / GB_KC;
-    size_t split = 0;
-    for (int w : {3, 5, 8}) {
-        const int keep = g_waves_x2;
-        g_waves_x2 = w;
-        split = std::max(split, (size_t)mt * nt * cn_splits(mt * nt, total));
-        g_waves_x2 = keep;
-    }
-    const int ctas = sm_count();
-    const int64_t len = ((int64_t)mt * nt * total + ctas - 1) / ctas;
-    const size_t sk = (size_t)ctas * (size_t)((len + total - 1) / total + 1);
-    return std::max(split, sk) * GB_NC * GB_M * sizeof(float2);
+    // the autotuner may take any of its schedules after the buffer is sized
+    size_t part = 0;
+    for (int w : {2, 5, 8}) part = std::max(part, cn_part_bytes(cn_plan(M, N, K, w)));
+    return part + tcg_image_bytes(K, M) + tcg_image_bytes(K, N);
 }
 
-size_t tcg_nn_work_bytes(int N, int K) {
-    const int nt = (N + GB_NC - 1) / GB_NC, total = (K + GB_KC - 1) / GB_KC;
-    return (size_t)nt * total * 2 * GB_PART;
-}
-
-size_t tcg_presplit_bytes(int M, int K) {
-    const size_t mt = (M + GB_M - 1) / GB_M, nst = (K + GB_KC - 1) / GB_KC;
-    return mt * nst * 2 * GB_PART;
-}
-
-bool tcg_presplit(int M, int K, const float2* A, int64_t lda, void* out, cudaStream_t st) {
-    if (g_npre >= kMaxPreSplit || !aligned(out, 16)) return false;
-    const int mt = (M + GB_M - 1) / GB_M, nst = (K + GB_KC - 1) / GB_KC;
-    const int64_t n = (int64_t)mt * nst * GB_M * 8;
-    unsigned char* o = static_cast<unsigned char*>(out);
-    roks::count_launch();
-    k_tcg_asplit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(M, K, A, lda, nst, mt, o);
-    if (cudaGetLastError() != cudaSuccess) return false;
-    g_pre[g_npre++] = PreSplit{A, lda, M, K, o};
-    return true;
-}
-
-void tcg_presplit_forget(const void* split) {
-    int w = 0;
-    for (int i = 0; i < g_npre; ++i)
-        if (g_pre[i].split != split) g_pre[w++] = g_pre[i];
-    g_npre = w;
-}
+size_t tcg_nn_work_bytes(int M, int N, int K) { return tcg_image_bytes(K, N) + tcg_image_bytes(M, K); }
 
 static long long g_tcg_launches = 0;
 long long tcg_launches_take() {
@@ -736,99 +697,79 @@ long long tcg_launches_take() {
 
 // C = A^H B on the tensor cores; false when the shape, the alignment or the
 // work buffer does not allow it (the caller then takes the SIMT kernels).
+// ia, ib: images of A and B that the caller has made (else they are made in
+// the work buffer; one serves both when A and B are the same block).
 bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2* B, int64_t ldb, double2* C, int ldc,
-                 void* work, size_t work_bytes, cudaStream_t st) {
-    if (!tcg_cn_takes(M, N, K)) return false;
-    if ((lda & 1) || (ldb & 1) || !aligned(A, 16) || !aligned(B, 16) || !aligned(work, 16)) return false;
-    const int mt = (M + GB_M - 1) / GB_M, nt = (N + GB_NC - 1) / GB_NC, total = (K + GB_KC - 1) / GB_KC;
-    const SkPlan sk = cn_stream_k(mt, nt, total);
-    const int ks = sk.ctas > 0 ? 1 : cn_splits(mt * nt, total);
-    const int per = (total + ks - 1) / ks;
-    if (tcg_cn_work_bytes(M, N, K) > work_bytes) return false;
-    // (A^H B converts both operands in the kernel: a pre-split A, copied as
-    // 32 KB hi/lo blocks while the workers still convert B, measured slower
-    // on P^H Psi at mgo-120, 1.45 -> 1.49 ms)
+                 void* work, size_t work_bytes, const TcImage* ia, const TcImage* ib, cudaStream_t st) {
+    if (!tcg_cn_takes(M, N, K) || !work || !aligned(work, 256)) return false;
+    const SkPlan sk = cn_plan(M, N, K, g_waves_x2);
+    const bool same = A == B && lda == ldb && M == N;
+    unsigned char* w = static_cast<unsigned char*>(work);
+    size_t need = cn_part_bytes(sk);
+    TcImage ma, mb;
+    if (ia) ma = *ia;
+    else if (same && ib) ma = *ib;
+    else {
+        ma = tcg_image_at(w + need, K, M);
+        need += tcg_image_bytes(K, M);
+    }
+    if (ib) mb = *ib;
+    else if (same) mb = ma;
+    else {
+        mb = tcg_image_at(w + need, K, N);
+        need += tcg_image_bytes(K, N);
+    }
+    if (need > work_bytes) return false;
     CUtensorMap tmA, tmB;
-    if (!tensor_map_2d(&tmA, A, K, M, lda, GB_KC, GB_M, true) || !tensor_map_2d(&tmB, B, K, N, ldb, GB_KC, GB_NC, true))
-        return false;
-    float2* part = static_cast<float2*>(work);
+    if (!image_map(&tmA, ma, 256, 16) || !image_map(&tmB, mb, 2 * sk.tn, 16)) return false;
+    if (!ia && !(same && ib) && !tcg_split(ma, A, lda, st)) return false;
+    if (!ib && !same && !tcg_split(mb, B, ldb, st)) return false;
     roks::count_launch();
     g_tcg_launches += 1;
-    if (sk.ctas > 0) {
-        set_attr<false, false, true>();
-        k_tcgemm<false, false, true><<<dim3(sk.ctas, 1, 1), GB_THREADS, GbPlan<false, false>::SMEM, st>>>(
-            M, N, per, total, sk, tmA, tmB, nullptr, nullptr, part, nullptr, 0, nullptr, 0, 0.f, 0.f, wait_polls());
-    } else {
-        set_attr<false, false>();
-        k_tcgemm<false, false><<<dim3(mt, nt, ks), GB_THREADS, GbPlan<false, false>::SMEM, st>>>(
-            M, N, per, total, sk, tmA, tmB, nullptr, nullptr, part, nullptr, 0, nullptr, 0, 0.f, 0.f, wait_polls());
-    }
-    const int64_t outs = (int64_t)M * N;
+    set_attr<false>();
+    const int T = stages(K);
+    float2* part = reinterpret_cast<float2*>(w);
+    k_tcgemm<false><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, T, sk, tmA, tmB, nullptr, part, nullptr, 0, nullptr, 0,
+                                                          0.f, 0.f, wait_polls());
     roks::count_launch();
-    if (sk.ctas > 0)
-        k_tcg_reduce_sk<<<(unsigned)((outs + 255) / 256), 256, 0, st>>>(M, N, mt, total, sk, part, C, ldc);
+    const int mt = (M + GB_M - 1) / GB_M;
+    // many CTAs per tile: their segments shared out over the warps of a block
+    if ((int64_t)T > 8 * sk.len)
+        k_tcg_reduce_sk<8><<<dim3((M + 31) / 32, N), 256, 0, st>>>(M, N, mt, T, sk, ma.ex, mb.ex, part, C, ldc);
     else
-        k_tcg_reduce<<<(unsigned)((outs + 255) / 256), 256, 0, st>>>(M, N, mt, mt * nt, ks, part, C, ldc);
+        k_tcg_reduce_sk<1><<<dim3((M + 31) / 32, (N + 7) / 8), 256, 0, st>>>(M, N, mt, T, sk, ma.ex, mb.ex, part, C,
+                                                                           ldc);
     return true;
 }
 
 // Cout = alpha A B + beta Cin on the tensor cores (B FP64, small); false when
-// not applicable.  Cout may be Cin; it must not overlap A.
+// not applicable.  Cout may be Cin; it must not overlap A unless ia, an image
+// of A that the caller has made, is given.
 bool gemm_nn_tcg(int M, int N, int K, const float2* A, int64_t lda, const double2* B, int ldb, const float2* Cin,
-                 int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, void* bwork, size_t bwork_bytes,
-                 cudaStream_t st) {
-    if (!tcg_nn_takes(M, N, K) || !bwork) return false;
-    if ((lda & 1) || !aligned(A, 16) || !aligned(bwork, 16) || !aligned(Cout, 8)) return false;
+                 int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, void* work, size_t work_bytes,
+                 const TcImage* ia, cudaStream_t st) {
+    if (!tcg_nn_takes(M, N, K) || !work || !aligned(work, 256) || !aligned(Cout, 8)) return false;
     if (beta != 0.f && (!Cin || !aligned(Cin, 8))) return false;
-    if (static_cast<const void*>(A) == static_cast<const void*>(Cout)) return false;
-    const int nt = (N + GB_NC - 1) / GB_NC, total = (K + GB_KC - 1) / GB_KC;
-    if (tcg_nn_work_bytes(N, K) > bwork_bytes) return false;
-    const unsigned char* as = find_presplit(A, lda, M, K);
-    CUtensorMap tmA{};
-    if (!as && !tensor_map_2d(&tmA, A, M, K, lda, GB_M, GB_KC, false)) return false;
-    unsigned char* bs = static_cast<unsigned char*>(bwork);
-    const int64_t nsplit = (int64_t)nt * total * GB_NR * 8;
-    roks::count_launch();
-    k_tcg_bsplit<<<(unsigned)((nsplit + 255) / 256), 256, 0, st>>>(K, N, B, ldb, total, nt, bs);
+    unsigned char* w = static_cast<unsigned char*>(work);
+    size_t need = tcg_image_bytes(K, N);
+    const TcImage mb = tcg_image_at(w, K, N);
+    TcImage ma;
+    if (ia) ma = *ia;
+    else {
+        ma = tcg_image_at(w + need, M, K);
+        need += tcg_image_bytes(M, K);
+    }
+    if (need > work_bytes) return false;
+    const SkPlan sk = nn_plan(M, N);
+    CUtensorMap tmA, tmB;
+    if (!image_map_mn(&tmA, ma) || !image_map(&tmB, mb, 2 * sk.tn, 16)) return false;
+    if (!ia && !tcg_split(ma, A, lda, st)) return false;
+    if (!launch_split<double2, false>(K, N, B, ldb, ma.ex, mb, st)) return false;
     roks::count_launch();
     g_tcg_launches += 1;
-    const int mt = (M + GB_M - 1) / GB_M;
-    const dim3 grid(nt, mt, 1);
-    // more tiles than SMs: persistent CTAs, one per SM, each looping over
-    // whole tiles (tile t: N tile t % nt, M tile t / nt) with its pipeline
-    // running on across them
-    SkPlan pp;
-    if ((int64_t)mt * nt > sm_count()) {
-        pp.ctas = sm_count();
-        pp.units = (int64_t)mt * nt;
-        pp.fast = nt;
-    }
-    if (pp.ctas > 0) {
-        const dim3 g1(pp.ctas, 1, 1);
-        if (as) {
-            set_attr<true, true, true>();
-            k_tcgemm<true, true, true><<<g1, GB_THREADS, GbPlan<true, true>::SMEM, st>>>(
-                M, N, total, total, pp, tmA, tmA, bs, as, nullptr, Cin, ldcin, Cout, ldc, alpha, beta,
-                wait_polls());
-        } else {
-            set_attr<true, false, true>();
-            k_tcgemm<true, false, true><<<g1, GB_THREADS, GbPlan<true, false>::SMEM, st>>>(
-                M, N, total, total, pp, tmA, tmA, bs, nullptr, nullptr, Cin, ldcin, Cout, ldc, alpha, beta,
-                wait_polls());
-        }
-        return true;
-    }
-    if (as) {
-        set_attr<true, true>();
-        k_tcgemm<true, true><<<grid, GB_THREADS, GbPlan<true, true>::SMEM, st>>>(
-            M, N, total, total, SkPlan{}, tmA, tmA, bs, as, nullptr, Cin, ldcin, Cout, ldc, alpha, beta,
-            wait_polls());
-    } else {
-        set_attr<true, false>();
-        k_tcgemm<true, false><<<grid, GB_THREADS, GbPlan<true, false>::SMEM, st>>>(
-            M, N, total, total, SkPlan{}, tmA, tmA, bs, nullptr, nullptr, Cin, ldcin, Cout, ldc, alpha, beta,
-            wait_polls());
-    }
+    set_attr<true>();
+    k_tcgemm<true><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, stages(K), sk, tmA, tmB, mb.ex, nullptr, Cin, ldcin,
+                                                         Cout, ldc, alpha, beta, wait_polls());
     return true;
 }
 

@@ -35,7 +35,7 @@ struct roks_ctx {
     double L = 0, omega = 0, ecut = 0, alpha = 0, e_tol = 1e-6, g_tol = 0;
     int max_iter = 0, wait_cap = 0, exx_kernel = 0, autotune = 0;
     // launch shapes (the autotuner's choices, or the defaults)
-    int dens_groups = kDensityGroups, tc_waves_x2 = 2;   // 2: stream-K A^H B
+    int dens_groups = kDensityGroups, tc_waves_x2 = 2;   // 2: one A^H B run per SM
     double tune_ms[6] = {0, 0, 0, 0, 0, 0};
     uint64_t seed = 0;
     long long steps = 0;   // PCG and DIIS steps since the orbitals were last set
@@ -55,9 +55,13 @@ struct roks_ctx {
     int gamma = 0, npw_full = 0, h0 = 0, nbt = 0, nct = 0, split_t = -1;
     int64_t ldc_pk = 0;
     void* d_Cpk = nullptr;   // packed full-sphere coefficients (npw_full rows, ldc_pk, nbt bands)
-    // the projector matrix split once into TF32 hi/lo operand blocks for the
-    // tensor-core tall products P Y, where they take it
-    void* d_Psplit_nn = nullptr;
+    // the projector matrix in the tensor cores' operand layout, where the
+    // contractions with it run there (data null: they don't)
+    TcImage P_img;
+    // the same for blocks that several contractions of a call take: the
+    // orbitals, S Psi, and the block being orthonormalised (null: not kept)
+    enum { IMG_PSI, IMG_S, IMG_ORTH, IMG_COUNT };
+    TcImage img[IMG_COUNT];
     double cM = 0, cT = 0;
     PotCoef cf{};
     std::vector<int32_t> miller;
@@ -275,11 +279,24 @@ struct Impl {
     static V* cv(void* p) { return static_cast<V*>(p); }
     static const V* ccv(const void* p) { return static_cast<const V*>(p); }
 
+    static const TcImage* P_image(const roks_ctx* ctx) { return ctx->P_img.data ? &ctx->P_img : nullptr; }
+
+    // The block X (npw x nb) split once for the contractions of this call that
+    // take it; null where no image is kept (they then make their own)
+    static const TcImage* image(roks_ctx* ctx, int slot, const void* X, int64_t ld) {
+        if constexpr (sizeof(T) == 4) {
+            const TcImage& im = ctx->img[slot];
+            if (im.data && tcg_split(im, static_cast<const float2*>(X), ld, ctx->st)) return &im;
+        }
+        return nullptr;
+    }
+
     // C = A^H B over the basis rows; at the Gamma point its real part (the
     // full-sphere product of real orbitals in the stored half-sphere form)
     static void cn(roks_ctx* ctx, int M, int N, int K, const V* A, int64_t lda, const V* B, int64_t ldb, double2* C,
-                   int ldc, cudaStream_t st) {
-        gemm_cn<T>(M, N, K, A, lda, B, ldb, C, ldc, ctx->d_gemm_work, ctx->gemm_work_elems, st);
+                   int ldc, cudaStream_t st, const TcImage* ia = nullptr, const TcImage* ib = nullptr) {
+        gemm_cn<T>(M, N, K, A, lda, B, ldb, C, ldc, ctx->d_gemm_work, ctx->gemm_work_elems, st,
+                   A == ccv(ctx->d_P) ? P_image(ctx) : ia, ib);
         if (ctx->gamma) gamma_real_part(M, N, C, ldc, st);
     }
 
@@ -414,8 +431,10 @@ struct Impl {
 
     // planes_ready: Yp already holds the planes of psi (yp_psi), so the
     // transform starts at the x stage
+    // ipsi: an image of psi, if the caller has one
     static roks_status apply(roks_ctx* ctx, const void* psi, int64_t ld, void* F, int64_t ldf, void* S,
-                             int64_t lds, bool reuse_B = false, bool planes_ready = false) {
+                             int64_t lds, bool reuse_B = false, bool planes_ready = false,
+                             const TcImage* ipsi = nullptr) {
         const Sphere s = sphere(ctx);
         cudaStream_t st = ctx->st;
         const V* p = ccv(psi);
@@ -463,7 +482,8 @@ struct Impl {
         if (ctx->nproj > 0) {
             if (!reuse_B) {
                 PROF("proj_PhPsi");
-                cn(ctx, ctx->nproj, ctx->nb, ctx->npw, ccv(ctx->d_P), ctx->ld_min, p, ld, ctx->d_B, ctx->nproj, st);
+                cn(ctx, ctx->nproj, ctx->nb, ctx->npw, ccv(ctx->d_P), ctx->ld_min, p, ld, ctx->d_B, ctx->nproj, st,
+                   nullptr, ipsi);
                 ctx->b_psi = psi;
                 ctx->b_ld = ld;
             }
@@ -471,7 +491,7 @@ struct Impl {
                      ctx->d_wband, ctx->d_DB, ctx->d_QB, st);
             PROF("proj_PX");
             gemm_nn<T>(ctx->npw, ctx->nb, ctx->nproj, ccv(ctx->d_P), ctx->ld_min, ctx->d_DB, ctx->nproj, cv(F), ldf,
-                       1.0, 1.0, ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                       1.0, 1.0, ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), P_image(ctx));
         }
         if (S) {
             CK(cudaMemcpy2DAsync(S, lds * sizeof(V), psi, ld * sizeof(V), ctx->npw * sizeof(V), ctx->nb,
@@ -479,7 +499,8 @@ struct Impl {
             if (ctx->nproj > 0) {
                 PROF("proj_PX");
                 gemm_nn<T>(ctx->npw, ctx->nb, ctx->nproj, ccv(ctx->d_P), ctx->ld_min, ctx->d_QB, ctx->nproj, cv(S),
-                           lds, 1.0, 1.0, ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                           lds, 1.0, 1.0, ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2),
+                           P_image(ctx));
             }
         }
         CK(cudaGetLastError());
@@ -490,14 +511,17 @@ struct Impl {
     static roks_status orth(roks_ctx* ctx, const void* in, int64_t ldi, void* out, int64_t ldo, double2* Bout) {
         cudaStream_t st = ctx->st;
         const int nb = ctx->nb;
+        const TcImage* ii = nullptr;
         {
             PROF("orth_overlap");
-            cn(ctx, nb, nb, ctx->npw, ccv(in), ldi, ccv(in), ldi, ctx->d_O, nb, st);
+            ii = image(ctx, roks_ctx::IMG_ORTH, in, ldi);
+            cn(ctx, nb, nb, ctx->npw, ccv(in), ldi, ccv(in), ldi, ctx->d_O, nb, st, ii, ii);
         }
         if (ctx->nproj > 0) {
             {
                 PROF("proj_PhPsi");
-                cn(ctx, ctx->nproj, nb, ctx->npw, ccv(ctx->d_P), ctx->ld_min, ccv(in), ldi, ctx->d_B2, ctx->nproj, st);
+                cn(ctx, ctx->nproj, nb, ctx->npw, ccv(ctx->d_P), ctx->ld_min, ccv(in), ldi, ctx->d_B2, ctx->nproj, st,
+                   nullptr, ii);
             }
             PROF("orth_small");
             apply_DQ(ctx->nproj, nb, ctx->d_B2, ctx->d_blk_off, ctx->d_blk_n, ctx->d_Drow, ctx->d_Qrow, nullptr,
@@ -529,10 +553,10 @@ struct Impl {
             PROF("orth_apply");
             if (dev)
                 gemm_nn_io<T>(ctx->npw, nb, nb, ccv(in), ldi, ctx->d_LinvH, nb, ccv(in), ldi, cv(out), ldo, 1.0, 1.0,
-                              ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                              ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), ii);
             else
                 gemm_nn<T>(ctx->npw, nb, nb, ccv(in), ldi, ctx->d_LinvH, nb, cv(out), ldo, 1.0, 0.0,
-                           ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                           ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), ii);
         }
         if (Bout && ctx->nproj > 0) {
             PROF("orth_small");
@@ -570,14 +594,15 @@ struct Impl {
     }
 
     // s-projection: out = x - Psi ((S Psi)^H x)
-    static void project(roks_ctx* ctx, const void* psi, int64_t ld, const void* x, void* out) {
+    static void project(roks_ctx* ctx, const void* psi, int64_t ld, const void* x, void* out, const TcImage* ipsi,
+                        const TcImage* is) {
         cudaStream_t st = ctx->st;
         const int nb = ctx->nb;
         const int64_t l = ctx->ld_min;
         PROF("subspace_project");
-        cn(ctx, nb, nb, ctx->npw, ccv(ctx->W_S), l, ccv(x), l, ctx->d_Msm, nb, st);
+        cn(ctx, nb, nb, ctx->npw, ccv(ctx->W_S), l, ccv(x), l, ctx->d_Msm, nb, st, is);
         gemm_nn_io<T>(ctx->npw, nb, nb, ccv(psi), ld, ctx->d_Msm, nb, ccv(x), l, cv(out), l, -1.0, 1.0,
-                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), ipsi);
     }
 
     // dst field = sum_n Re <x_n|y_n>
@@ -663,9 +688,11 @@ struct Impl {
         // F Psi, S Psi, theta, d
         r = apply(ctx, psi, ld, ctx->W_F, l, ctx->W_S, l, true, true);
         if (r != ROKS_OK) return r;
+        const TcImage *ipsi = nullptr, *is = nullptr;
         {
             PROF("subspace_theta");
-            cn(ctx, nb, nb, npw, ccv(psi), ld, ccv(ctx->W_F), l, ctx->d_Th, nb, st);
+            ipsi = image(ctx, roks_ctx::IMG_PSI, psi, ld);
+            cn(ctx, nb, nb, npw, ccv(psi), ld, ccv(ctx->W_F), l, ctx->d_Th, nb, st, ipsi);
         }
         const int ia = (ctx->mode == ROKS_MODE_SINGLET) ? ctx->nc : -1;
         const int ib = (ctx->mode == ROKS_MODE_SINGLET) ? ctx->nc + 1 : -1;
@@ -682,12 +709,13 @@ struct Impl {
         // (their g_I is the F^c residual, the empty bands' own direction)
         {
         PROF("gradient_precond");
+        is = image(ctx, roks_ctx::IMG_S, ctx->W_S, l);
         gemm_nn_io<T>(npw, nb, nb, ccv(ctx->W_S), l, ctx->d_Th, nb, ccv(ctx->W_F), l, cv(ctx->W_gI), l, -1.0, 1.0,
-                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), is);
         if (ctx->ne > 0) CK(cudaMemsetAsync(static_cast<V*>(ctx->W_F) + (int64_t)ctx->nocc * l, 0,
                                             sizeof(V) * l * ctx->ne, st));
         gemm_nn_io<T>(npw, nb, nb, ccv(ctx->W_S), l, ctx->d_Gam, nb, ccv(ctx->W_F), l, cv(ctx->W_G), l, -1.0, 1.0,
-                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2));
+                      ctx->d_gemm_work, st, ctx->gemm_work_elems * sizeof(double2), is);
         column_total<T>(3, npw, nb, ccv(ctx->W_G), l, nullptr, 0, static_cast<const T*>(ctx->d_g2half), ctx->d_colpart,
                         reinterpret_cast<double*>(ctx->d_sc) + SC_FIELD(gnorm2), 1.0, st);
         // p_I = K g_I - Psi (S Psi)^H K g_I
@@ -698,14 +726,14 @@ struct Impl {
         else
             precondition<T>(npw, nb, ccv(ctx->W_gI), l, static_cast<const T*>(ctx->d_g2half), ctx->d_colout, cv(ctx->W_K), l, st);
         }
-        project(ctx, psi, ld, ctx->W_K, ctx->W_K);
+        project(ctx, psi, ld, ctx->W_K, ctx->W_K, ipsi, is);
         // the Fletcher-Reeves ratio of the energy's gradient: occupied bands
         dot_to(ctx, ctx->W_K, ctx->W_gI, SC_FIELD(pgI), ctx->nocc);
         pcg_rot_dots(nb, ctx->d_A, ctx->d_Aprev, ctx->d_Gin, ctx->d_colpart, ctx->d_sc, st);
         // u = p_I (projected above; the S-projector is idempotent on
         // S-orthonormal orbitals, so projecting again changes nothing),
         // v = proj(s_prev) (s_prev was projected against the previous orbitals)
-        project(ctx, psi, ld, ctx->W_sprev, ctx->W_v);
+        project(ctx, psi, ld, ctx->W_sprev, ctx->W_v, ipsi, is);
         dot_to(ctx, ctx->W_K, ctx->W_G, SC_FIELD(a1));
         dot_to(ctx, ctx->W_v, ctx->W_G, SC_FIELD(a2));
         pcg_direction(ctx->d_sc, st);
@@ -886,13 +914,15 @@ struct Impl {
         const double b = 2.0 * M_PI / ctx->L;
         {
             PROF("force");
-            cn(ctx, nb, nb, npw, ccv(psi), ld, ccv(ctx->W_F), l, ctx->d_Th, nb, st);
+            // (the occupied bands are the image's first columns)
+            const TcImage* ipsi = image(ctx, roks_ctx::IMG_PSI, psi, ld);
+            cn(ctx, nb, nb, npw, ccv(psi), ld, ccv(ctx->W_F), l, ctx->d_Th, nb, st, ipsi);
             diis_multipliers(nb, ctx->d_Th, -1, -1, 0.5, 0.5, ctx->d_Gam, st);   // Gam = (theta + theta^H)/2
             if (np_ > 0) {
                 for (int nu = 0; nu < 3; ++nu) {
                     force_dP<T>(npw, np_, ccv(ctx->d_P), l, ctx->d_miller, b, nu, cv(ctx->d_fdP), st);
                     cn(ctx, np_, nb, npw, ccv(ctx->d_fdP), l, ccv(psi), ld, ctx->d_fdB + (int64_t)nu * np_ * nb, np_,
-                       st);
+                       st, nullptr, ipsi);
                 }
                 apply_DQ(np_, nb, ctx->d_B, ctx->d_blk_off, ctx->d_blk_n, ctx->d_Drow, ctx->d_Qrow, ctx->d_wband,
                          ctx->d_DB, ctx->d_QB, st);
@@ -1056,8 +1086,8 @@ void reset_history(roks_ctx* ctx) {
     cudaStreamSynchronize(ctx->st);
 }
 
-// The context's wait cap and tensor-core split depth for the launches of
-// one entry point.
+// The context's wait cap and tensor-core schedule for the launches of one
+// entry point.
 void enter(roks_ctx* ctx) {
     set_wait_cap(ctx->wait_cap);
     tcg_set_waves(ctx->tc_waves_x2);
@@ -1093,7 +1123,7 @@ int pick_fastest(roks_ctx* ctx, const int* cand, int nc, double* ms, F fn) {
 
 // Autotuner (roks_options.autotune): the band grouping of the density's x
 // stage (grid depth against the fixed-order reduction of the group slots)
-// and, on the mixed path, the split depth of the tensor-core A^H B products,
+// and, on the mixed path, the schedule of the tensor-core A^H B products,
 // each timed on the context's own buffers and sizes.
 roks_status autotune(roks_ctx* ctx) {
     enter(ctx);
@@ -1113,13 +1143,12 @@ roks_status autotune(roks_ctx* ctx) {
     const int M = ctx->nproj >= ctx->nb ? ctx->nproj : ctx->nb;
     const void* A = ctx->nproj >= ctx->nb ? ctx->d_P : ctx->W_Y;
     if (ctx->prec == ROKS_MIXED && tcg_cn_takes(M, ctx->nb, ctx->npw)) {
-        // 2: stream-K over one wave; 5, 8: K split into 2.5 or 4 waves
         const int w_cand[3] = {2, 5, 8};
         ctx->tc_waves_x2 = pick_fastest(ctx, w_cand, 3, ctx->tune_ms + 3, [&](int w) {
             tcg_set_waves(w);
             gemm_cn<float>(M, ctx->nb, ctx->npw, static_cast<const float2*>(A), ctx->ld_min,
                            static_cast<const float2*>(ctx->W_Y), ctx->ld_min, ctx->d_B2, M, ctx->d_gemm_work,
-                           ctx->gemm_work_elems, ctx->st);
+                           ctx->gemm_work_elems, ctx->st, A == ctx->d_P ? Impl<float>::P_image(ctx) : nullptr);
         });
         tcg_set_waves(ctx->tc_waves_x2);
     }
@@ -1374,16 +1403,15 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
     AL(ctx->d_B2, sizeof(double2) * np_ * nb);
     size_t gw = gemm_cn_work(np_ > nb ? np_ : nb, nb, npw);
     if (!f64) {
-        // partial sums of the tensor-core contractions and the split B blocks
-        // of their tall products share the buffer
-        // (sized for the deepest split the autotuner may choose)
-        tcg_set_waves(opt->autotune ? 8 : ctx->tc_waves_x2);
-        const size_t tb = std::max(std::max(tcg_cn_work_bytes(np_, nb, npw), tcg_cn_work_bytes(nb, nb, npw)),
-                                   std::max(tcg_nn_work_bytes(nb, np_), tcg_nn_work_bytes(nb, nb)));
+        // operand images and partial sums of the tensor-core contractions
+        size_t tb = 0;
+        for (int m : {np_, nb}) {
+            if (tcg_cn_takes(m, nb, npw)) tb = std::max(tb, tcg_cn_work_bytes(m, nb, npw));
+            if (tcg_nn_takes(npw, nb, m)) tb = std::max(tb, tcg_nn_work_bytes(npw, nb, m));
+        }
         gw = std::max(gw, (tb + sizeof(double2) - 1) / sizeof(double2));
     }
     ctx->gemm_work_elems = gw;
-    tcg_set_waves(ctx->tc_waves_x2);
     AL(ctx->d_gemm_work, sizeof(double2) * gw);
     AL(ctx->d_kin_b, sizeof(double) * nb);
     AL(ctx->d_nl_b, sizeof(double) * nb);
@@ -1428,8 +1456,18 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
         AL(ctx->d_hf2, sizeof(double) * 2);
         AL(ctx->d_exopen, sizeof(double) * 2);
     }
-    if (!f64 && ctx->nproj > 0 && tcg_nn_takes(npw, nb, ctx->nproj))
-        AL(ctx->d_Psplit_nn, tcg_presplit_bytes(npw, ctx->nproj));
+    if (!f64 && ctx->nproj > 0 && tcg_keep_images() &&
+        (tcg_nn_takes(npw, nb, ctx->nproj) || tcg_cn_takes(ctx->nproj, nb, npw))) {
+        void* pi = nullptr;
+        AL(pi, tcg_image_bytes(npw, ctx->nproj));
+        ctx->P_img = tcg_image_at(pi, npw, ctx->nproj);
+    }
+    if (!f64 && tcg_keep_images() && tcg_nn_takes(npw, nb, nb))
+        for (TcImage& im : ctx->img) {
+            void* b = nullptr;
+            AL(b, tcg_image_bytes(npw, nb));
+            im = tcg_image_at(b, npw, nb);
+        }
     double* d_atoms = nullptr;
     double* d_proj = nullptr;
     AL(d_atoms, sizeof(double) * (atomtab.size() + 1));
@@ -1514,9 +1552,8 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
         if (f64) gamma_scale_rows<double>(npw, ctx->nproj, static_cast<double2*>(ctx->d_P), l, ctx->st);
         else gamma_scale_rows<float>(npw, ctx->nproj, static_cast<float2*>(ctx->d_P), l, ctx->st);
     }
-    if (ctx->d_Psplit_nn &&
-        !tcg_presplit(npw, ctx->nproj, static_cast<const float2*>(ctx->d_P), l, ctx->d_Psplit_nn, ctx->st))
-        return bail(ROKS_ECUDA, "projector split");
+    if (ctx->P_img.data && !tcg_split(ctx->P_img, static_cast<const float2*>(ctx->d_P), l, ctx->st))
+        return bail(ROKS_ECUDA, "projector image");
     if (opt->alpha != 0.0) {
         const int bare = opt->exx_kernel == ROKS_EXX_BARE ? 1 : 0;
         if (f64) exx_setup_kernel<double>(N, cell->L, bare, static_cast<double*>(ctx->d_vG), ctx->st);
@@ -1666,8 +1703,10 @@ roks_status roks_gradient_parts(roks_ctx* ctx, const void* psi, int64_t ld, void
     const int nb = ctx->nb;
     void* S = spsi ? spsi : ((grad || grad_I) ? ctx->W_S : nullptr);
     const int64_t lds = spsi ? ld : l;
+    const TcImage* ipsi =
+        ctx->prec == ROKS_MIXED && (grad || grad_I) ? Impl<float>::image(ctx, roks_ctx::IMG_PSI, psi, ld) : nullptr;
     if (ctx->prec == ROKS_FP64) r = Impl<double>::apply(ctx, psi, ld, fpsi, ld, S, lds);
-    else r = Impl<float>::apply(ctx, psi, ld, fpsi, ld, S, lds);
+    else r = Impl<float>::apply(ctx, psi, ld, fpsi, ld, S, lds, false, false, ipsi);
     if (r != ROKS_OK || !(grad || grad_I)) return r;
     // theta = Psi^H F Psi; g = F - S Gam, Gam_mn = (theta_mn + conj theta_nm) / 2; g_I = F - S theta
     if (ctx->prec == ROKS_FP64) {
@@ -1675,8 +1714,10 @@ roks_status roks_gradient_parts(roks_ctx* ctx, const void* psi, int64_t ld, void
                         ctx->d_Th, nb, ctx->d_gemm_work, ctx->gemm_work_elems, ctx->st);
     } else {
         gemm_cn<float>(nb, nb, ctx->npw, static_cast<const float2*>(psi), ld, static_cast<const float2*>(fpsi), ld,
-                       ctx->d_Th, nb, ctx->d_gemm_work, ctx->gemm_work_elems, ctx->st);
+                       ctx->d_Th, nb, ctx->d_gemm_work, ctx->gemm_work_elems, ctx->st, ipsi);
     }
+    const TcImage* is =
+        ctx->prec == ROKS_MIXED && grad && grad_I ? Impl<float>::image(ctx, roks_ctx::IMG_S, S, lds) : nullptr;
     if (ctx->gamma) gamma_real_part(nb, nb, ctx->d_Th, nb, ctx->st);
     const size_t es = ctx->prec == ROKS_FP64 ? sizeof(double2) : sizeof(float2);
     for (int part = 0; part < 2; ++part) {
@@ -1700,7 +1741,7 @@ roks_status roks_gradient_parts(roks_ctx* ctx, const void* psi, int64_t ld, void
                             ld, -1.0, 1.0, ctx->d_gemm_work, ctx->st, ctx->gemm_work_elems * sizeof(double2));
         else
             gemm_nn<float>(ctx->npw, nb, nb, static_cast<const float2*>(S), lds, M, nb, static_cast<float2*>(out), ld,
-                           -1.0, 1.0, ctx->d_gemm_work, ctx->st, ctx->gemm_work_elems * sizeof(double2));
+                           -1.0, 1.0, ctx->d_gemm_work, ctx->st, ctx->gemm_work_elems * sizeof(double2), is);
     }
     CK(cudaGetLastError());
     return ROKS_OK;
@@ -2020,7 +2061,6 @@ void roks_destroy(roks_ctx* ctx) {
     if (ctx->st) cudaStreamSynchronize(ctx->st);
     else cudaDeviceSynchronize();
     if (ctx->pcg_exec) cudaGraphExecDestroy(ctx->pcg_exec);
-    if (ctx->d_Psplit_nn) tcg_presplit_forget(ctx->d_Psplit_nn);
     if (ctx->h_sc) cudaFreeHost(ctx->h_sc);
     if (ctx->h_diis) cudaFreeHost(ctx->h_diis);
     if (ctx->cap_st) cudaStreamDestroy(ctx->cap_st);

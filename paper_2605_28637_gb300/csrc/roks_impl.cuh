@@ -156,6 +156,14 @@ void grid_fft3(int N, const c2<T>* tw, c2<T>* data, int dir, cudaStream_t st);
 template <typename T>
 void grid_fft3_batched(int N, const c2<T>* tw, c2<T>* data, int batch, int64_t bstride, int dir, cudaStream_t st);
 
+// A block split into the tensor cores' operand layout (k_tcgemm.cu): the
+// FP16 hi/lo parts of its column-scaled elements and the columns' exponents.
+struct TcImage {
+    void* data = nullptr;
+    int* ex = nullptr;
+    int rows = 0, cols = 0;
+};
+
 // ------------------------------------------------------------ dense complex contractions
 // Cpart[chunk] (element type T, M x N column major) = sum over the k of the
 // chunk of conj(A[k, m]) B[k, n]; then C = sum_chunks Cpart (double2, ldc)
@@ -163,7 +171,8 @@ void grid_fft3_batched(int N, const c2<T>* tw, c2<T>* data, int batch, int64_t b
 // the tensor cores (gemm_cn_tcg), the others to the streamed SIMT kernel.
 template <typename T>
 void gemm_cn(int M, int N, int K, const c2<T>* A, int64_t lda, const c2<T>* B, int64_t ldb,
-             double2* C, int ldc, double2* work, size_t work_elems, cudaStream_t st);
+             double2* C, int ldc, double2* work, size_t work_elems, cudaStream_t st, const TcImage* ia = nullptr,
+             const TcImage* ib = nullptr);
 size_t gemm_cn_work(int M, int N, int K);
 // C (ldc) = fixed-order sum of nchunk partials (M x N double2 each)
 void chunk_sum(int M, int N, int nchunk, const double2* part, double2* C, int ldc, cudaStream_t st);
@@ -195,43 +204,41 @@ void gemm_cn_capped(int M, int N, int K, const c2<T>* A, int64_t lda, const c2<T
 // For T = float, bwork receives an FP32 copy of B (K x N float2); it may be
 // the partial-sum buffer of gemm_cn (not in use across calls).
 // bwork_bytes: size of bwork; the tensor-core path (FP32, large blocks)
-// needs tcg_nn_work_bytes(N, K) and is skipped when it is 0 or too small.
+// needs tcg_nn_work_bytes(M, N, K) and is skipped when it is 0 or too small.
 template <typename T>
 void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B, int ldb,
              c2<T>* C, int64_t ldc, double alpha, double beta, void* bwork, cudaStream_t st,
-             size_t bwork_bytes = 0);
+             size_t bwork_bytes = 0, const TcImage* ia = nullptr);
 
 // Cout (ldc) = alpha A B + beta Cin (ldcin); Cin may differ from Cout (when
 // beta != 0 and it does, Cin is not modified).
 template <typename T>
 void gemm_nn_io(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B, int ldb, const c2<T>* Cin,
                 int64_t ldcin, c2<T>* Cout, int64_t ldc, double alpha, double beta, void* bwork, cudaStream_t st,
-                size_t bwork_bytes = 0);
+                size_t bwork_bytes = 0, const TcImage* ia = nullptr);
 
 // ------------------------------------------------------------ tensor-core contractions (k_tcgemm.cu)
-// Complex FP32 contractions of large blocks on tcgen05 (three TF32 products
-// per FP32 product, every K-step drained into round-to-nearest FP32 sums).
+// Complex FP32 contractions of large blocks on tcgen05 (three FP16 products
+// per FP32 product on column-scaled hi/lo splits, every stage drained into
+// round-to-nearest FP32 sums).
 bool tcg_enabled();
 bool tcg_cn_takes(int M, int N, int K);
 bool tcg_nn_takes(int M, int N, int K);
-// K-split depth of the A^H B products: about waves_x2 / 2 waves of CTAs
-// (the work buffer is sized for the deepest candidate, 4 waves)
+// runs of the A^H B products' unit sequence, in half waves of one CTA per SM
 void tcg_set_waves(int waves_x2);
 size_t tcg_cn_work_bytes(int M, int N, int K);
-size_t tcg_nn_work_bytes(int N, int K);
+size_t tcg_nn_work_bytes(int M, int N, int K);
+// Image of the block X (im.rows x im.cols, ld) in im's storage.
+size_t tcg_image_bytes(int rows, int cols);
+TcImage tcg_image_at(void* buf, int rows, int cols);
+bool tcg_split(const TcImage& im, const float2* X, int64_t ld, cudaStream_t st);
+// false: no image is kept from one contraction for the next (ROKS_TC_PRESPLIT=0)
+bool tcg_keep_images();
 bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2* B, int64_t ldb, double2* C, int ldc,
-                 void* work, size_t work_bytes, cudaStream_t st);
+                 void* work, size_t work_bytes, const TcImage* ia, const TcImage* ib, cudaStream_t st);
 bool gemm_nn_tcg(int M, int N, int K, const float2* A, int64_t lda, const double2* B, int ldb, const float2* Cin,
-                 int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, void* bwork, size_t bwork_bytes,
-                 cudaStream_t st);
-// An operand that does not change (the projector matrix) split once into
-// TF32 hi/lo blocks in the kernels' operand layout: the tall products A B
-// whose A is that matrix (same address, leading dimension and shape) then
-// copy it instead of converting it.  out holds tcg_presplit_bytes(M, K);
-// false when not registered.
-size_t tcg_presplit_bytes(int M, int K);
-bool tcg_presplit(int M, int K, const float2* A, int64_t lda, void* out, cudaStream_t st);
-void tcg_presplit_forget(const void* split);
+                 int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, void* work, size_t work_bytes,
+                 const TcImage* ia, cudaStream_t st);
 // 1 if a tensor-core wait gave up since the last call (then cleared)
 int tcg_timeout_take();
 // tensor-core contraction launches since the last call

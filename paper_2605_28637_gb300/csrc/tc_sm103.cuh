@@ -3,13 +3,13 @@
 // operand descriptors, commit to an mbarrier, bounded mbarrier waits and
 // tensor-memory loads.
 //
-// Operand layout used by this library: K-major without swizzle.  A tile of
-// R rows (the M or N extent) and KT 32-bit elements along K is stored as
-// 8-row x 16-byte core matrices: core (g, c) for row group g and K chunk c
-// (4 elements) starts at (g * KT/4 + c) * 128 bytes; row r of the core at
-// +16 r.  The descriptor's leading byte offset is the step between K chunks
-// (128 bytes) and its stride byte offset the step between row groups
-// (KT/4 * 128 bytes).
+// Operand layouts used by this library, without swizzle: core matrices of
+// 128 contiguous bytes.  K-major: a core matrix holds 8 rows (of the M or N
+// extent) of 16 bytes along K; the descriptor's leading byte offset is the
+// step to the next 16 bytes of K and its stride byte offset the step to the
+// next 8 rows.  MN-major: a core matrix holds 8 K of 16 bytes along the M (N)
+// extent; the leading byte offset is the step to the next 8 K and the stride
+// byte offset the step to the next 16 bytes of M (N).
 #pragma once
 
 #include <cstdint>
@@ -32,15 +32,15 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 
-// Instruction descriptor for kind::tf32: D = F32, A = B = TF32, both K-major,
+// Instruction descriptor for kind::f16: D = F32, A = B = FP16, both K-major,
 // dense; N >> 3 at bit 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
     return (1u << 4)                       // D format F32
-           | (2u << 7)                     // A format TF32
-           | (2u << 10)                    // B format TF32
            | ((uint32_t)(N >> 3) << 17)
            | ((uint32_t)(M >> 4) << 24);
 }
+constexpr uint32_t IDESC_NEG_A = 1u << 13;   // D += -A B
+constexpr uint32_t IDESC_A_MN = 1u << 15;    // A is MN-major
 
 // One warp allocates ncols tensor-memory columns; the base address is
 // written to *dst (shared memory).
@@ -56,12 +56,12 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 
 // D[tmem] (+)= A * B^T, issued by one thread.
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
@@ -111,20 +111,6 @@ __device__ __forceinline__ void fence_after_sync() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// 32 lanes x 8 consecutive columns of 32-bit tensor memory into v[0..7]
-// (lane = thread of the warp); the warp must own the lane quarter.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-    uint32_t r[8];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // 32 lanes x 16 consecutive columns of 32-bit tensor memory into v[0..15],
 // without waiting (tmem_wait_ld before the registers are read).
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float* v) {
@@ -160,13 +146,6 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
         : "memory");
     return done != 0;
 }
-// global -> shared bulk copy (bytes a multiple of 16, both ends 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
 // 2-D tensor copy of the box at (x = first row, y = first column)
 __device__ __forceinline__ void tma_2d(void* dst, const void* map, int x, int y, uint64_t* bar) {
     asm volatile(
@@ -176,19 +155,13 @@ __device__ __forceinline__ void tma_2d(void* dst, const void* map, int x, int y,
         : "memory");
 }
 
-// Round to the nearest TF32 value (kept in an FP32 container).
-__device__ __forceinline__ float to_tf32(float x) {
-    uint32_t u;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
-    return __uint_as_float(u);
-}
-
-// x = hi + mid + lo with TF32 values; |x - hi - mid - lo| <= 2^-33 |x|.
-__device__ __forceinline__ void split3_tf32(float x, float& hi, float& mid, float& lo) {
-    hi = to_tf32(x);
-    const float r = x - hi;
-    mid = to_tf32(r);
-    lo = to_tf32(r - mid);
+// 4-D tensor copy of the box at (0, y, z, w)
+__device__ __forceinline__ void tma_4d(void* dst, const void* map, int y, int z, int w, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5}], [%6];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
+        : "memory");
 }
 
 }  // namespace tc
