@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
     __shared__ uint32_t tmem_base;
     __shared__ volatile int failed;
     unsigned char* ring = gb_smem + ((1024u - (tc::smem_u32(gb_smem) & 1023u)) & 1023u);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
     const int64_t u0 = NN ? 0 : sk.len * blockIdx.x;
     // the first tile and stage (the loops then step them); after a tile's
     // last stage the next tile is t + tstep
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------ producer
-        if (warp == 0 && lane == 0) {
+        if (warp == 0 && tc::elect_one()) {
             int issued = 0, t_cur = t_first, s_cur = s_first;
             for (int i = 0; i < ns; ++i) {
                 const int ma = NN ? t_cur / sk.fast : t_cur % sk.fast;
@@ -189,7 +189,11 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                 gwait(&full[i % GB_ST], (uint32_t)((i / GB_ST) & 1), GB_DEFAULT_WAIT, &failed);
         }
         // ------------------------------------------------ MMA issue
-        if (warp == 1 && lane == 0) {
+        if (warp == 1) {
+            // (one elected lane of a whole warp issues: 57 cycles an MMA; under a
+            // test of the lane the loop's bookkeeping was per lane, 85 cycles,
+            // and P (D B) at mgo-120 took 479 us instead of 448)
+            const bool leader = tc::elect_one();
             // A: K-major over [chunk 8192][part 4096][plane 2048][group 128], or
             // MN-major over [part 16384][plane 8192][group 2048][chunk 128];
             // B: K-major over [chunk 4 wb][part 2 wb][plane wb][group 128]
@@ -198,10 +202,11 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
             const uint64_t db0 = tc::make_desc(0, 4 * wb, 128);
             constexpr uint32_t a_part = NN ? 16384 : 4096, a_plane = NN ? 8192 : 2048, a_k = NN ? 4096 : 16384;
             bool ok = true;
+            int sl = 0;
             for (int i = 0; i < ns && ok; ++i) {
-                const int sl = i % GB_ST, b = i % GB_ACC;
-                if (!gwait(&full[sl], (uint32_t)((i / GB_ST) & 1), wcap, &failed) ||
-                    (i >= GB_ACC && !gwait(&acc_empty[b], (uint32_t)((i / GB_ACC - 1) & 1), wcap, &failed))) {
+                const int b = i % GB_ACC;
+                if (!warp_wait(&full[sl], (uint32_t)((i / GB_ST) & 1), wcap, &failed) ||
+                    (i >= GB_ACC && !warp_wait(&acc_empty[b], (uint32_t)((i / GB_ACC - 1) & 1), wcap, &failed))) {
                     ok = false;
                     break;
                 }
@@ -222,22 +227,27 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                 // products are those with Br: in A B, where B is near a real
                 // multiple of the identity or has a real diagonal, its large
                 // elements are then truncated least often
+                if (leader) {
 #pragma unroll
-                for (int o = 0; o < 2; ++o) {
-                    const bool n0 = !NN && o == 1, n1 = NN && o == 0;   // the terms with Br, with Bi
-                    mm(o, 1, 1 - o, 0, 1, n1, 1u);
-                    mm(o, 0, 1 - o, 1, 1, n1, 0u);
-                    mm(o, 1, o, 0, 0, n0, 0u);
-                    mm(o, 0, o, 1, 0, n0, 0u);
-                    mm(o, 0, 1 - o, 0, 1, n1, 0u);
-                    mm(o, 0, o, 0, 0, n0, 0u);
+                    for (int o = 0; o < 2; ++o) {
+                        const bool n0 = !NN && o == 1, n1 = NN && o == 0;   // the terms with Br, with Bi
+                        mm(o, 1, 1 - o, 0, 1, n1, 1u);
+                        mm(o, 0, 1 - o, 1, 1, n1, 0u);
+                        mm(o, 1, o, 0, 0, n0, 0u);
+                        mm(o, 0, o, 1, 0, n0, 0u);
+                        mm(o, 0, 1 - o, 0, 1, n1, 0u);
+                        mm(o, 0, o, 0, 0, n0, 0u);
+                    }
+                    tc::commit(&acc_full[b]);
+                    tc::commit(&empty[sl]);   // the slot is free once these MMAs complete
                 }
-                tc::commit(&acc_full[b]);
-                tc::commit(&empty[sl]);   // the slot is free once these MMAs complete
+                __syncwarp();
+                sl = sl == GB_ST - 1 ? 0 : sl + 1;
             }
             if (!ok) give_up(&failed);
             // every MMA issued completes before the tensor memory is freed
-            tc::commit(&mma_done);
+            if (leader) tc::commit(&mma_done);
+            __syncwarp();
             gwait(&mma_done, 0u, GB_DEFAULT_WAIT, &failed);
         }
         __syncwarp();   // the role's lane rejoins its warp
@@ -771,6 +781,21 @@ bool gemm_nn_tcg(int M, int N, int K, const float2* A, int64_t lda, const double
     k_tcgemm<true><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, stages(K), sk, tmA, tmB, mb.ex, nullptr, Cin, ldcin,
                                                          Cout, ldc, alpha, beta, wait_polls());
     return true;
+}
+
+// device address of the flag (null if it cannot be had)
+int* tcg_timeout_flag() {
+    constexpr int kMaxDev = 64;
+    static int* addr[kMaxDev] = {nullptr};
+    int dev = 0;
+    void* p = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev ||
+        (!addr[dev] && cudaGetSymbolAddress(&p, g_tcg_timeout) != cudaSuccess)) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (!addr[dev]) addr[dev] = static_cast<int*>(p);
+    return addr[dev];
 }
 
 int tcg_timeout_take() {

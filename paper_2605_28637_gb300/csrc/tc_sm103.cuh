@@ -21,6 +21,18 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// One lane of a converged warp (the same one on every call).  Code that
+// issues MMAs runs in a warp-uniform branch under this predicate, so that its
+// descriptors stay in uniform registers: under a test of the thread index
+// each MMA's operands were moved there one by one, 85 cycles an MMA.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// the warp's index, known to be the same for all its lanes
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // Shared-memory matrix descriptor (no swizzle, sm_100-family version bits).
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
     uint64_t d = 0;
@@ -41,6 +53,7 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
 }
 constexpr uint32_t IDESC_NEG_A = 1u << 13;   // D += -A B
 constexpr uint32_t IDESC_A_MN = 1u << 15;    // A is MN-major
+constexpr uint32_t IDESC_B_MN = 1u << 16;    // B is MN-major
 
 // One warp allocates ncols tensor-memory columns; the base address is
 // written to *dst (shared memory).
@@ -123,6 +136,18 @@ __device__ __forceinline__ void fence_after_sync() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// 32 lanes x 8 consecutive columns of 32-bit tensor memory into v[0..7],
+// without waiting.
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, float* v) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // 32 lanes x 16 consecutive columns of 32-bit tensor memory into v[0..15],
 // without waiting (tmem_wait_ld before the registers are read).
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float* v) {
@@ -168,6 +193,13 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
         : "r"(smem_u32(b)), "r"(parity)
         : "memory");
     return done != 0;
+}
+// global -> shared bulk copy (bytes a multiple of 16, both ends 16-byte aligned)
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
 }
 // 2-D tensor copy of the box at (x = first row, y = first column)
 __device__ __forceinline__ void tma_2d(void* dst, const void* map, int x, int y, uint64_t* bar) {
