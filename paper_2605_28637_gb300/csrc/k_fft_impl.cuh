@@ -609,6 +609,9 @@ struct BandFft {
         else
             pr ? go(k_band_x_density<T, N, true, true>) : go(k_band_x_density<T, N, true, false>);
         if (!sl) return;
+        density_reduce(ng, sl, r3, st);
+    }
+    static void density_reduce(int ng, const typename DensAcc<T>::S* sl, typename DensAcc<T>::S* r3, cudaStream_t st) {
         const int N3 = N * N * N;
         roks::count_launch(), k_density_reduce<T><<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, ng, sl, r3);
     }
@@ -673,6 +676,12 @@ void band_x_density(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, double* r
                                                        part_sel, cls_override, st)));
 }
 template <typename T>
+void band_density_reduce(int N, int ng, const double* slot, double* rho3, cudaStream_t st) {
+    using DS = typename DensAcc<T>::S;
+    ROKS_GRID_DISPATCH(N, (BandFft<T, NN>::density_reduce(ng, reinterpret_cast<const DS*>(slot),
+                                                          reinterpret_cast<DS*>(rho3), st)));
+}
+template <typename T>
 void grid_fft3(int N, const c2<T>* tw, c2<T>* data, int dir, cudaStream_t st) {
     ROKS_GRID_DISPATCH(N, (BandFft<T, NN>::grid3(tw, data, dir, 1, 0, st)));
 }
@@ -694,6 +703,7 @@ void grid_fft3_batched(int N, const c2<T>* tw, c2<T>* data, int batch, int64_t b
                                 int64_t, const T*, const T*, int, int, int, cudaStream_t);                      \
     template void band_x_density<T>(const Sphere&, const c2<T>*, const c2<T>*, double*, double*, int, int, int,  \
                                     int, double, cudaStream_t, int, int);                                        \
+    template void band_density_reduce<T>(int, int, const double*, double*, cudaStream_t);                        \
     template void grid_fft3<T>(int, const c2<T>*, c2<T>*, int, cudaStream_t);
 
 }  // namespace roks

@@ -567,15 +567,21 @@ __global__ void __launch_bounds__(RB) k_hartree_G(int N, T inv, T fpb, c2<T>* __
     if (threadIdx.x == 0) part[blockIdx.x] = deh;
 }
 
-// V^k = w_k (V_loc + V_H) + xc3[k]; partial sums <a|V^c|a>, <b|V^c|b> (rho_a, rho_b).
+// V^k = w_k (V_loc + V_H) + xc3[k]; partial sums <a|V^c|a>, <b|V^c|b> (rho_a,
+// rho_b); the largest |V^k| of each class in vmax, when given.
 template <typename T>
 __global__ void __launch_bounds__(RB) k_pot_class(int N3, const T* __restrict__ vloc,
                                                   const c2<T>* __restrict__ vh, const T* __restrict__ xc3,
                                                   const typename DensAcc<T>::S* __restrict__ rho3, PotCoef cf,
                                                   T* __restrict__ Vk,
-                                                  double* __restrict__ Vk64, double* __restrict__ part) {
+                                                  double* __restrict__ Vk64, double* __restrict__ part,
+                                                  float* __restrict__ vmax) {
     __shared__ double sh[RB];
+    __shared__ int vm[3];
+    if (threadIdx.x < 3) vm[threadIdx.x] = 0;
+    __syncthreads();
     T ea = 0, eb = 0;
+    float mc = 0.f, ma = 0.f, mb = 0.f;
     const T w0 = T(cf.w[0]), w1 = T(cf.w[1]), w2 = T(cf.w[2]);
     for (int p = blockIdx.x * RB + threadIdx.x; p < N3; p += gridDim.x * RB) {
         const T v0 = vloc[p] + vh[p].x;
@@ -585,6 +591,11 @@ __global__ void __launch_bounds__(RB) k_pot_class(int N3, const T* __restrict__ 
         Vk[p] = vc;
         Vk[N3 + p] = va;
         Vk[2 * N3 + p] = vb;
+        if (vmax) {
+            mc = fmaxf(mc, fabsf(float(vc)));
+            ma = fmaxf(ma, fabsf(float(va)));
+            mb = fmaxf(mb, fabsf(float(vb)));
+        }
         if (Vk64) {
             Vk64[p] = double(vc);
             Vk64[N3 + p] = double(va);
@@ -593,8 +604,15 @@ __global__ void __launch_bounds__(RB) k_pot_class(int N3, const T* __restrict__ 
         ea += vc * T(DensAcc<T>::value(rho3[N3 + p]));
         eb += vc * T(DensAcc<T>::value(rho3[2 * N3 + p]));
     }
+    if (vmax) {
+        // floats >= 0 order like their bits; vmax was zeroed before the launch
+        atomicMax(&vm[0], __float_as_int(mc));
+        atomicMax(&vm[1], __float_as_int(ma));
+        atomicMax(&vm[2], __float_as_int(mb));
+    }
     const double dea = block_sum_t<T>(ea, sh);
     const double deb = block_sum_t<T>(eb, sh);
+    if (vmax && threadIdx.x < 3) atomicMax(reinterpret_cast<int*>(vmax) + threadIdx.x, vm[threadIdx.x]);
     if (threadIdx.x == 0) {
         part[blockIdx.x * 2 + 0] = dea;
         part[blockIdx.x * 2 + 1] = deb;
@@ -723,7 +741,7 @@ constexpr int kPotBlocks = 512;
 template <typename T>
 void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoef& cf, c2<T>* grid,
                 T* xc3, const c2<T>* tw, T* Vk, double* Vk64, double* part, double* out6,
-                cudaStream_t st, bool energies_only, const GgaWork* gga) {
+                cudaStream_t st, bool energies_only, const GgaWork* gga, float* vmax) {
     // out6: [E_x^M, E_x^T, E_loc, E_H, <a|V^c|a>, <b|V^c|b>]; energies_only
     // stops after E_H (out6[4..5] and Vk are left as they were)
     const int N3 = N * N * N;
@@ -773,7 +791,9 @@ void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoe
                                                                            gg, xc3);
     }
     grid_fft3<T>(N, tw, grid, +1, st);
-    roks::count_launch(), k_pot_class<T><<<kPotBlocks, RB, 0, st>>>(N3, vloc, grid, xc3, r3, cf, Vk, Vk64, part);
+    if (vmax) cudaMemsetAsync(vmax, 0, 3 * sizeof(float), st);
+    roks::count_launch(), k_pot_class<T><<<kPotBlocks, RB, 0, st>>>(N3, vloc, grid, xc3, r3, cf, Vk, Vk64, part,
+                                                                        vmax);
     roks::count_launch(), k_partials_final<<<2, RB, 0, st>>>(kPotBlocks, 2, part, out6 + 4, dvol, dvol, 0, 0);
 }
 
@@ -805,7 +825,7 @@ void axpy(int npw, int nb, const c2<T>* x, int64_t ldx, const c2<T>* y, int64_t 
                                   double*, double*, double, cudaStream_t);                                     \
     template void potentials<T>(int, double, const double*, const T*, const PotCoef&, c2<T>*, T*,             \
                                 const c2<T>*, T*, double*, double*, double*, cudaStream_t, bool,              \
-                                const GgaWork*);                                                               \
+                                const GgaWork*, float*);                                                       \
     template void precondition<T>(int, int, const c2<T>*, int64_t, const T*, const double*, c2<T>*,           \
                                   int64_t, cudaStream_t);                                                      \
     template void axpy<T>(int, int, const c2<T>*, int64_t, const c2<T>*, int64_t, const double*, double,      \

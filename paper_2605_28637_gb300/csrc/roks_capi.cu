@@ -82,6 +82,8 @@ struct roks_ctx {
     double2* d_tw64 = nullptr;     // twiddles (FP64)
     // band transforms
     void *d_Zc = nullptr, *d_Yp = nullptr;
+    void* d_xtab = nullptr;       // table of the x stages on the tensor cores (null: not taken)
+    float* d_vmax = nullptr;      // largest |V^k| of each class (with d_xtab)
     // grid
     double* d_rho3 = nullptr;
     double* d_rho_slot = nullptr;   // closed-shell density partials per band group
@@ -319,6 +321,50 @@ struct Impl {
         ctx->yp_ld = ld;
     }
 
+    // x stage of the density (bands b0 ... with the planes from Yp on), on the
+    // tensor cores where they take it ((Re psi)^2 or (Im psi)^2 alone: never)
+    static void x_density(roks_ctx* ctx, const V* Yp, double* rho3, double* slot, int ngroups, int b0, int nbb,
+                          int n_closed, int part_sel = 0, int cls_override = -1) {
+        const Sphere s = sphere(ctx);
+        const double scale = 1.0 / ctx->omega;
+        if constexpr (sizeof(T) == 4) {
+            if (ctx->d_xtab && part_sel == 0 && nbb > 0) {
+                const int gs = (nbb + ngroups - 1) / ngroups, ng = (nbb + gs - 1) / gs;
+                xdft_density(s, ctx->d_xtab, Yp, rho3, slot, gs, ng, b0, nbb, n_closed, (float)scale, cls_override,
+                             ctx->st);
+                if (slot) band_density_reduce<T>(ctx->N, ng, slot, rho3, ctx->st);
+                return;
+            }
+        }
+        band_x_density<T>(s, ccv(ctx->d_tw), Yp, rho3, slot, ngroups, b0, nbb, n_closed, scale, ctx->st, part_sel,
+                          cls_override);
+    }
+
+    // x stage of the apply, in place on the planes Yp of bands b0 ...
+    static void x_apply(roks_ctx* ctx, V* Yp, const V* Xx, int b0, int nbb, int n_closed, int split_band) {
+        const Sphere s = sphere(ctx);
+        const T scale = T(1.0 / (double(ctx->N) * ctx->N * ctx->N));
+        const T* Vk = static_cast<const T*>(ctx->d_Vk);
+        if constexpr (sizeof(T) == 4) {
+            if (ctx->d_xtab && !Xx) {
+                auto run = [&](int first, int count) {
+                    xdft_apply(s, ctx->d_xtab, Yp + (int64_t)(first - b0) * s.np * s.N * s.N, Vk, ctx->d_vmax, first,
+                               count, n_closed, scale, ctx->st);
+                };
+                if (split_band < b0 || split_band >= b0 + nbb) {
+                    run(b0, nbb);
+                } else {
+                    run(b0, split_band - b0);
+                    band_x_apply<T>(s, ccv(ctx->d_tw), Yp + (int64_t)(split_band - b0) * s.np * s.N * s.N, Vk, nullptr,
+                                    split_band, 1, n_closed, split_band, scale, ctx->st);
+                    run(split_band + 1, b0 + nbb - split_band - 1);
+                }
+                return;
+            }
+        }
+        band_x_apply<T>(s, ccv(ctx->d_tw), Yp, Vk, Xx, b0, nbb, n_closed, split_band, scale, ctx->st);
+    }
+
     // Exact exchange of the bands whose plane data sit in Yp: real-space
     // orbitals, pair integrals, energies and (want_field) the exchange fields.
     static void exchange(roks_ctx* ctx, bool want_field) {
@@ -362,8 +408,8 @@ struct Impl {
             PROF("fft_x_density");
             if (ctx->split_t < 0) {
                 // the occupied bands (the empty ones carry no density)
-                band_x_density<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot, ctx->dens_groups,
-                                  0, ctx->nbt - ctx->ne, ctx->nct, 1.0 / ctx->omega, st);
+                x_density(ctx, cv(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot, ctx->dens_groups, 0, ctx->nbt - ctx->ne,
+                          ctx->nct);
                 if (ctx->ne > 0) {
                     // each empty band's own density, for its <e|V^k|e> (the
                     // kernel indexes the planes from the launch's first band
@@ -373,21 +419,19 @@ struct Impl {
                     for (int i = 0; i < ctx->ne; ++i) {
                         const int e = ctx->nocc + i;
                         const V* yo = ccv(ctx->d_Yp) + (int64_t)e * ctx->np * ctx->N * ctx->N;
-                        band_x_density<T>(s, ccv(ctx->d_tw), yo, ctx->d_rho_e + i * N3, nullptr, 1, e, 1, ctx->nc,
-                                          1.0 / ctx->omega, st, 0, 1);
+                        x_density(ctx, yo, ctx->d_rho_e + i * N3, nullptr, 1, e, 1, ctx->nc, 0, 1);
                     }
                 }
             } else {
                 // Gamma point: the closed pairs, then the packed open pair's
                 // real part (a) and imaginary part (b) into their own classes
                 if (ctx->nct > 0)
-                    band_x_density<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot,
-                                      ctx->dens_groups, 0, ctx->nct, ctx->nct, 1.0 / ctx->omega, st);
+                    x_density(ctx, cv(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot, ctx->dens_groups, 0, ctx->nct,
+                              ctx->nct);
                 // (the kernel indexes the plane buffer from the launch's first band)
                 const V* yo = ccv(ctx->d_Yp) + (int64_t)ctx->split_t * ctx->np * ctx->N * ctx->N;
                 for (int part = 1; part <= 2; ++part)
-                    band_x_density<T>(s, ccv(ctx->d_tw), yo, ctx->d_rho3, nullptr, 1, ctx->split_t, 1, ctx->nct,
-                                      1.0 / ctx->omega, st, part, part);
+                    x_density(ctx, yo, ctx->d_rho3, nullptr, 1, ctx->split_t, 1, ctx->nct, part, part);
             }
         }
         column_sums<T>(0, ctx->npw, ctx->nb, p, ld, nullptr, 0, static_cast<const T*>(ctx->d_g2half), ctx->d_colpart, ctx->d_kin_b, st);
@@ -416,7 +460,7 @@ struct Impl {
         potentials<T>(ctx->N, ctx->L, ctx->d_rho3, static_cast<const T*>(ctx->d_vloc_t), ctx->cf,
                       reinterpret_cast<V*>(ctx->d_grid), reinterpret_cast<T*>(ctx->d_xc3), ccv(ctx->d_tw),
                       static_cast<T*>(ctx->d_Vk), nullptr, ctx->d_part, ctx->d_out6, st, energies_only,
-                      ctx->xc == ROKS_XC_PBE_X ? &ctx->gga : nullptr);
+                      ctx->xc == ROKS_XC_PBE_X ? &ctx->gga : nullptr, ctx->d_vmax);
         energy_combine(ctx->d_kin_b, ctx->d_nl_b, ctx->nocc, ctx->d_wband, ctx->d_out6, ctx->cM, ctx->cT,
                        ctx->alpha, ctx->alpha != 0.0 ? ctx->d_hf2 : nullptr, ctx->d_E, st);
         CK(cudaGetLastError());
@@ -447,14 +491,10 @@ struct Impl {
         {
             PROF("fft_x_apply");
             const int nx = ctx->nbt - ctx->ne;
-            band_x_apply<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp), static_cast<const T*>(ctx->d_Vk),
-                            ctx->alpha != 0.0 ? ccv(ctx->d_Xx) : nullptr, 0, nx, ctx->nct, ctx->split_t,
-                            T(1.0 / (double(N) * N * N)), st);
+            x_apply(ctx, cv(ctx->d_Yp), ctx->alpha != 0.0 ? ccv(ctx->d_Xx) : nullptr, 0, nx, ctx->nct, ctx->split_t);
             // empty bands: F^c (a closed count past the last band gives class 0)
             if (ctx->ne > 0)
-                band_x_apply<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp) + (int64_t)nx * ctx->np * N * N,
-                                static_cast<const T*>(ctx->d_Vk), nullptr, nx, ctx->ne, ctx->nb, -1,
-                                T(1.0 / (double(N) * N * N)), st);
+                x_apply(ctx, cv(ctx->d_Yp) + (int64_t)nx * ctx->np * N * N, nullptr, nx, ctx->ne, ctx->nb, -1);
         }
         ctx->yp_psi = nullptr;   // the x stage works in place
         { PROF("fft_y_fwd"); band_y_fwd<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp), cv(ctx->d_Zc), ctx->nbt, st); }
@@ -1127,17 +1167,16 @@ int pick_fastest(roks_ctx* ctx, const int* cand, int nc, double* ms, F fn) {
 // each timed on the context's own buffers and sizes.
 roks_status autotune(roks_ctx* ctx) {
     enter(ctx);
-    const Sphere s = sphere(ctx);
     const int g_cand[3] = {2, 4, 8};
     if (ctx->prec == ROKS_FP64)
         ctx->dens_groups = pick_fastest(ctx, g_cand, 3, ctx->tune_ms, [&](int g) {
-            band_x_density<double>(s, static_cast<const double2*>(ctx->d_tw), static_cast<double2*>(ctx->d_Yp),
-                                   ctx->d_rho3, ctx->d_rho_slot, g, 0, ctx->nbt - ctx->ne, ctx->nct, 1.0 / ctx->omega, ctx->st);
+            Impl<double>::x_density(ctx, static_cast<double2*>(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot, g, 0,
+                                    ctx->nbt - ctx->ne, ctx->nct);
         });
     else
         ctx->dens_groups = pick_fastest(ctx, g_cand, 3, ctx->tune_ms, [&](int g) {
-            band_x_density<float>(s, static_cast<const float2*>(ctx->d_tw), static_cast<float2*>(ctx->d_Yp),
-                                  ctx->d_rho3, ctx->d_rho_slot, g, 0, ctx->nbt - ctx->ne, ctx->nct, 1.0 / ctx->omega, ctx->st);
+            Impl<float>::x_density(ctx, static_cast<float2*>(ctx->d_Yp), ctx->d_rho3, ctx->d_rho_slot, g, 0,
+                                   ctx->nbt - ctx->ne, ctx->nct);
         });
     // the largest A^H B product of a step that runs on the tensor cores
     const int M = ctx->nproj >= ctx->nb ? ctx->nproj : ctx->nb;
@@ -1368,6 +1407,10 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
     AL(ctx->d_tw64, sizeof(double2) * N);
     AL(ctx->d_Zc, cs * (size_t)ctx->nbt * ctx->ncol * N);
     AL(ctx->d_Yp, cs * (size_t)ctx->nbt * ctx->np * N * N);
+    if (!f64 && xdft_takes(N, n)) {
+        AL(ctx->d_xtab, xdft_table_bytes());
+        AL(ctx->d_vmax, sizeof(float) * 3);
+    }
     if (ctx->gamma) AL(ctx->d_Cpk, cs * (size_t)ctx->ldc_pk * ctx->nbt);
     AL(ctx->d_rho3, sizeof(double) * 3 * N3);
     AL(ctx->d_rho_slot, sizeof(double) * (opt->autotune ? kDensityGroupsMax : kDensityGroups) * N3);
@@ -1537,6 +1580,13 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
         std::vector<float2> t32(N);
         for (int t = 0; t < N; ++t) t32[t] = make_float2((float)tw64[t].x, (float)tw64[t].y);
         cudaMemcpyAsync(ctx->d_tw, t32.data(), sizeof(float2) * N, cudaMemcpyHostToDevice, ctx->st);
+        cudaStreamSynchronize(ctx->st);
+    }
+    if (ctx->d_xtab) {
+        std::vector<unsigned char> tab(xdft_table_bytes());
+        xdft_table(N, n, tab.data());
+        tcg_timeout_flag();   // (looks its address up outside any capture)
+        cudaMemcpyAsync(ctx->d_xtab, tab.data(), tab.size(), cudaMemcpyHostToDevice, ctx->st);
         cudaStreamSynchronize(ctx->st);
     }
     // -------- model on the device

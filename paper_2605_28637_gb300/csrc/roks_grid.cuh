@@ -74,7 +74,7 @@ struct GgaWork {
 template <typename T>
 void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoef& cf, c2<T>* grid,
                 T* xc3, const c2<T>* tw, T* Vk, double* Vk64, double* part, double* out6,
-                cudaStream_t st, bool energies_only = false, const GgaWork* gga = nullptr);
+                cudaStream_t st, bool energies_only = false, const GgaWork* gga = nullptr, float* vmax = nullptr);
 size_t potentials_part_elems();
 template <typename T>
 void precondition(int npw, int nb, const c2<T>* gI, int64_t ld, const T* g2h, const double* sums, c2<T>* out,

@@ -122,6 +122,24 @@ void band_x_density(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, double* r
                     int b0, int nbb, int n_closed, double scale, cudaStream_t st, int part_sel = 0,
                     int cls_override = -1);
 
+// rho3[0] = sum of the ng closed-shell slots in group order
+template <typename T>
+void band_density_reduce(int N, int ng, const double* slot, double* rho3, cudaStream_t st);
+
+// ------------------------------------------------------------ x stages on the tensor cores (k_xdft.cu)
+// FP32, N = 72, 96, 120, spheres that fit the pruned first passes.  tab: the
+// transform's table (xdft_table_bytes(), filled on the host by xdft_table).
+bool xdft_takes(int N, int nmax);
+size_t xdft_table_bytes();
+void xdft_table(int N, int nmax, void* host);
+// band_x_apply without exchange fields or a split band; vmax[class]: an upper
+// bound of |V| (device)
+void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, const float* vmax, int b0, int nbb,
+                int n_closed, float scale, cudaStream_t st);
+// band_x_density of |psi|^2 without the sum of the slots; bands in ng groups of gs
+void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rho3, double* slot, int gs, int ng,
+                  int b0, int nbb, int n_closed, float scale, int cls_override, cudaStream_t st);
+
 // ------------------------------------------------------------ Gamma point (k_gamma.cu)
 // Real orbitals are stored on the half sphere (G = 0 and the Miller triples
 // after it in the basis order, the contiguous tail of the full basis from
@@ -239,8 +257,10 @@ bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2
 bool gemm_nn_tcg(int M, int N, int K, const float2* A, int64_t lda, const double2* B, int ldb, const float2* Cin,
                  int64_t ldcin, float2* Cout, int64_t ldc, float alpha, float beta, void* work, size_t work_bytes,
                  const TcImage* ia, cudaStream_t st);
-// 1 if a tensor-core wait gave up since the last call (then cleared)
+// 1 if a tensor-core wait gave up since the last call (then cleared); the
+// flag's device address
 int tcg_timeout_take();
+int* tcg_timeout_flag();
 // tensor-core contraction launches since the last call
 long long tcg_launches_take();
 
