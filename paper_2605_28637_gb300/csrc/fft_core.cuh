@@ -82,7 +82,9 @@ __device__ __forceinline__ float2 cfma(float2 a, float s, float2 c) { return __f
 // ---------------------------------------------------------------- plans
 // Radix sequence of a transform length.  The grid sizes of the workloads get
 // two passes with register codelets up to 16 points (96 = 12 x 8,
-// 120 = 15 x 8, 72 = 9 x 8, 48 = 8 x 6, 24 = 8 x 3, 32 = 8 x 4, 16 = 4 x 4);
+// 120 = 15 x 8, 72 = 9 x 8, 48 = 8 x 6, 24 = 8 x 3, 32 = 8 x 4, 16 = 4 x 4),
+// and so do the exchange grid's others (54 = 9 x 6, 60 = 10 x 6, 80 = 10 x 8,
+// 108 = 12 x 9, 40 = 8 x 5, 64 = 8 x 8);
 // other lengths fall back to factors of 8, 5, 4, 3, 2 in that order.
 __host__ __device__ constexpr int plan_radix(int n, int pass) {
     switch (n) {
@@ -90,6 +92,10 @@ __host__ __device__ constexpr int plan_radix(int n, int pass) {
         case 120: return pass == 0 ? 15 : (pass == 1 ? 8 : 1);
         case 72: return pass == 0 ? 9 : (pass == 1 ? 8 : 1);
         case 48: return pass == 0 ? 8 : (pass == 1 ? 6 : 1);
+        case 54: return pass == 0 ? 9 : (pass == 1 ? 6 : 1);
+        case 60: return pass == 0 ? 10 : (pass == 1 ? 6 : 1);
+        case 80: return pass == 0 ? 10 : (pass == 1 ? 8 : 1);
+        case 108: return pass == 0 ? 12 : (pass == 1 ? 9 : 1);
         case 16: return pass == 0 ? 4 : (pass == 1 ? 4 : 1);
         default: break;
     }

@@ -2,9 +2,11 @@
 // screened-hybrid workload): pair densities rho_jn = psi_j^* psi_n on the
 // full grid, W_jn = sum_G v(G) rho_jn(G) e^{iGr}, the exchange field
 // X_n = -alpha Omega^{1/2} sum_j w(k_n, k_j) psi_j W_jn that the x-stage apply
-// adds next to V psi, and the pair integrals K_jn = Omega sum_G v |rho_jn(G)|^2.
+// adds next to V psi (or, from a grid of its own, z_fwd_add to F|n>), and the pair integrals K_jn = Omega sum_G v |rho_jn(G)|^2.
 // Pairs j <= n are used once: W_nj = conj(W_jn).  The grid work of a batch
 // of pairs (k_exx_grid.cuh) fuses the pointwise steps into the transforms.
+#include <algorithm>
+
 #include "roks_exx.cuh"
 
 namespace roks {
@@ -90,6 +92,28 @@ __global__ void k_exx_open_diag(int nb, const double* __restrict__ Kmat, ExxCoef
 }
 
 // ------------------------------------------------------------------ host side
+int exx_grid(int N, int nmax, int nb) {
+    for (int m : {16, 24, 32, 40, 48, 54, 60, 64, 72, 80, 96, 108, 120}) {
+        if (m < 4 * nmax + 1 || m > N) continue;
+        // five launches, some 12 us, against 14 ps a point and pair
+        const int64_t saved = (int64_t)nb * (nb + 1) / 2 * ((int64_t)N * N * N - (int64_t)m * m * m);
+        return saved >= 1 << 20 ? m : N;
+    }
+    return N;
+}
+
+int exx_tiles(int nb, int tile, std::vector<ExxTile>& out) {
+    int p0 = 0;
+    for (int n0 = 0; n0 < nb; n0 += tile)
+        for (int j0 = 0; j0 <= n0; j0 += tile) {
+            const int bn = std::min(tile, nb - n0), bj = std::min(tile, nb - j0);
+            const int np = j0 == n0 ? bn * (bn + 1) / 2 : bn * bj;
+            out.push_back(ExxTile{j0, bj, n0, bn, p0, np});
+            p0 += np;
+        }
+    return p0;
+}
+
 template <typename T>
 void exx_setup_kernel(int N, double L, int bare, T* vG, cudaStream_t st) {
     const int64_t N3 = (int64_t)N * N * N;
@@ -100,16 +124,17 @@ void exx_setup_kernel(int N, double L, int bare, T* vG, cudaStream_t st) {
 
 template <typename T>
 void exx_pairs(const ExxArgs<T>& a, bool want_field, cudaStream_t st) {
-    const int64_t N3 = (int64_t)a.N * a.N * a.N;
-    const int nblk = kExxBlocks;
+    const int64_t M3 = (int64_t)a.M * a.M * a.M;
     const double omega = a.L * a.L * a.L;
-    if (want_field) cudaMemsetAsync(a.X, 0, sizeof(c2<T>) * N3 * a.nb, st);
-    for (int p0 = 0; p0 < a.npairs; p0 += a.batch) {
-        const int np = a.npairs - p0 < a.batch ? a.npairs - p0 : a.batch;
-        exx_batch_grid<T>(a, p0, np, want_field, st);
-        roks::count_launch(), k_exx_pair_sum<<<(np + 127) / 128, 128, 0, st>>>(np, nblk, a.part, a.pj, a.pn, p0,
-                                                                              omega / double(N3), a.nb, a.Kmat);
+    if (want_field) cudaMemsetAsync(a.X, 0, sizeof(c2<T>) * M3 * a.nb, st);
+    for (int t0 = 0; t0 < a.ntiles;) {
+        int t1 = t0 + 1;
+        while (t1 < a.ntiles && a.tiles[t1].p0 + a.tiles[t1].np - a.tiles[t0].p0 <= a.batch) ++t1;
+        exx_batch_grid<T>(a, t0, t1, want_field, st);
+        t0 = t1;
     }
+    roks::count_launch(), k_exx_pair_sum<<<(a.npairs + 127) / 128, 128, 0, st>>>(a.npairs, a.M, a.part, a.pj, a.pn, 0,
+                                                                                omega / double(M3), a.nb, a.Kmat);
     roks::count_launch(), k_exx_energy<<<1, 256, 0, st>>>(a.nb, a.Kmat, a.cf, a.hf2);
     roks::count_launch(), k_exx_open_diag<<<1, 32, 0, st>>>(a.nb, a.Kmat, a.cf, a.open_diag);
 }

@@ -79,9 +79,11 @@ __global__ void __launch_bounds__(kThreads) k_band_z_inv(Sphere s, const c2<T>* 
     }
 }
 
-// KIN: add the kinetic term w_k |G|^2/2 psi(G) while scattering out; without
-// it the transform alone (the Gamma-point unpack adds the kinetic term)
-template <typename T, int N, bool KIN>
+// ZK_KIN: add the kinetic term w_k |G|^2/2 psi(G) while scattering out;
+// ZK_PLAIN: the transform alone (the Gamma-point unpack adds the kinetic
+// term); ZK_ADD: added to what out holds (the exchange fields)
+enum { ZK_PLAIN, ZK_KIN, ZK_ADD };
+template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(kThreads) k_band_z_fwd(Sphere s, const c2<T>* __restrict__ tw,
                                                          const c2<T>* __restrict__ Zc,
                                                          c2<T>* __restrict__ out, int64_t ldo,
@@ -116,9 +118,9 @@ __global__ void __launch_bounds__(kThreads) k_band_z_fwd(Sphere s, const c2<T>* 
     __syncthreads();
     tile_fft<V, N, -1, TL, LS, kThreads>(buf, tws);
     const int cls = b < n_closed ? 0 : b - n_closed + 1;
-    const T w = KIN ? wk[cls] : T(0);
+    const T w = MODE == ZK_KIN ? wk[cls] : T(0);
     V* o = out + (int64_t)b * ldo;
-    const V* p = KIN ? psi + (int64_t)b * ldp : nullptr;
+    const V* p = MODE == ZK_KIN ? psi + (int64_t)b * ldp : nullptr;
 #pragma unroll
     for (int r = 0; r < (TL * N + kThreads - 1) / kThreads; ++r) {
         const int idx = threadIdx.x + r * kThreads;
@@ -129,10 +131,12 @@ __global__ void __launch_bounds__(kThreads) k_band_z_fwd(Sphere s, const c2<T>* 
             if (k >= -km && k <= km) {
                 const int g = cstart[line] + k + km;
                 const V loc = buf[e * LS + line];
-                if constexpr (KIN) {
+                if constexpr (MODE == ZK_KIN) {
                     const V ps = p[g];
                     const T kin = w * g2half[g];
                     o[g] = mk<T>(loc.x + kin * ps.x, loc.y + kin * ps.y);
+                } else if constexpr (MODE == ZK_ADD) {
+                    o[g] = cadd(o[g], loc);
                 } else {
                     o[g] = loc;
                 }
@@ -247,7 +251,8 @@ __global__ void __launch_bounds__(x_threads(N)) k_band_x_apply(Sphere s, const c
     const int nmax = s.nmax;
     constexpr int NN = N * N;
     // inverse x transform; the last pass forms (V psi + X) * scale in the tile,
-    // X being the exchange field of the band (absent without exact exchange)
+    // X being the exchange field of the band (absent without exact exchange,
+    // and where that has a grid of its own)
     fft_io<V, N, +1, TL, LS, NT, false, true, PRUNE ? sphere_zero_mask(N) : 0u>(
         buf, tws,
         [&](int line, int e) {
@@ -576,14 +581,19 @@ struct BandFft {
                       const T* g2half, const T* wk, int b0, int nbb, int nc, cudaStream_t st) {
         dim3 gz((s.ncol + TLZ - 1) / TLZ, nbb);
         if (psi) {
-            set_smem(k_band_z_fwd<T, N, true>, SMZ);
-            roks::count_launch(), k_band_z_fwd<T, N, true><<<gz, kThreads, SMZ, st>>>(s, tw, Zc, out, ldo, psi, ldp,
-                                                                                      g2half, wk, b0, nc);
+            set_smem(k_band_z_fwd<T, N, ZK_KIN>, SMZ);
+            roks::count_launch(), k_band_z_fwd<T, N, ZK_KIN><<<gz, kThreads, SMZ, st>>>(s, tw, Zc, out, ldo, psi, ldp,
+                                                                                        g2half, wk, b0, nc);
         } else {
-            set_smem(k_band_z_fwd<T, N, false>, SMZ);
-            roks::count_launch(), k_band_z_fwd<T, N, false><<<gz, kThreads, SMZ, st>>>(s, tw, Zc, out, ldo, psi,
-                                                                                       ldp, g2half, wk, b0, nc);
+            set_smem(k_band_z_fwd<T, N, ZK_PLAIN>, SMZ);
+            roks::count_launch(), k_band_z_fwd<T, N, ZK_PLAIN><<<gz, kThreads, SMZ, st>>>(s, tw, Zc, out, ldo, psi,
+                                                                                          ldp, g2half, wk, b0, nc);
         }
+    }
+    static void z_fwd_add(const Sphere& s, const V* tw, const V* Zc, V* out, int64_t ldo, int nbb, cudaStream_t st) {
+        set_smem(k_band_z_fwd<T, N, ZK_ADD>, SMZ);
+        roks::count_launch(), k_band_z_fwd<T, N, ZK_ADD><<<dim3((s.ncol + TLZ - 1) / TLZ, nbb), kThreads, SMZ, st>>>(
+                                  s, tw, Zc, out, ldo, nullptr, 0, nullptr, nullptr, 0, nbb);
     }
     // slot null: the bands are open-shell ones (or cls_override >= 0) and go
     // straight to rho3, no group slots are written and none are reduced
@@ -655,11 +665,6 @@ void band_x_apply(const Sphere& s, const c2<T>* tw, c2<T>* Yp, const T* Vk, cons
     ROKS_GRID_DISPATCH(s.N, (BandFft<T, NN>::x_apply(s, tw, Yp, Vk, Xx, b0, nbb, n_closed, split_band, scale, st)));
 }
 template <typename T>
-void band_x_inv_full(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, c2<T>* Phi, int b0, int nbb, T scale,
-                     cudaStream_t st) {
-    ROKS_GRID_DISPATCH(s.N, (BandFft<T, NN>::x_inv_full(s, tw, Yp, Phi, b0, nbb, scale, st)));
-}
-template <typename T>
 void band_y_fwd(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, c2<T>* Zc, int nbb, cudaStream_t st) {
     ROKS_GRID_DISPATCH(s.N, (BandFft<T, NN>::y_fwd(s, tw, Yp, Zc, nbb, st)));
 }
@@ -696,7 +701,6 @@ void grid_fft3_batched(int N, const c2<T>* tw, c2<T>* data, int batch, int64_t b
     template void band_y_inv<T>(const Sphere&, const c2<T>*, const c2<T>*, c2<T>*, int, cudaStream_t);          \
     template void band_x_apply<T>(const Sphere&, const c2<T>*, c2<T>*, const T*, const c2<T>*, int, int, int, int, \
                                   T, cudaStream_t);                                                              \
-    template void band_x_inv_full<T>(const Sphere&, const c2<T>*, const c2<T>*, c2<T>*, int, int, T, cudaStream_t); \
     template void grid_fft3_batched<T>(int, const c2<T>*, c2<T>*, int, int64_t, int, cudaStream_t);             \
     template void band_y_fwd<T>(const Sphere&, const c2<T>*, const c2<T>*, c2<T>*, int, cudaStream_t);          \
     template void band_z_fwd<T>(const Sphere&, const c2<T>*, const c2<T>*, c2<T>*, int64_t, const c2<T>*,        \

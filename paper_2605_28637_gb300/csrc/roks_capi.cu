@@ -112,10 +112,12 @@ struct roks_ctx {
     int* h_flag = nullptr;
     PcgScalars* d_sc = nullptr;
     // exact exchange (alpha != 0)
-    void *d_Phi = nullptr, *d_Xx = nullptr, *d_exbuf = nullptr, *d_vG = nullptr;
+    void *d_Phi = nullptr, *d_Xx = nullptr, *d_exbuf = nullptr, *d_vG = nullptr, *d_Ypx = nullptr, *d_twx = nullptr;
     int *d_pj = nullptr, *d_pn = nullptr;
     double *d_expart = nullptr, *d_Kmat = nullptr, *d_hf2 = nullptr, *d_exopen = nullptr;
-    int npairs = 0, exx_batch = 0;
+    int npairs = 0, exx_M = 0, exx_batch = 0;   // exchange grid, pairs in d_exbuf
+    std::vector<ExxTile> exx_tiles_h;
+    ExxTile* d_tiles = nullptr;
     ExxCoef exc{};
     // state: the density/potentials and d_B = P^H psi belong to the buffer
     // (address and leading dimension) a step or force call last used
@@ -261,6 +263,13 @@ Sphere sphere(const roks_ctx* c) {
     return s;
 }
 
+// the sphere on the exchange's grid
+Sphere exx_sphere(const roks_ctx* c) {
+    Sphere s = sphere(c);
+    s.N = c->exx_M;
+    return s;
+}
+
 bool grid_supported(int n) {
     for (int g : kGrids)
         if (g == n) return true;
@@ -365,20 +374,26 @@ struct Impl {
         band_x_apply<T>(s, ccv(ctx->d_tw), Yp, Vk, Xx, b0, nbb, n_closed, split_band, scale, ctx->st);
     }
 
-    // Exact exchange of the bands whose plane data sit in Yp: real-space
-    // orbitals, pair integrals, energies and (want_field) the exchange fields.
-    static void exchange(roks_ctx* ctx, bool want_field) {
-        const Sphere s = sphere(ctx);
+    // Exact exchange of psi (its planes are in Yp): real-space orbitals, pair
+    // integrals, energies and (want_field) the exchange fields.  On a grid of
+    // its own the orbitals are transformed anew; Zc serves as work space there:
+    // nothing reads it between two transforms.
+    static void exchange(roks_ctx* ctx, const V* psi, int64_t ld, bool want_field) {
         cudaStream_t st = ctx->st;
-        band_x_inv_full<T>(s, ccv(ctx->d_tw), cv(ctx->d_Yp), cv(ctx->d_Phi), 0, ctx->nb, T(1.0 / std::sqrt(ctx->omega)),
-                           st);
+        const bool own = ctx->exx_M != ctx->N;
+        const V* tw = ccv(own ? ctx->d_twx : ctx->d_tw);
+        exx_orbitals<T>(exx_sphere(ctx), tw, own ? psi : nullptr, ld, ctx->nb, cv(ctx->d_Zc),
+                        cv(own ? ctx->d_Ypx : ctx->d_Yp), cv(ctx->d_Phi), T(1.0 / std::sqrt(ctx->omega)), st);
         ExxArgs<T> a;
-        a.N = ctx->N;
+        a.M = ctx->exx_M;
         a.nb = ctx->nb;
         a.npairs = ctx->npairs;
         a.batch = ctx->exx_batch;
+        a.ntiles = (int)ctx->exx_tiles_h.size();
+        a.tiles = ctx->exx_tiles_h.data();
+        a.d_tiles = ctx->d_tiles;
         a.L = ctx->L;
-        a.tw = ccv(ctx->d_tw);
+        a.tw = tw;
         a.vG = static_cast<const T*>(ctx->d_vG);
         a.Phi = ccv(ctx->d_Phi);
         a.X = cv(ctx->d_Xx);
@@ -401,7 +416,7 @@ struct Impl {
         inv_planes(ctx, psi, ld);
         if (ctx->alpha != 0.0) {
             PROF("exchange");
-            exchange(ctx, false);
+            exchange(ctx, p, ld, false);
         }
         CK(cudaMemsetAsync(ctx->d_rho3, 0, sizeof(double) * 3 * (size_t)ctx->N * ctx->N * ctx->N, st));
         {
@@ -486,12 +501,12 @@ struct Impl {
         if (!planes_ready) planes(ctx, psi, ld);
         if (ctx->alpha != 0.0) {
             PROF("exchange");
-            exchange(ctx, true);
+            exchange(ctx, p, ld, true);
         }
         {
             PROF("fft_x_apply");
             const int nx = ctx->nbt - ctx->ne;
-            x_apply(ctx, cv(ctx->d_Yp), ctx->alpha != 0.0 ? ccv(ctx->d_Xx) : nullptr, 0, nx, ctx->nct, ctx->split_t);
+            x_apply(ctx, cv(ctx->d_Yp), ctx->alpha != 0.0 && ctx->exx_M == N ? ccv(ctx->d_Xx) : nullptr, 0, nx, ctx->nct, ctx->split_t);
             // empty bands: F^c (a closed count past the last band gives class 0)
             if (ctx->ne > 0)
                 x_apply(ctx, cv(ctx->d_Yp) + (int64_t)nx * ctx->np * N * N, nullptr, nx, ctx->ne, ctx->nb, -1);
@@ -518,6 +533,12 @@ struct Impl {
                                   p, ld, static_cast<const T*>(ctx->d_g2half), static_cast<const T*>(ctx->d_wk),
                                   ctx->nocc, ctx->ne, ctx->nb, st);
             }
+        }
+        if (ctx->alpha != 0.0 && ctx->exx_M != N) {
+            PROF("exchange");
+            const double M3 = double(ctx->exx_M) * ctx->exx_M * ctx->exx_M;
+            exx_add_fields<T>(exx_sphere(ctx), ccv(ctx->d_twx), ccv(ctx->d_Xx), ctx->nb, cv(ctx->d_Ypx),
+                              cv(ctx->d_Zc), cv(F), ldf, T(1.0 / M3), st);
         }
         if (ctx->nproj > 0) {
             if (!reuse_B) {
@@ -1476,25 +1497,36 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
     AL(ctx->d_sc, sizeof(PcgScalars));
     std::vector<int> pj, pn;
     if (opt->alpha != 0.0) {
-        for (int n2 = 0; n2 < nb; ++n2)
-            for (int j2 = 0; j2 <= n2; ++j2) {
-                pj.push_back(j2);
-                pn.push_back(n2);
-            }
-        ctx->npairs = (int)pj.size();
-        const size_t grid_bytes = cs * N3;
-        int batch = (int)((256u << 20) / grid_bytes);
-        if (batch < 1) batch = 1;
-        if (batch > 64) batch = 64;
-        if (batch > ctx->npairs) batch = ctx->npairs;
-        ctx->exx_batch = batch;
-        AL(ctx->d_Phi, cs * N3 * nb);
-        AL(ctx->d_Xx, cs * N3 * nb);
-        AL(ctx->d_exbuf, cs * N3 * batch);
-        AL(ctx->d_vG, rs * N3);
+        // Tiles of 8 x 8 bands, or smaller ones that fit 256 MB (tiles of 7 at
+        // hybrid-72: 19.6 ms an apply instead of 18.8, of 6: 20.9, though their
+        // grids leave the L2 more room: more, smaller launches), as many to a
+        // batch as fit 96 MB.
+        const int M = ctx->exx_M = exx_grid(N, n, nb);
+        const size_t M3 = (size_t)M * M * M;
+        int tile = kExxTileMax;
+        while (tile > 2 && cs * M3 * tile * tile > (256u << 20)) tile /= 2;
+        ctx->npairs = exx_tiles(nb, tile, ctx->exx_tiles_h);
+        for (const ExxTile& t : ctx->exx_tiles_h) {
+            for (int n2 = t.n0; n2 < t.n0 + t.bn; ++n2)
+                for (int j2 = t.j0; j2 < t.j0 + t.bj && j2 <= n2; ++j2) {
+                    pj.push_back(j2);
+                    pn.push_back(n2);
+                }
+            ctx->exx_batch = std::max(ctx->exx_batch, t.np);
+        }
+        ctx->exx_batch = (int)std::min<size_t>(ctx->npairs, std::max<size_t>(ctx->exx_batch, (96u << 20) / (cs * M3)));
+        AL(ctx->d_tiles, sizeof(ExxTile) * ctx->exx_tiles_h.size());
+        AL(ctx->d_Phi, cs * M3 * nb);
+        AL(ctx->d_Xx, cs * M3 * nb);
+        if (M != N) {
+            AL(ctx->d_Ypx, cs * (size_t)nb * ctx->np * M * M);
+            AL(ctx->d_twx, cs * M);
+        }
+        AL(ctx->d_exbuf, cs * M3 * ctx->exx_batch);
+        AL(ctx->d_vG, rs * M3);
         AL(ctx->d_pj, sizeof(int) * ctx->npairs);
         AL(ctx->d_pn, sizeof(int) * ctx->npairs);
-        AL(ctx->d_expart, sizeof(double) * batch * kExxBlocks);
+        AL(ctx->d_expart, sizeof(double) * (size_t)ctx->npairs * M);
         AL(ctx->d_Kmat, sizeof(double) * nb * nb);
         AL(ctx->d_hf2, sizeof(double) * 2);
         AL(ctx->d_exopen, sizeof(double) * 2);
@@ -1555,6 +1587,8 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
     if (e == cudaSuccess) e = up(d_proj, proj.data(), sizeof(double) * proj.size());
     if (e == cudaSuccess && ctx->npairs > 0) e = up(ctx->d_pj, pj.data(), sizeof(int) * pj.size());
     if (e == cudaSuccess && ctx->npairs > 0) e = up(ctx->d_pn, pn.data(), sizeof(int) * pn.size());
+    if (e == cudaSuccess && ctx->npairs > 0)
+        e = up(ctx->d_tiles, ctx->exx_tiles_h.data(), sizeof(ExxTile) * ctx->exx_tiles_h.size());
     if (e != cudaSuccess) return bail(ROKS_ECUDA, "upload");
     // typed tables
     std::vector<double> wk(ctx->cf.w, ctx->cf.w + 3);
@@ -1606,8 +1640,20 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
         return bail(ROKS_ECUDA, "projector image");
     if (opt->alpha != 0.0) {
         const int bare = opt->exx_kernel == ROKS_EXX_BARE ? 1 : 0;
-        if (f64) exx_setup_kernel<double>(N, cell->L, bare, static_cast<double*>(ctx->d_vG), ctx->st);
-        else exx_setup_kernel<float>(N, cell->L, bare, static_cast<float*>(ctx->d_vG), ctx->st);
+        const int M = ctx->exx_M;
+        if (f64) exx_setup_kernel<double>(M, cell->L, bare, static_cast<double*>(ctx->d_vG), ctx->st);
+        else exx_setup_kernel<float>(M, cell->L, bare, static_cast<float*>(ctx->d_vG), ctx->st);
+        if (M != N) {
+            std::vector<double2> t64(M);
+            std::vector<float2> t32(M);
+            for (int t = 0; t < M; ++t) {
+                t64[t] = make_double2(std::cos(-2.0 * M_PI * t / M), std::sin(-2.0 * M_PI * t / M));
+                t32[t] = make_float2((float)t64[t].x, (float)t64[t].y);
+            }
+            cudaMemcpyAsync(ctx->d_twx, f64 ? (const void*)t64.data() : (const void*)t32.data(),
+                            (f64 ? sizeof(double2) : sizeof(float2)) * M, cudaMemcpyHostToDevice, ctx->st);
+            cudaStreamSynchronize(ctx->st);
+        }
     }
     e = cudaStreamSynchronize(ctx->st);
     if (e == cudaSuccess) e = cudaGetLastError();

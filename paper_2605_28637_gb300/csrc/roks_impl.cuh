@@ -68,10 +68,6 @@ void band_y_inv(const Sphere& s, const c2<T>* tw, const c2<T>* Zc, c2<T>* Yp, in
 template <typename T>
 void band_x_apply(const Sphere& s, const c2<T>* tw, c2<T>* Yp, const T* Vk, const c2<T>* Xx, int b0, int nbb,
                   int n_closed, int split_band, T scale, cudaStream_t st);
-// x stage, inverse, full real-space lines: Phi[b0 + b] = scale * psi~ (N^3 each)
-template <typename T>
-void band_x_inv_full(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, c2<T>* Phi, int b0, int nbb, T scale,
-                     cudaStream_t st);
 // y stage, forward: Yp -> Zc (columns of the sphere only)
 template <typename T>
 void band_y_fwd(const Sphere& s, const c2<T>* tw, const c2<T>* Yp, c2<T>* Zc, int nbb, cudaStream_t st);
