@@ -10,6 +10,7 @@
 
 #include <cooperative_groups.h>
 
+#include "roks_chol.cuh"
 #include "roks_impl.cuh"
 
 namespace roks {
@@ -127,19 +128,23 @@ __global__ void __launch_bounds__(256) k_gemm_cn(int M, int N, int K, int kchunk
         __syncthreads();
         const V* as = As + (t & 1) * KT * SA + ty * padgroup<RM>();
         const V* bs = Bs + (t & 1) * KT * SB + tx * padgroup<RN>();
-#pragma unroll 8
-        for (int kk = 0; kk < KT; ++kk) {
-            V a[RM], b[RN];
+        // (FP64: a chunk of half a slice does not multiply the other half's zeros)
+        const int kc = sizeof(T) == 8 ? min(KT, kend - kbeg - t * KT) : KT;
+        for (int k8 = 0; k8 < kc; k8 += 8) {
 #pragma unroll
-            for (int i = 0; i < RM; ++i) a[i] = as[i];
+            for (int kk = 0; kk < 8; ++kk) {
+                V a[RM], b[RN];
 #pragma unroll
-            for (int j = 0; j < RN; ++j) b[j] = bs[j];
-            as += SA;
-            bs += SB;
+                for (int i = 0; i < RM; ++i) a[i] = as[i];
 #pragma unroll
-            for (int i = 0; i < RM; ++i)
+                for (int j = 0; j < RN; ++j) b[j] = bs[j];
+                as += SA;
+                bs += SB;
 #pragma unroll
-                for (int j = 0; j < RN; ++j) mac_cn<T>(acc[i][j], a[i], b[j]);
+                for (int i = 0; i < RM; ++i)
+#pragma unroll
+                    for (int j = 0; j < RN; ++j) mac_cn<T>(acc[i][j], a[i], b[j]);
+            }
         }
         __syncthreads();
     }
@@ -349,7 +354,11 @@ int cn_resident_blocks(int rm, int rn, int threads, size_t smem) {
 
 // Register tile and thread grid with the least padded work (plus the
 // shared-memory loads per multiply-add), then K chunks for whole waves of
-// resident blocks, each at least two K slices long.
+// resident blocks, each at least two K slices long.  FP64 products are bound
+// by the pipe of the SMs that take part (two multiply-adds a cycle each), so
+// their chunks go down to half a slice, up to as many as there are SMs: 44 x 6
+// over 1050 rows, 33 chunks of 32 46.7 us, 131 of 8 15.8 us.  (With more, the
+// sum of the partials takes what is gained: 5 us at 20 x 20 over 4000.)
 template <typename T>
 CnPlan cn_plan(int M, int N, int K, int max_chunks) {
     constexpr int KT = CnTile<T>::KT;
@@ -377,13 +386,15 @@ CnPlan cn_plan(int M, int N, int K, int max_chunks) {
     size_t smem = 0;
     cn_layout<T>(best, SA, SB, smem);
     int want = (cn_resident_blocks<T>(best.rm, best.rn, best.ty * best.tx, smem) * sm_count() + tiles - 1) / tiles;
-    const int by_len = (K + 2 * KT - 1) / (2 * KT);
+    const int least = sizeof(T) == 8 ? KT / 2 : 2 * KT;
+    int by_len = (K + 2 * KT - 1) / (2 * KT);
+    if (sizeof(T) == 8) by_len = std::max(by_len, std::min((K + least - 1) / least, sm_count()));
     if (want > by_len) want = by_len;
     if (max_chunks > 0 && want > max_chunks) want = max_chunks;
     if (want < 1) want = 1;
     int kc = (K + want - 1) / want;
-    kc = ((kc + KT - 1) / KT) * KT;
-    if (kc < KT) kc = KT;
+    const int step = kc < KT && least < KT ? least : KT;
+    kc = std::max(step, (kc + step - 1) / step * step);
     best.kchunk = kc;
     best.nchunk = K > 0 ? (K + kc - 1) / kc : 1;
     return best;
@@ -570,10 +581,9 @@ __global__ void k_b_to_f32(int K, int N, const double2* __restrict__ B, int ldb,
 }
 
 namespace {
-template <typename T, int RN>
+template <typename T, int RN, int RM>
 void launch_nn(int M, int N, int K, int ty, int nt, const c2<T>* A, int64_t lda, const c2<T>* B, int ldb, c2<T>* C,
                int64_t ldc, T alpha, T beta, cudaStream_t st) {
-    constexpr int RM = 4;
     const size_t smem = sizeof(c2<T>) * (2 * NN_KT * (32 * RM + 8 * RN + 1) + (size_t)(8 * RN) * (32 * RM));
     static bool attr = false;
     if (!attr) {
@@ -597,9 +607,18 @@ void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B,
                         ldc, (float)alpha, (float)beta, bwork, bwork_bytes, ia, st))
             return;
     }
-    // column tiles of at most 64: RN = ceil(tile / 8) columns per thread, TY <= 8 warps
-    const int nt = (N + 63) / 64;
+    // Column tiles of at most 64: RN = ceil(tile / 8) columns per thread, TY <= 8
+    // warps.  Where tiles of 128 rows leave SMs idle the rows go down to 32 and
+    // the columns are split, as long as SMs are free (FP64 runs at the pipe of
+    // the SMs that take part: 1050 x 6 x 44 on 9 blocks 16.8 us, on 198 6.6;
+    // 4000 x 48 x 200 785 and 202).  Short FP32 sums are bound by latency either
+    // way and keep the fewer blocks (a DIIS step of 12 bands 430 us, 435 split;
+    // a PCG step of 53 bands, 150 projectors: 1070 us, 916 split).
+    int nt = (N + 63) / 64;
+    const bool low = (sizeof(T) == 8 || K >= 48) && (int64_t)((M + 127) / 128) * nt < sm_count();
+    while (low && nt < N && (int64_t)((M + 31) / 32) * nt < sm_count()) nt = std::min(N, 2 * nt);
     const int tn = (N + nt - 1) / nt;
+    nt = (N + tn - 1) / tn;
     const int rn = (tn + 7) / 8;
     const int ty = (tn + rn - 1) / rn;
     const c2<T>* Bt;
@@ -620,8 +639,9 @@ void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B,
         Bt = B;
         ldbt = ldb;
     }
-#define NN_CASE(RN_) \
-    if (rn == RN_) launch_nn<T, RN_>(M, N, K, ty, nt, A, lda, Bt, ldbt, C, ldc, T(alpha), T(beta), st);
+#define NN_CASE(RN_)                                                                                             \
+    if (rn == RN_ && low) launch_nn<T, RN_, 1>(M, N, K, ty, nt, A, lda, Bt, ldbt, C, ldc, T(alpha), T(beta), st); \
+    if (rn == RN_ && !low) launch_nn<T, RN_, 4>(M, N, K, ty, nt, A, lda, Bt, ldbt, C, ldc, T(alpha), T(beta), st);
     NN_CASE(1) NN_CASE(2) NN_CASE(3) NN_CASE(4) NN_CASE(5) NN_CASE(6) NN_CASE(7) NN_CASE(8)
 #undef NN_CASE
 }
@@ -885,83 +905,26 @@ void small_gemm_f32(int M, int N, int K, const double2* A, int lda, bool ca, con
                               M, N, K, A, lda, ca, B, ldb, cb, C, ldc, alpha, beta);
 }
 
-// Cholesky inverse held in shared memory (n <= kSmallN), FP64: right-looking
-// factorisation O = L L^H (two barriers per column), then X = L^{-1} by
-// forward substitution with one warp per column (lanes split the dot
-// products); LinvH = X^H.
+// Cholesky inverse held in shared memory (n <= kSmallN), FP64
+// (chol_inverse_block): 6 bands 15.7 -> 10.8 us, 20 bands 75 -> 37, 42 bands
+// 269 -> 103.
 constexpr int kSmallN = 64;
 
-__global__ void __launch_bounds__(1024) k_cholesky_small(int n, const double2* __restrict__ O,
-                                                         double2* __restrict__ LinvH, int* flag) {
+template <int NT>
+__global__ void __launch_bounds__(NT) k_cholesky_small(int n, const double2* __restrict__ O,
+                                                       double2* __restrict__ LinvH, int* flag) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* L = reinterpret_cast<double2*>(smem_raw);          // n x n, column major
     double2* X = L + n * n;                                      // n x n, column major
-    __shared__ int bad;
-    __shared__ double dinv[kSmallN];                             // 1 / L_jj
-    if (threadIdx.x == 0) bad = 0;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    __shared__ double dinv[kSmallN];
+    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
         L[idx] = O[idx];
         X[idx] = make_double2(0.0, 0.0);
     }
     __syncthreads();
-    // FP64 throughput is a per-SM resource: the pivot square root and
-    // reciprocal are computed once, by one thread, not by every thread.
-    for (int j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            double d = L[j * n + j].x;
-            if (!(d > 0.0)) {
-                if (!bad) bad = j + 1;
-                d = 1.0;
-            }
-            const double piv = sqrt(d);
-            L[j * n + j] = make_double2(piv, 0.0);
-            dinv[j] = 1.0 / piv;
-        }
-        __syncthreads();
-        const double inv = dinv[j];
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            const double2 v = L[j * n + i];
-            L[j * n + i] = make_double2(v.x * inv, v.y * inv);
-        }
-        __syncthreads();
-        // trailing update A_ik -= L_ij conj(L_kj), j < k <= i
-        const int m = n - j - 1;
-        for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-            const int k = t / m;
-            const int i = t - k * m;
-            if (k > i) continue;
-            const double2 a = L[j * n + j + 1 + i], b = L[j * n + j + 1 + k];
-            double2 c = L[(j + 1 + k) * n + j + 1 + i];
-            c.x -= a.x * b.x + a.y * b.y;
-            c.y -= a.y * b.x - a.x * b.y;
-            L[(j + 1 + k) * n + j + 1 + i] = c;
-        }
-        __syncthreads();
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int c = warp; c < n; c += nw) {
-        for (int i = c; i < n; ++i) {
-            double sr = 0.0, si = 0.0;
-            for (int k = c + lane; k < i; k += 32) {
-                const double2 l = L[k * n + i], x = X[c * n + k];
-                sr += l.x * x.x - l.y * x.y;
-                si += l.x * x.y + l.y * x.x;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sr += __shfl_xor_sync(0xffffffffu, sr, o);
-                si += __shfl_xor_sync(0xffffffffu, si, o);
-            }
-            if (lane == 0) {
-                const double di = dinv[i];
-                X[c * n + i] = make_double2(((i == c) ? 1.0 - sr : -sr) * di, -si * di);
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
+    const int bad = chol_inverse_block<NT>(n, L, X, dinv);
     // LinvH (row c, column i) = conj X (row i, column c)
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < n * n; idx += NT) {
         const int c = idx % n, i = idx / n;
         const double2 x = X[c * n + i];
         LinvH[idx] = make_double2(x.x, -x.y);
@@ -1164,8 +1127,11 @@ __global__ void __launch_bounds__(1024) k_cholesky_inverse(int n, const double2*
 void cholesky_inverse(int n, const double2* O, double2* Lw, double2* LinvH, int* flag, cudaStream_t st) {
     if (n <= kSmallN) {
         const size_t sm = sizeof(double2) * 2 * n * n;
-        if (sm > 48 * 1024) cudaFuncSetAttribute(k_cholesky_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        roks::count_launch(), k_cholesky_small<<<1, 1024, sm, st>>>(n, O, LinvH, flag);
+        if (sm > 48 * 1024)
+            cudaFuncSetAttribute(k_cholesky_small<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        roks::count_launch();
+        if (n <= 16) k_cholesky_small<128><<<1, 128, sm, st>>>(n, O, LinvH, flag);
+        else k_cholesky_small<1024><<<1, 1024, sm, st>>>(n, O, LinvH, flag);
         return;
     }
     roks::count_launch(), k_cholesky_inverse<<<1, 1024, 0, st>>>(n, O, Lw, LinvH, flag);
@@ -1373,6 +1339,126 @@ __global__ void __cluster_dims__(kExpmCluster, 1, 1) __launch_bounds__(kExpmThre
     }
 }
 
+// The same in FP64 for n <= kExpmF64N, on CL blocks (one up to 12 x 12, whose
+// matrices are too small to spread): ||s A||_1 / 2^q <= 1/2, Taylor degree 16
+// from X .. X^4 in six products (Horner over X^4), q squarings.  Bound by the
+// chain of products and, from some 32 bands on, by the FP64 pipes of its eight
+// SMs; launches of their own for every product spread over more SMs and take
+// over beyond (times of the launches and here: 6 bands 116 and 15 us, 20 bands
+// 226 and 44, 42 bands 389 and 144, 48 bands 413 and 234).
+constexpr int kExpmF64N = 48;
+struct ExpmPoly {
+    double a[5];   // I, X, X^2, X^3, X^4
+};
+template <int CL>
+__device__ __forceinline__ void cluster_mm_f64(cg::cluster_group& cluster, int n, int c0, int c1, const double2* A,
+                                               const double2* B, const double2* X, const ExpmPoly& p, double2* C) {
+    const int nn = n * n;
+    for (int t = threadIdx.x; t < n * (c1 - c0); t += blockDim.x) {
+        const int c = c0 + t / n, m = t % n, e = c * n + m;
+        double2 v = make_double2(m == c ? p.a[0] : 0.0, 0.0);
+#pragma unroll
+        for (int k = 1; k < 5; ++k)
+            if (p.a[k] != 0.0) {
+                const double2 x = X[(k - 1) * nn + e];
+                v.x += p.a[k] * x.x;
+                v.y += p.a[k] * x.y;
+            }
+        if (A) {
+            double2 w = make_double2(0.0, 0.0);
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) {
+                const double2 a = A[k * n + m], b = B[c * n + k];
+                v.x = fma(a.x, b.x, v.x);
+                v.y = fma(a.x, b.y, v.y);
+                w.x = fma(-a.y, b.y, w.x);
+                w.y = fma(a.y, b.x, w.y);
+            }
+            v.x += w.x;
+            v.y += w.y;
+        }
+        if constexpr (CL == 1) {
+            C[e] = v;
+        } else {
+#pragma unroll
+            for (int r = 0; r < CL; ++r) cluster.map_shared_rank(C, r)[e] = v;
+        }
+    }
+    if constexpr (CL == 1) __syncthreads();
+    else cluster.sync();
+}
+
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kExpmThreads)
+    k_expm_small_f64(int n, const double2* __restrict__ A, const double* __restrict__ s, double2* __restrict__ E) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = CL == 1 ? 0 : (int)cluster.block_rank(), nn = n * n;
+    double2* X = reinterpret_cast<double2*>(smem_raw);   // X, X^2, X^3, X^4, T, U
+    double2 *P = X + 4 * nn, *Q = P + nn;
+    __shared__ double wmax[kExpmThreads / 32];
+    __shared__ int qs;
+    const int cp = (n + CL - 1) / CL, c0 = min(n, rank * cp), c1 = min(n, c0 + cp);
+    for (int idx = threadIdx.x; idx < nn; idx += blockDim.x) X[idx] = A[idx];
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    double best = 0.0;
+    for (int c = warp; c < n; c += nw) {
+        double sum = 0.0;
+        for (int r = lane; r < n; r += 32) {
+            const double2 a = X[c * n + r];
+            sum += sqrt(a.x * a.x + a.y * a.y);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        best = fmax(best, sum);
+    }
+    if (lane == 0) wmax[warp] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double m = 0.0;
+        for (int w = 0; w < nw; ++w) m = fmax(m, wmax[w]);
+        double scaled = fabs(s[0]) * m;
+        int q = 0;
+        while (scaled > 0.5 && q < kExpmMaxSquare) {
+            scaled *= 0.5;
+            ++q;
+        }
+        qs = q;
+    }
+    __syncthreads();
+    const int q = qs;
+    const double f = s[0] * ldexp(1.0, -q);
+    for (int idx = threadIdx.x; idx < nn; idx += blockDim.x) X[idx] = make_double2(f * X[idx].x, f * X[idx].y);
+    // the peers write into this block's matrices from here on
+    if constexpr (CL == 1) __syncthreads();
+    else cluster.sync();
+    double c[17];
+    c[0] = 1.0;
+#pragma unroll
+    for (int k = 1; k <= 16; ++k) c[k] = c[k - 1] / k;
+    const ExpmPoly none{{0.0, 0.0, 0.0, 0.0, 0.0}};
+    cluster_mm_f64<CL>(cluster, n, c0, c1, X, X, X, none, X + nn);
+    cluster_mm_f64<CL>(cluster, n, c0, c1, X + nn, X, X, none, X + 2 * nn);
+    cluster_mm_f64<CL>(cluster, n, c0, c1, X + nn, X + nn, X, none, X + 3 * nn);
+    cluster_mm_f64<CL>(cluster, n, c0, c1, nullptr, nullptr, X, ExpmPoly{{c[12], c[13], c[14], c[15], c[16]}}, P);
+#pragma unroll
+    for (int k = 2; k >= 0; --k) {
+        cluster_mm_f64<CL>(cluster, n, c0, c1, X + 3 * nn, P, X,
+                           ExpmPoly{{c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3], 0.0}}, Q);
+        double2* t = P;
+        P = Q;
+        Q = t;
+    }
+    for (int r = 0; r < q; ++r) {
+        cluster_mm_f64<CL>(cluster, n, c0, c1, P, P, X, none, Q);
+        double2* t = P;
+        P = Q;
+        Q = t;
+    }
+    for (int idx = c0 * n + threadIdx.x; idx < c1 * n; idx += blockDim.x) E[idx] = P[idx];
+}
+
 bool expm_small_f32(int n, const double2* A, const double* scale_dev, double2* E, cudaStream_t st) {
     if (n > kSmallN) return false;
     const int ldm = (n + 1) & ~1;
@@ -1389,6 +1475,19 @@ bool expm_small_f32(int n, const double2* A, const double* scale_dev, double2* E
 
 void expm_scaled(int n, const double2* A, const double* scale_dev, double2* E, double2* w1, double2* w2,
                  double2* w3, double* sdev, cudaStream_t st) {
+    if (n <= kExpmF64N) {
+        const size_t sm = sizeof(double2) * 6 * n * n;
+        static bool attr = false;
+        if (!attr) {
+            cudaFuncSetAttribute(k_expm_small_f64<kExpmCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(double2) * 6 * kExpmF64N * kExpmF64N));
+            attr = true;
+        }
+        roks::count_launch();
+        if (n <= 12) k_expm_small_f64<1><<<1, kExpmThreads, sm, st>>>(n, A, scale_dev, E);
+        else k_expm_small_f64<kExpmCluster><<<kExpmCluster, kExpmThreads, sm, st>>>(n, A, scale_dev, E);
+        return;
+    }
     roks::count_launch(), k_expm_scale<<<1, 256, 0, st>>>(n, A, scale_dev, w1, sdev);
     const int blocks = (n * n + 127) / 128;
     // Horner: E_deg = I + X / deg, ..., E_1 = I + X E_2
