@@ -503,6 +503,130 @@ __global__ void __launch_bounds__(kThreads) k_grid_fft_strided(const c2<T>* __re
     else fft_io<V, N, -1, TL, LS, kThreads, false, false>(buf, tws, ld, st);
 }
 
+// 4 pi / G^2 of one coefficient (m2 = |G|^2 in units of b^2; inv = 1 / N^3, fpb
+// = 4 pi / b^2) and its share of the Hartree energy
+template <typename T>
+__device__ __forceinline__ c2<T> hartree_point(c2<T> g, int m2, T inv, T fpb, T& eh) {
+    if (m2 == 0) return mk<T>(T(0), T(0));
+    const T rx = g.x * inv, ry = g.y * inv, k = fpb / T(m2);
+    eh += k * (rx * rx + ry * ry);
+    return mk<T>(k * rx, k * ry);
+}
+
+// Threads of the plane pass: whole rounds of the butterflies of its passes
+__host__ __device__ constexpr int plane_threads(int n) {
+    return n == 16 ? 64 : n == 24 || n == 48 ? 192 : n == 72 ? 352 : n == 96 ? 384 : n == 120 ? 480 : 256;
+}
+
+// The y and z transforms of plane x = blockIdx.x of grid blockIdx.y in one stay
+// in shared memory (rows M + 1 apart, so that lines along either axis meet no
+// bank twice).  MODE -1, +1: that direction.  MODE 0: forward, 4 pi / G^2 (with
+// the block's partial of the Hartree energy in part[x]; vmax, when given, is
+// cleared for the pass that follows), inverse; the z transforms join in
+// registers, since the last pass of a plan R0 x R1 leaves a thread the elements
+// j + r R0 in place, which the first pass of the plan R1 x R0 reads.  Against y
+// and z passes of their own: organic-96 (FP32) 17 -> 10 us a grid, with the
+// Hartree kernel 43 -> 13.
+template <typename T, int N, int MODE>
+__global__ void __launch_bounds__(plane_threads(N)) k_grid_plane(const c2<T>* __restrict__ tw, c2<T>* data,
+                                                                 int64_t bstride, T inv, T fpb,
+                                                                 double* __restrict__ part, float* vmax) {
+    using V = c2<T>;
+    constexpr int NT = plane_threads(N), PZ = N + 1, R0 = plan_radix(N, 0), R1 = plan_radix(N, 1);
+    static_assert(plan_passes(N) == 2 && R0 * R1 == N, "the plane pass takes two-pass plans");
+    extern __shared__ __align__(16) unsigned char smem[];
+    V* pl = reinterpret_cast<V*>(smem);
+    V* tws = pl + N * PZ;
+    load_twiddles<V, N>(tws, tw);
+    const int x = blockIdx.x, tid = threadIdx.x;
+    V* d = data + (int64_t)blockIdx.y * bstride + (int64_t)x * N * N;
+    auto yl = [&](int line, int e) { return pl[e * PZ + line]; };
+    auto ys = [&](int line, int e, V v, int, int) { pl[e * PZ + line] = v; };
+    auto zl = [&](int line, int e) { return pl[line * PZ + e]; };
+    auto zs = [&](int line, int e, V v, int, int) { pl[line * PZ + e] = v; };
+    constexpr int DIR = MODE == 0 ? -1 : MODE;
+    pass_io<V, N, 0, DIR, N, NT, false>(tws, [&](int line, int e) { return d[e * N + line]; }, ys);
+    __syncthreads();
+    pass_io<V, N, 1, DIR, N, NT, false>(tws, yl, ys);   // in place, element by element
+    __syncthreads();
+    pass_io<V, N, 0, DIR, N, NT, true>(tws, zl, zs);
+    __syncthreads();
+    if constexpr (MODE != 0) {
+        pass_io<V, N, 1, DIR, N, NT, false>(tws, zl, zs);
+        __syncthreads();
+        for (int idx = tid; idx < N * N; idx += NT) {
+            const int y = idx / N;
+            d[idx] = pl[y * PZ + idx - y * N];
+        }
+    } else {
+        T eh = T(0);
+        {
+            constexpr int TOT = R0 * N, PER = (TOT + NT - 1) / NT;
+            const int fx = signed_freq(x, N), mx = fx * fx;
+            V v[PER][R1];
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int beta = tid + q * NT;
+                if (beta < TOT) {
+                    const int line = beta % N, j = beta / N, fy = signed_freq(line, N), mxy = mx + fy * fy;
+#pragma unroll
+                    for (int r = 0; r < R1; ++r) v[q][r] = pl[line * PZ + j + r * R0];
+                    twiddle_dft<V, N, R1, R0, -1>(v[q], tws, j);
+#pragma unroll
+                    for (int r = 0; r < R1; ++r) {
+                        const int fz = signed_freq(j + r * R0, N);
+                        v[q][r] = hartree_point<T>(v[q][r], mxy + fz * fz, inv, fpb, eh);
+                    }
+                    twiddle_dft<V, N, R1, 1, +1>(v[q], tws, j);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int beta = tid + q * NT;
+                if (beta < TOT) {
+                    const int line = beta % N, j = beta / N;
+#pragma unroll
+                    for (int r = 0; r < R1; ++r) pl[line * PZ + j * R1 + r] = v[q][r];
+                }
+            }
+        }
+        __syncthreads();
+        {
+            constexpr int TOT = R1 * N, PER = (TOT + NT - 1) / NT;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int beta = tid + q * NT;
+                if (beta < TOT) {
+                    const int line = beta % N, j = beta / N;
+                    V v[R0];
+#pragma unroll
+                    for (int r = 0; r < R0; ++r) v[r] = pl[line * PZ + j + r * R1];
+                    twiddle_dft<V, N, R0, R1, +1>(v, tws, j);
+#pragma unroll
+                    for (int r = 0; r < R0; ++r) pl[line * PZ + j + r * R1] = v[r];
+                }
+            }
+        }
+        __syncthreads();
+        pass_io<V, N, 0, +1, N, NT, true>(tws, yl, ys);
+        __syncthreads();
+        pass_io<V, N, 1, +1, N, NT, false>(tws, yl, [&](int line, int e, V v, int, int) { d[e * N + line] = v; });
+        __shared__ double red[NT / 32];
+        double s = double(eh);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((tid & 31) == 0) red[tid >> 5] = s;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int k = 0; k < NT / 32; ++k) t += red[k];
+            part[x] = t;
+        }
+        if (vmax && x == 0 && tid < 3) vmax[tid] = 0.f;
+    }
+}
+
 // ------------------------------------------------------------------ launchers
 template <typename K>
 static void set_smem(K kernel, size_t bytes) {
@@ -625,16 +749,36 @@ struct BandFft {
         const int N3 = N * N * N;
         roks::count_launch(), k_density_reduce<T><<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, ng, sl, r3);
     }
-    static void grid3(const V* tw, V* data, int dir, int batch, int64_t bstride, cudaStream_t st) {
-        set_smem(k_grid_fft_z<T, N>, SM);
+    // The plane pass: every FP32 grid (116 KB at N = 120).  FP64 is bound by the
+    // pipes, and N planes occupy N of them: at 96 109 us a grid, 83 in two
+    // passes over all SMs; up to 32 the launch saved is worth more.
+    static constexpr size_t SMP = sizeof(V) * (size_t)(N * (N + 1) + N);
+    static constexpr bool PLANE = sizeof(T) == 4 || N <= 32;
+    static void grid_x(const V* tw, V* data, int dir, int batch, int64_t bstride, cudaStream_t st) {
         set_smem(k_grid_fft_strided<T, N>, SM);
-        dim3 gz((N * N + TL - 1) / TL, batch);
-        roks::count_launch(), k_grid_fft_z<T, N><<<gz, kThreads, SM, st>>>(tw, data, dir, bstride);
-        dim3 g((N + TL - 1) / TL, N, batch);
-        roks::count_launch(), k_grid_fft_strided<T, N><<<g, kThreads, SM, st>>>(tw, data, (int64_t)N * N, (int64_t)N,
-                                                                               dir, bstride);
-        roks::count_launch(), k_grid_fft_strided<T, N><<<g, kThreads, SM, st>>>(tw, data, (int64_t)N, (int64_t)N * N,
-                                                                               dir, bstride);
+        roks::count_launch(), k_grid_fft_strided<T, N><<<dim3((N + TL - 1) / TL, N, batch), kThreads, SM, st>>>(
+                                  tw, data, (int64_t)N, (int64_t)N * N, dir, bstride);
+    }
+    static void grid_yz(const V* tw, V* data, int dir, int batch, int64_t bstride, cudaStream_t st) {
+        if constexpr (PLANE) {
+            auto go = [&](auto kernel) {
+                set_smem(kernel, SMP);
+                roks::count_launch(), kernel<<<dim3(N, batch), plane_threads(N), SMP, st>>>(tw, data, bstride, T(0),
+                                                                                            T(0), nullptr, nullptr);
+            };
+            dir > 0 ? go(k_grid_plane<T, N, 1>) : go(k_grid_plane<T, N, -1>);
+        } else {
+            set_smem(k_grid_fft_z<T, N>, SM);
+            set_smem(k_grid_fft_strided<T, N>, SM);
+            roks::count_launch(), k_grid_fft_z<T, N><<<dim3((N * N + TL - 1) / TL, batch), kThreads, SM, st>>>(
+                                      tw, data, dir, bstride);
+            roks::count_launch(), k_grid_fft_strided<T, N><<<dim3((N + TL - 1) / TL, N, batch), kThreads, SM, st>>>(
+                                      tw, data, (int64_t)N * N, (int64_t)N, dir, bstride);
+        }
+    }
+    static void grid3(const V* tw, V* data, int dir, int batch, int64_t bstride, cudaStream_t st) {
+        grid_yz(tw, data, dir, batch, bstride, st);
+        grid_x(tw, data, dir, batch, bstride, st);
     }
 };
 

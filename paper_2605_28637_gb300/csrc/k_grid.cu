@@ -331,56 +331,6 @@ __global__ void k_band_quadratic(int nproj, int nb, const double2* __restrict__ 
 
 // ------------------------------------------------------------------ potentials
 // Channel densities rho^{ch} = sum_k f[k][ch] rho_k; total rho = up M + down M.
-// xc3[k] = sum_ch C[k][ch] v^{ch},  v = -(1-alpha) (6 rho / pi)^{1/3};
-// partial sums of (1-alpha) Slater energies per configuration and of V_loc rho.
-template <typename T>
-__global__ void __launch_bounds__(RB) k_pot_xc(int N3, const typename DensAcc<T>::S* __restrict__ rho3,
-                                               const T* __restrict__ vloc, PotCoefT<T> cf, T c6, T cx,
-                                               c2<T>* __restrict__ rho_grid, T* __restrict__ xc3,
-                                               double* __restrict__ part) {
-    // pointwise arithmetic in the element type T (constants come from the
-    // host: FP64 arithmetic per thread is slow on this part); per-thread
-    // partial energies in T over a few points, block and grid sums in FP64
-    __shared__ double sh[RB];
-    T exM = 0, exT = 0, eloc = 0;
-    const T xs = cf.xscale;
-    for (int p = blockIdx.x * RB + threadIdx.x; p < N3; p += gridDim.x * RB) {
-        using DA = DensAcc<T>;
-        const T rk[3] = {T(DA::value(rho3[p])), T(DA::value(rho3[N3 + p])), T(DA::value(rho3[2 * N3 + p]))};
-        T v[4];
-        T rho_tot = 0;
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-            T r = 0;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) r += cf.f[k][ch] * rk[k];
-            r = r > T(0) ? r : T(0);
-            const T c = cbrt(r);
-            v[ch] = -xs * c6 * c;
-            const T e = -xs * cx * c * r;
-            if (ch < 2) { exM += e; rho_tot += r; } else exT += e;
-        }
-        eloc += vloc[p] * rho_tot;
-        rho_grid[p] = mk<T>(rho_tot, T(0));
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            T s = 0;
-#pragma unroll
-            for (int ch = 0; ch < 4; ++ch) s += cf.C[k][ch] * v[ch];
-            xc3[k * N3 + p] = s;
-        }
-    }
-    const double dexM = block_sum_t<T>(exM, sh);
-    const double dexT = block_sum_t<T>(exT, sh);
-    const double deloc = block_sum_t<T>(eloc, sh);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x * 4 + 0] = dexM;
-        part[blockIdx.x * 4 + 1] = dexT;
-        part[blockIdx.x * 4 + 2] = deloc;
-        part[blockIdx.x * 4 + 3] = 0.0;
-    }
-}
-
 // ------------------------------------------------------------------ PBE exchange
 // Channel densities (clamped at 0) packed in pairs, gg = (up M + i down M,
 // up T + i down T); the total density for the Hartree solve; V_loc rho.
@@ -540,97 +490,20 @@ __global__ void __launch_bounds__(RB) k_gga_combine(int N3, PotCoefT<T> cf, cons
     }
 }
 
-// After the forward transform: rho(G) = grid / N^3; E_H partial
-// sum 4 pi |rho(G)|^2 / G^2; grid <- V_H(G) = 4 pi rho(G) / G^2 (G = 0 -> 0).
-template <typename T>
-__global__ void __launch_bounds__(RB) k_hartree_G(int N, T inv, T fpb, c2<T>* __restrict__ grid,
-                                                  double* __restrict__ part) {
-    // inv = 1 / N^3, fpb = 4 pi / b^2 with b = 2 pi / L (from the host)
-    __shared__ double sh[RB];
-    const int N3 = N * N * N;
-    T eh = 0;
-    for (int p = blockIdx.x * RB + threadIdx.x; p < N3; p += gridDim.x * RB) {
-        const int z = p % N, y = (p / N) % N, x = p / (N * N);
-        const int fx = signed_freq(x, N), fy = signed_freq(y, N), fz = signed_freq(z, N);
-        const int m2 = fx * fx + fy * fy + fz * fz;
-        const c2<T> gv = grid[p];
-        const T rx = gv.x * inv, ry = gv.y * inv;
-        c2<T> o = mk<T>(T(0), T(0));
-        if (m2 > 0) {
-            const T k = fpb / T(m2);              // 4 pi / G^2
-            eh += k * (rx * rx + ry * ry);
-            o = mk<T>(k * rx, k * ry);
-        }
-        grid[p] = o;
-    }
-    const double deh = block_sum_t<T>(eh, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = deh;
-}
-
-// V^k = w_k (V_loc + V_H) + xc3[k]; partial sums <a|V^c|a>, <b|V^c|b> (rho_a,
-// rho_b); the largest |V^k| of each class in vmax, when given.
-template <typename T>
-__global__ void __launch_bounds__(RB) k_pot_class(int N3, const T* __restrict__ vloc,
-                                                  const c2<T>* __restrict__ vh, const T* __restrict__ xc3,
-                                                  const typename DensAcc<T>::S* __restrict__ rho3, PotCoef cf,
-                                                  T* __restrict__ Vk,
-                                                  double* __restrict__ Vk64, double* __restrict__ part,
-                                                  float* __restrict__ vmax) {
-    __shared__ double sh[RB];
-    __shared__ int vm[3];
-    if (threadIdx.x < 3) vm[threadIdx.x] = 0;
-    __syncthreads();
-    T ea = 0, eb = 0;
-    float mc = 0.f, ma = 0.f, mb = 0.f;
-    const T w0 = T(cf.w[0]), w1 = T(cf.w[1]), w2 = T(cf.w[2]);
-    for (int p = blockIdx.x * RB + threadIdx.x; p < N3; p += gridDim.x * RB) {
-        const T v0 = vloc[p] + vh[p].x;
-        const T vc = w0 * v0 + xc3[p];
-        const T va = w1 * v0 + xc3[N3 + p];
-        const T vb = w2 * v0 + xc3[2 * N3 + p];
-        Vk[p] = vc;
-        Vk[N3 + p] = va;
-        Vk[2 * N3 + p] = vb;
-        if (vmax) {
-            mc = fmaxf(mc, fabsf(float(vc)));
-            ma = fmaxf(ma, fabsf(float(va)));
-            mb = fmaxf(mb, fabsf(float(vb)));
-        }
-        if (Vk64) {
-            Vk64[p] = double(vc);
-            Vk64[N3 + p] = double(va);
-            Vk64[2 * N3 + p] = double(vb);
-        }
-        ea += vc * T(DensAcc<T>::value(rho3[N3 + p]));
-        eb += vc * T(DensAcc<T>::value(rho3[2 * N3 + p]));
-    }
-    if (vmax) {
-        // floats >= 0 order like their bits; vmax was zeroed before the launch
-        atomicMax(&vm[0], __float_as_int(mc));
-        atomicMax(&vm[1], __float_as_int(ma));
-        atomicMax(&vm[2], __float_as_int(mb));
-    }
-    const double dea = block_sum_t<T>(ea, sh);
-    const double deb = block_sum_t<T>(eb, sh);
-    if (vmax && threadIdx.x < 3) atomicMax(reinterpret_cast<int*>(vmax) + threadIdx.x, vm[threadIdx.x]);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x * 2 + 0] = dea;
-        part[blockIdx.x * 2 + 1] = deb;
-    }
-}
-
-// Sum per-block partials in a fixed order: out[q] = scale[q] * sum_b part[b * nq + q];
-// one block per quantity.
-__global__ void __launch_bounds__(RB) k_partials_final(int nblocks, int nq, const double* __restrict__ part,
-                                                       double* __restrict__ out, double s0, double s1, double s2,
-                                                       double s3) {
+// The potentials' sums, one block per quantity, partials in a fixed order:
+// out[0..2] from a (4 per block: E_x^M, E_x^T, E_loc), out[3] from b (E_H),
+// out[4..5] from c (2 per block: <a|V^c|a>, <b|V^c|b>).
+__global__ void __launch_bounds__(RB) k_pot_final(int na, const double* __restrict__ a, int nb,
+                                                  const double* __restrict__ b, int nc, const double* __restrict__ c,
+                                                  double dvol, double eh, double* __restrict__ out) {
     __shared__ double sh[RB];
     const int q = blockIdx.x;
+    const double* p = q < 3 ? a + q : (q == 3 ? b : c + q - 4);
+    const int n = q < 3 ? na : (q == 3 ? nb : nc), stride = q < 3 ? 4 : (q == 3 ? 1 : 2);
     double s = 0;
-    for (int b = threadIdx.x; b < nblocks; b += RB) s += part[b * nq + q];
+    for (int k = threadIdx.x; k < n; k += RB) s += p[k * stride];
     s = block_sum(s, sh);
-    const double sc[4] = {s0, s1, s2, s3};
-    if (threadIdx.x == 0) out[q] = s * sc[q];
+    if (threadIdx.x == 0) out[q] = s * (q == 3 ? eh : dvol);
 }
 
 // ------------------------------------------------------------------ PCG pointwise
@@ -736,11 +609,11 @@ void density_to_f64(int64_t n, const double* rho3, double* out, cudaStream_t st)
 template void density_to_f64<float>(int64_t, const double*, double*, cudaStream_t);
 template void density_to_f64<double>(int64_t, const double*, double*, cudaStream_t);
 
-constexpr int kPotBlocks = 512;
+constexpr int kPotBlocks = 512;   // also the most blocks of a pass over tiles of x lines (N * ceil(N / lines))
 
 template <typename T>
 void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoef& cf, c2<T>* grid,
-                T* xc3, const c2<T>* tw, T* Vk, double* Vk64, double* part, double* out6,
+                T* xc3, const c2<T>* tw, T* Vk, double* part, double* out6,
                 cudaStream_t st, bool energies_only, const GgaWork* gga, float* vmax) {
     // out6: [E_x^M, E_x^T, E_loc, E_H, <a|V^c|a>, <b|V^c|b>]; energies_only
     // stops after E_H (out6[4..5] and Vk are left as they were)
@@ -749,55 +622,65 @@ void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoe
     const double c6 = std::cbrt(6.0 / kPi);                 // (6 / pi)^{1/3}
     const double b = 2.0 * kPi / L;
     using DS = typename DensAcc<T>::S;
-    const DS* r3 = reinterpret_cast<const DS*>(rho3);
-    PotCoefT<T> ct;
-    for (int k = 0; k < 3; ++k)
+    PotArgs<T> a;
+    a.N = N;
+    a.tw = tw;
+    a.rho3 = reinterpret_cast<const DS*>(rho3);
+    a.vloc = vloc;
+    for (int k = 0; k < 3; ++k) {
+        a.w[k] = T(cf.w[k]);
         for (int ch = 0; ch < 4; ++ch) {
-            ct.f[k][ch] = T(cf.f[k][ch]);
-            ct.C[k][ch] = T(cf.C[k][ch]);
+            a.ct.f[k][ch] = T(cf.f[k][ch]);
+            a.ct.C[k][ch] = T(cf.C[k][ch]);
         }
-    ct.xscale = T(cf.xscale);
+    }
+    a.ct.xscale = T(cf.xscale);
+    a.c6 = T(c6);
+    a.cx = T(0.75 * c6);
+    a.inv = T(1.0 / double(N3));
+    a.fpb = T(4.0 * kPi / (b * b));
+    a.grid = grid;
+    a.xc3 = xc3;
+    a.Vk = Vk;
+    a.partA = part;
+    a.partB = part + 4 * kPotBlocks;
+    a.partC = a.partB + kPotBlocks;
+    a.vmax = vmax;
     c2<T>* gg = gga ? static_cast<c2<T>*>(gga->gg) : nullptr;
     c2<T>* dd = gga ? static_cast<c2<T>*>(gga->dd) : nullptr;
+    int na = kPotBlocks;
     if (!gga) {
-        roks::count_launch(), k_pot_xc<T><<<kPotBlocks, RB, 0, st>>>(N3, r3, vloc, ct, T(c6), T(0.75 * c6), grid,
-                                                                      xc3, part);
+        na = pot_x_fwd<T>(a, !energies_only, st);
     } else {
         // PBE exchange: the channels' gradients by two forward and six
         // inverse grid transforms, then the pointwise energy, de/drho and flux
-        const T inv = T(1.0 / double(N3));
-        roks::count_launch(), k_gga_pack<T><<<kPotBlocks, RB, 0, st>>>(N3, r3, vloc, ct, grid, gg, part);
+        roks::count_launch(), k_gga_pack<T><<<kPotBlocks, RB, 0, st>>>(N3, a.rho3, vloc, a.ct, grid, gg, part);
         grid_fft3_batched<T>(N, tw, gg, 2, (int64_t)N3, -1, st);
-        roks::count_launch(), k_gga_grad<T><<<kPotBlocks, RB, 0, st>>>(N, T(b), inv, gg, dd);
+        roks::count_launch(), k_gga_grad<T><<<kPotBlocks, RB, 0, st>>>(N, T(b), a.inv, gg, dd);
         grid_fft3_batched<T>(N, tw, dd, 6, (int64_t)N3, +1, st);
         roks::count_launch(), k_gga_point<T><<<kPotBlocks, RB, 0, st>>>(
-                                  N3, r3, ct, T(0.75 * c6), T(std::pow(6.0 * kPi * kPi, 2.0 / 3.0)), T(gga->mu),
+                                  N3, a.rho3, a.ct, a.cx, T(std::pow(6.0 * kPi * kPi, 2.0 / 3.0)), T(gga->mu),
                                   T(gga->kappa), T(gga->rho_min), dd, static_cast<T*>(gga->v4), part);
     }
-    roks::count_launch(), k_partials_final<<<4, RB, 0, st>>>(kPotBlocks, 4, part, out6, dvol, dvol, dvol, 0.0);
-    grid_fft3<T>(N, tw, grid, -1, st);
-    roks::count_launch(), k_hartree_G<T><<<kPotBlocks, RB, 0, st>>>(N, T(1.0 / double(N3)), T(4.0 * kPi / (b * b)),
-                                                                     grid, part);
-    roks::count_launch(), k_partials_final<<<1, RB, 0, st>>>(kPotBlocks, 1, part, out6 + 3, 0.5 * L * L * L, 0, 0, 0);
-    if (energies_only) return;
-    if (gga) {
-        // the divergence of the fluxes: six forward transforms, i G . flux,
-        // two inverse transforms
-        const T inv = T(1.0 / double(N3));
-        grid_fft3_batched<T>(N, tw, dd, 6, (int64_t)N3, -1, st);
-        roks::count_launch(), k_gga_div<T><<<kPotBlocks, RB, 0, st>>>(N, T(b), inv, dd, gg);
-        grid_fft3_batched<T>(N, tw, gg, 2, (int64_t)N3, +1, st);
-        roks::count_launch(), k_gga_combine<T><<<kPotBlocks, RB, 0, st>>>(N3, ct, static_cast<const T*>(gga->v4),
-                                                                           gg, xc3);
+    const int nb = pot_hartree<T>(a, !gga, st);
+    int nc = 0;
+    if (!energies_only) {
+        if (gga) {
+            // the divergence of the fluxes: six forward transforms, i G . flux,
+            // two inverse transforms
+            grid_fft3_batched<T>(N, tw, dd, 6, (int64_t)N3, -1, st);
+            roks::count_launch(), k_gga_div<T><<<kPotBlocks, RB, 0, st>>>(N, T(b), a.inv, dd, gg);
+            grid_fft3_batched<T>(N, tw, gg, 2, (int64_t)N3, +1, st);
+            roks::count_launch(), k_gga_combine<T><<<kPotBlocks, RB, 0, st>>>(
+                                      N3, a.ct, static_cast<const T*>(gga->v4), gg, xc3);
+        }
+        nc = pot_x_class<T>(a, st);
     }
-    grid_fft3<T>(N, tw, grid, +1, st);
-    if (vmax) cudaMemsetAsync(vmax, 0, 3 * sizeof(float), st);
-    roks::count_launch(), k_pot_class<T><<<kPotBlocks, RB, 0, st>>>(N3, vloc, grid, xc3, r3, cf, Vk, Vk64, part,
-                                                                        vmax);
-    roks::count_launch(), k_partials_final<<<2, RB, 0, st>>>(kPotBlocks, 2, part, out6 + 4, dvol, dvol, 0, 0);
+    roks::count_launch(), k_pot_final<<<energies_only ? 4 : 6, RB, 0, st>>>(na, a.partA, nb, a.partB, nc, a.partC,
+                                                                           dvol, 0.5 * L * L * L, out6);
 }
 
-size_t potentials_part_elems() { return (size_t)kPotBlocks * 4; }
+size_t potentials_part_elems() { return (size_t)kPotBlocks * 7; }
 
 template <typename T>
 void precondition(int npw, int nb, const c2<T>* gI, int64_t ld, const T* g2h, const double* sums, c2<T>* out,
@@ -824,8 +707,8 @@ void axpy(int npw, int nb, const c2<T>* x, int64_t ldx, const c2<T>* y, int64_t 
     template void column_total<T>(int, int, int, const c2<T>*, int64_t, const c2<T>*, int64_t, const T*,      \
                                   double*, double*, double, cudaStream_t);                                     \
     template void potentials<T>(int, double, const double*, const T*, const PotCoef&, c2<T>*, T*,             \
-                                const c2<T>*, T*, double*, double*, double*, cudaStream_t, bool,              \
-                                const GgaWork*, float*);                                                       \
+                                const c2<T>*, T*, double*, double*, cudaStream_t, bool, const GgaWork*,       \
+                                float*);                                                                       \
     template void precondition<T>(int, int, const c2<T>*, int64_t, const T*, const double*, c2<T>*,           \
                                   int64_t, cudaStream_t);                                                      \
     template void axpy<T>(int, int, const c2<T>*, int64_t, const c2<T>*, int64_t, const double*, double,      \

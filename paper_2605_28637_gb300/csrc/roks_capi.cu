@@ -474,7 +474,7 @@ struct Impl {
         PROF("potential");
         potentials<T>(ctx->N, ctx->L, ctx->d_rho3, static_cast<const T*>(ctx->d_vloc_t), ctx->cf,
                       reinterpret_cast<V*>(ctx->d_grid), reinterpret_cast<T*>(ctx->d_xc3), ccv(ctx->d_tw),
-                      static_cast<T*>(ctx->d_Vk), nullptr, ctx->d_part, ctx->d_out6, st, energies_only,
+                      static_cast<T*>(ctx->d_Vk), ctx->d_part, ctx->d_out6, st, energies_only,
                       ctx->xc == ROKS_XC_PBE_X ? &ctx->gga : nullptr, ctx->d_vmax);
         energy_combine(ctx->d_kin_b, ctx->d_nl_b, ctx->nocc, ctx->d_wband, ctx->d_out6, ctx->cM, ctx->cT,
                        ctx->alpha, ctx->alpha != 0.0 ? ctx->d_hf2 : nullptr, ctx->d_E, st);

@@ -71,9 +71,32 @@ struct GgaWork {
     void* v4 = nullptr;   // 4 N^3 T: de/drho per channel
     double mu = 0, kappa = 0, rho_min = 0;
 };
+// The potentials' passes over the grid (k_pot_impl.cuh), each returning the
+// number of its partial sums: x lines forward with the Slater exchange (fields
+// null: energies alone), planes with the Hartree kernel (x_done: the x lines
+// are transformed already), x lines inverse with the class potentials.
+template <typename T>
+struct PotArgs {
+    int N;
+    const c2<T>* tw;
+    const typename DensAcc<T>::S* rho3;
+    const T* vloc;
+    PotCoefT<T> ct;
+    T w[3], c6, cx, inv, fpb;   // (6 / pi)^{1/3}, 0.75 of it, 1 / N^3, 4 pi / b^2
+    c2<T>* grid;
+    T *xc3, *Vk;
+    double *partA, *partB, *partC;   // 4, 1, 2 values per block
+    float* vmax;
+};
+template <typename T>
+int pot_x_fwd(const PotArgs<T>& a, bool fields, cudaStream_t st);
+template <typename T>
+int pot_hartree(const PotArgs<T>& a, bool x_done, cudaStream_t st);
+template <typename T>
+int pot_x_class(const PotArgs<T>& a, cudaStream_t st);
 template <typename T>
 void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoef& cf, c2<T>* grid,
-                T* xc3, const c2<T>* tw, T* Vk, double* Vk64, double* part, double* out6,
+                T* xc3, const c2<T>* tw, T* Vk, double* part, double* out6,
                 cudaStream_t st, bool energies_only = false, const GgaWork* gga = nullptr, float* vmax = nullptr);
 size_t potentials_part_elems();
 template <typename T>
