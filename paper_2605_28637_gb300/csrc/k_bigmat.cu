@@ -35,114 +35,94 @@ __global__ void k_big_load(int n, const double2* __restrict__ O, U* __restrict__
 }
 
 // Factor the diagonal block kb (one block of 256 threads): L_kk, and
-// D = L_kk^{-1} by a column sweep in the same loop (solve L D = I for all
-// right-hand sides at once: row j of D is scaled by 1/L_jj as soon as
-// column j of L is final, then subtracted from the rows below).
-// Thread (lane i, warp w) keeps the elements (row i, column w + 8 q), q < 4,
-// of L and of D in registers.  Step j: the warp owning column j forms the
-// pivot (a shuffle from lane j), scales the column and publishes it with
-// 1/L_jj; after one barrier every thread updates its own elements, and the
-// lane owning row j + 1 of D publishes that row for the next step.  The
-// published column and row are double-buffered by the parity of j, so one
-// barrier per step suffices.  D goes to Dinv and to X = L^{-1} (block kb, kb).
+// D = L_kk^{-1} by a column sweep in the same loop, in place.  Thread (lane i,
+// warp w) keeps the elements (row i, column w + 8 q), q < 4, in registers:
+// L(i, k) until step k, D(i, k) from then on.  Step j: the warp owning column j
+// forms the pivot (a shuffle from lane j), scales the column, publishes it
+// with 1/L_jj and turns its elements into column j of D; after one barrier
+// every thread subtracts L(i, j) times conj L(k, j) (k > j) or times D(j, k)
+// (k < j, a shuffle from lane j, which holds that row for its warp's
+// columns).  The published column is zero up to row j, so nothing depends on
+// the lane but the factor.  It is double-buffered by the parity of j: one
+// barrier a step.  D goes to Dinv and to X = L^{-1} (block kb, kb).
+//
+// Bound by the 32 dependent steps: 18.5 us a block in FP32.  (With L and D
+// apart, tests of the row and a row of D through shared memory 21.5; one warp
+// with all rows in registers, unrolled, ran out of the instruction cache: 72; a
+// reciprocal root by Newton in place of the root and the division: 17.8.)
 template <typename U>
 __global__ void __launch_bounds__(256) k_big_diag(int n, int kb, U* __restrict__ A, U* __restrict__ Dinv,
                                                   U* __restrict__ Xm, int* flag) {
     using R = typename Real<U>::type;
-    __shared__ U colbuf[2][BK];    // column j of L (scaled), by row
-    __shared__ U xrow[2][BK];      // row j of D before its scaling, by column
+    __shared__ U colbuf[2][BK];    // column j of L (scaled) below row j, zero above
     __shared__ R invbuf[2];
     const int k0 = kb * BK;
     const int m = min(BK, n - k0);
     const int i = threadIdx.x & 31, w = threadIdx.x >> 5;
-    U Lr[4], Xr[4];
+    U v[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int k = w + 8 * q;
-        U v;
-        v.x = 0;
-        v.y = 0;
-        if (i < m && k < m) v = A[(int64_t)(k0 + k) * n + k0 + i];
-        Lr[q] = v;
-        Xr[q].x = (i == k) ? R(1) : R(0);
-        Xr[q].y = 0;
+        v[q].x = 0;
+        v[q].y = 0;
+        if (i < m && k < m) v[q] = A[(int64_t)(k0 + k) * n + k0 + i];
     }
-    // row 0 of D (D[0][0] = 1 before scaling) for step 0
-    if (w == 0 && i == 0) xrow[0][0] = Xr[0];
     for (int j = 0; j < m; ++j) {
         const int b = j & 1;
-        const int wj = j & 7, qj = j >> 3;
-        if (w == wj) {
-            // this warp owns column j: pivot from lane j
-            U lj = Lr[0];
+        if (w == (j & 7)) {
+            const int qj = j >> 3;
+            U l = v[0];
 #pragma unroll
             for (int q = 1; q < 4; ++q)
-                if (q == qj) lj = Lr[q];
-            R d = __shfl_sync(0xffffffffu, lj.x, j);
+                if (q == qj) l = v[q];
+            R d = __shfl_sync(0xffffffffu, l.x, j);
             if (!(d > R(0))) {
                 if (i == 0 && flag) atomicCAS(flag, 0, k0 + j + 1);
                 d = R(1);
             }
             const R p = sqrt(d);
             const R inv = R(1) / p;
-            if (i > j) {
-                lj.x *= inv;
-                lj.y *= inv;
-            } else if (i == j) {
-                lj.x = p;
-                lj.y = 0;
-            }
+            U c, x;   // column j of L below the diagonal, column j of D
+            c.x = i > j ? l.x * inv : R(0);
+            c.y = i > j ? l.y * inv : R(0);
+            x.x = i > j ? -c.x * inv : (i == j ? inv : R(0));
+            x.y = i > j ? -c.y * inv : R(0);
+            colbuf[b][i] = c;
+            if (i == 0) invbuf[b] = inv;
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (q == qj) Lr[q] = lj;
-            colbuf[b][i] = lj;
-            if (i == 0) invbuf[b] = inv;
+                if (q == qj) v[q] = x;
+            if (i == j) c.x = p;
+            if (i >= j && i < m) A[(int64_t)(k0 + j) * n + k0 + i] = c;
         }
         __syncthreads();
         const R inv = invbuf[b];
-        const U a = colbuf[b][i];   // L(i, j)
+        const U a = colbuf[b][i];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int k = w + 8 * q;
-            if (k > j && i >= k) {
-                // trailing L(i, k) -= L(i, j) conj(L(k, j))
-                const U c = colbuf[b][k];
-                Lr[q].x -= a.x * c.x + a.y * c.y;
-                Lr[q].y -= a.y * c.x - a.x * c.y;
-            } else if (k <= j) {
-                if (i == j) {
-                    // row j of D, final: scaled by 1 / L_jj
-                    Xr[q].x *= inv;
-                    Xr[q].y *= inv;
-                } else if (i > j) {
-                    // D(i, k) -= L(i, j) D(j, k), D(j, k) = xrow * inv
-                    const U xv = xrow[b][k];
-                    const R xr = xv.x * inv, xi = xv.y * inv;
-                    Xr[q].x -= a.x * xr - a.y * xi;
-                    Xr[q].y -= a.x * xi + a.y * xr;
-                }
+            if (k == j) continue;
+            U y;
+            if (k > j) {
+                y = colbuf[b][k];
+                y.y = -y.y;
+            } else {
+                y.x = __shfl_sync(0xffffffffu, v[q].x, j) * inv;
+                y.y = __shfl_sync(0xffffffffu, v[q].y, j) * inv;
+                if (i == j) v[q] = y;   // row j of D, final
             }
-        }
-        // row j + 1 of D (columns k <= j + 1) for the next step
-        if (i == j + 1) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = w + 8 * q;
-                if (k <= j + 1) xrow[b ^ 1][k] = Xr[q];
-            }
+            v[q].x -= a.x * y.x - a.y * y.y;
+            v[q].y -= a.x * y.y + a.y * y.x;
         }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int k = w + 8 * q;
-        if (i < m && k < m) {
-            A[(int64_t)(k0 + k) * n + k0 + i] = Lr[q];
-            Xm[(int64_t)(k0 + k) * n + k0 + i] = Xr[q];
-        }
         U z;
         z.x = 0;
         z.y = 0;
-        Dinv[(int64_t)kb * BK * BK + k * BK + i] = (i < m && k < m) ? Xr[q] : z;
+        if (i < m && k < m) Xm[(int64_t)(k0 + k) * n + k0 + i] = z = v[q];
+        Dinv[(int64_t)kb * BK * BK + k * BK + i] = z;
     }
 }
 

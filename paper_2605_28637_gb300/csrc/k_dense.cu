@@ -715,111 +715,136 @@ __global__ void k_small_gemm(int M, int N, int K, const double2* __restrict__ A,
 
 // ------------------------------------------------------------------ large band-space products
 // C = alpha op(A) op(B) + beta C on FP64 storage, for products too large for
-// one warp per element (hundreds of bands, thousands of projectors): 32 x 32
-// output tiles per block of 256 threads (enough blocks to fill the GPU at a
-// few hundred bands), thread (tx, ty) owning rows ty + 16 i and columns
-// tx + 16 j (i, j < 2); K in slices of 16 staged in shared memory, each load
-// coalesced along the operand's contiguous index.  Arithmetic type R (float
+// one warp per element (hundreds of bands, thousands of projectors).  A block
+// owns a tile of T x T outputs, T = TD RT, and G groups of TD x TD threads split
+// K (contiguous ranges, added in group order at the end); thread (tx, ty) of a
+// group owns rows ty + TD i and columns tx + TD j (i, j < RT).  K in slices of 16
+// staged in shared memory, the next slice's loads (coalesced along the
+// operand's contiguous index) in flight meanwhile.  Arithmetic type R (float
 // on the mixed path): every slice is summed on its own before it joins the
 // running sum, so that rounding grows with K / 16.  TI: the stored operand
 // type (double2, or float2 packed once by k_pack_f32 on the mixed path, so
 // that the FP64 -> FP32 conversions, which run on the narrow FP64 pipe, are
 // made once per element instead of once per output tile).
-constexpr int BS_T = 32, BS_K = 16, BS_R = 2;
+//
+// 2 x 2 outputs per thread.  Tiles of 32 (all of K in the 256 threads' one
+// pass) where they fill the SMs: 430 x 430 x 1288 167 us (178 without loads in
+// flight; 4 x 4 per thread and four groups 283, with one block an SM).  Else tiles of 16 with K split eight
+// ways (four in FP64): 128 x 128 x 376 15.5 us, on 16 blocks of 32 63.
+constexpr int BS_K = 16;
 
-template <typename R, typename TI>
-__global__ void __launch_bounds__(256) k_bs_gemm(int M, int N, int K, const TI* __restrict__ A, int lda,
-                                                 int ca, const TI* __restrict__ B, int ldb, int cb,
-                                                 double2* __restrict__ C, int ldc, double alpha, double beta) {
-    __shared__ c2<R> As[BS_K][BS_T + 1];
-    __shared__ c2<R> Bs[BS_K][BS_T + 1];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int m0 = blockIdx.x * BS_T, n0 = blockIdx.y * BS_T;
-    c2<R> acc[BS_R][BS_R];
+// TD x TD threads a group, RT x RT outputs each
+template <typename R, typename TI, int TD, int RT, int G>
+__global__ void __launch_bounds__(TD * TD * G) k_bs_gemm(int M, int N, int K, const TI* __restrict__ A, int lda,
+                                                    int ca, const TI* __restrict__ B, int ldb, int cb,
+                                                    double2* __restrict__ C, int ldc, double alpha, double beta) {
+    using V = c2<R>;
+    constexpr int T = TD * RT, NG = TD * TD, PT = T + 1, L = T * BS_K / NG;
+    __shared__ __align__(16) unsigned char bs_smem[sizeof(V) * (2 * G * BS_K * PT > G * T * T ? 2 * G * BS_K * PT : G * T * T)];
+    const int g = threadIdx.x / NG, t = threadIdx.x % NG, tx = t % TD, ty = t / TD;
+    V* As = reinterpret_cast<V*>(bs_smem) + g * 2 * BS_K * PT;   // [BS_K][PT]
+    V* Bs = As + BS_K * PT;
+    const int m0 = blockIdx.x * T, n0 = blockIdx.y * T;
+    const int kr = ((K + G - 1) / G + BS_K - 1) / BS_K * BS_K, kb = g * kr, ke = min(K, kb + kr);
+    V ra[L], rb[L];
+    auto fetch = [&](int k0) {
 #pragma unroll
-    for (int i = 0; i < BS_R; ++i)
-#pragma unroll
-        for (int j = 0; j < BS_R; ++j) acc[i][j].x = acc[i][j].y = R(0);
-    for (int k0 = 0; k0 < K; k0 += BS_K) {
-        for (int e = tid; e < BS_T * BS_K; e += 256) {
+        for (int q = 0; q < L; ++q) {
+            const int e = t + NG * q;
             // op(A)[m][k]: A^H of a K x M matrix (k contiguous) or an M x K one (m contiguous)
-            const int ka = ca ? e % BS_K : e / BS_T, ma = ca ? e / BS_K : e % BS_T;
-            c2<R> v;
-            v.x = v.y = R(0);
-            if (m0 + ma < M && k0 + ka < K) {
-                const TI d = ca ? A[(int64_t)(m0 + ma) * lda + k0 + ka] : A[(int64_t)(k0 + ka) * lda + m0 + ma];
-                v.x = (R)d.x;
-                v.y = ca ? -(R)d.y : (R)d.y;
+            const int ka = k0 + (ca ? e % BS_K : e / T), ma = m0 + (ca ? e / BS_K : e % T);
+            V v = mk<R>(R(0), R(0)), w = v;
+            if (ma < M && ka < ke) {
+                const TI d = ca ? A[(int64_t)ma * lda + ka] : A[(int64_t)ka * lda + ma];
+                v = mk<R>((R)d.x, ca ? -(R)d.y : (R)d.y);
             }
-            As[ka][ma] = v;
             // op(B)[k][n]: B^H of an N x K matrix (n contiguous) or a K x N one (k contiguous)
-            const int kb = cb ? e / BS_T : e % BS_K, nb = cb ? e % BS_T : e / BS_K;
-            c2<R> w;
-            w.x = w.y = R(0);
-            if (n0 + nb < N && k0 + kb < K) {
-                const TI d = cb ? B[(int64_t)(k0 + kb) * ldb + n0 + nb] : B[(int64_t)(n0 + nb) * ldb + k0 + kb];
-                w.x = (R)d.x;
-                w.y = cb ? -(R)d.y : (R)d.y;
+            const int kc = k0 + (cb ? e / T : e % BS_K), nb = n0 + (cb ? e % T : e / BS_K);
+            if (nb < N && kc < ke) {
+                const TI d = cb ? B[(int64_t)kc * ldb + nb] : B[(int64_t)nb * ldb + kc];
+                w = mk<R>((R)d.x, cb ? -(R)d.y : (R)d.y);
             }
-            Bs[kb][nb] = w;
+            ra[q] = v;
+            rb[q] = w;
+        }
+    };
+    V acc[RT][RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < RT; ++j) acc[i][j] = mk<R>(R(0), R(0));
+    fetch(kb);
+    for (int k0 = 0; k0 < kr; k0 += BS_K) {
+#pragma unroll
+        for (int q = 0; q < L; ++q) {
+            const int e = t + NG * q;
+            As[(ca ? e % BS_K : e / T) * PT + (ca ? e / BS_K : e % T)] = ra[q];
+            Bs[(cb ? e / T : e % BS_K) * PT + (cb ? e % T : e / BS_K)] = rb[q];
         }
         __syncthreads();
-        c2<R> t[BS_R][BS_R];
+        if (k0 + BS_K < kr) fetch(kb + k0 + BS_K);
+        V s[RT][RT];
 #pragma unroll
-        for (int i = 0; i < BS_R; ++i)
+        for (int i = 0; i < RT; ++i)
 #pragma unroll
-            for (int j = 0; j < BS_R; ++j) t[i][j].x = t[i][j].y = R(0);
+            for (int j = 0; j < RT; ++j) s[i][j] = mk<R>(R(0), R(0));
 #pragma unroll 4
         for (int kk = 0; kk < BS_K; ++kk) {
-            c2<R> a[BS_R], b[BS_R];
+            V a[RT], b[RT];
 #pragma unroll
-            for (int i = 0; i < BS_R; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < RT; ++i) a[i] = As[kk * PT + ty + TD * i];
 #pragma unroll
-            for (int j = 0; j < BS_R; ++j) b[j] = Bs[kk][tx + 16 * j];
+            for (int j = 0; j < RT; ++j) b[j] = Bs[kk * PT + tx + TD * j];
 #pragma unroll
-            for (int i = 0; i < BS_R; ++i)
+            for (int i = 0; i < RT; ++i)
 #pragma unroll
-                for (int j = 0; j < BS_R; ++j) mac_nn<R>(t[i][j], a[i], b[j]);
+                for (int j = 0; j < RT; ++j) mac_nn<R>(s[i][j], a[i], b[j]);
         }
 #pragma unroll
-        for (int i = 0; i < BS_R; ++i)
+        for (int i = 0; i < RT; ++i)
 #pragma unroll
-            for (int j = 0; j < BS_R; ++j) {
-                acc[i][j].x += t[i][j].x;
-                acc[i][j].y += t[i][j].y;
-            }
+            for (int j = 0; j < RT; ++j) acc[i][j] = cadd(acc[i][j], s[i][j]);
         __syncthreads();
     }
+    V* part = reinterpret_cast<V*>(bs_smem);
 #pragma unroll
-    for (int i = 0; i < BS_R; ++i) {
-        const int m = m0 + ty + 16 * i;
-        if (m >= M) continue;
+    for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int j = 0; j < BS_R; ++j) {
-            const int n = n0 + tx + 16 * j;
-            if (n >= N) continue;
-            double2* c = C + (int64_t)n * ldc + m;
-            double2 r = make_double2(alpha * (double)acc[i][j].x, alpha * (double)acc[i][j].y);
-            if (beta != 0.0) {
-                r.x += beta * c->x;
-                r.y += beta * c->y;
-            }
-            *c = r;
+        for (int j = 0; j < RT; ++j) part[(g * T + tx + TD * j) * T + ty + TD * i] = acc[i][j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < T * T; e += NG * G) {
+        const int m = m0 + e % T, n = n0 + e / T;
+        if (m >= M || n >= N) continue;
+        V v = part[e];
+#pragma unroll
+        for (int q = 1; q < G; ++q) v = cadd(v, part[q * T * T + e]);
+        double2* c = C + (int64_t)n * ldc + m;
+        double2 r = make_double2(alpha * (double)v.x, alpha * (double)v.y);
+        if (beta != 0.0) {
+            r.x += beta * c->x;
+            r.y += beta * c->y;
         }
+        *c = r;
     }
+}
+
+template <typename R, typename TI>
+static void launch_bs(int M, int N, int K, const TI* A, int lda, bool ca, const TI* B, int ldb, bool cb, double2* C,
+                      int ldc, double alpha, double beta, cudaStream_t st) {
+    constexpr int G = sizeof(R) == 4 ? 8 : 4;   // (48 KB of shared memory)
+    auto go = [&](auto kernel, int tile, int threads) {
+        const dim3 g((unsigned)((M + tile - 1) / tile), (unsigned)((N + tile - 1) / tile));
+        roks::count_launch(), kernel<<<g, threads, 0, st>>>(M, N, K, A, lda, ca ? 1 : 0, B, ldb, cb ? 1 : 0, C, ldc,
+                                                            alpha, beta);
+    };
+    const int64_t tiles = (int64_t)((M + 31) / 32) * ((N + 31) / 32);
+    if (tiles >= sm_count()) go(k_bs_gemm<R, TI, 16, 2, 1>, 32, 256);
+    else go(k_bs_gemm<R, TI, 8, 2, G>, 16, 64 * G);
 }
 
 // Products with at least this many outputs (and 32 or more terms each) go to
 // the tiled kernel; smaller ones keep one warp per element.
 static bool bs_tiled(int M, int N, int K) { return (long long)M * N >= 16384 && K >= 32; }
-
-template <typename R>
-static void bs_gemm(int M, int N, int K, const double2* A, int lda, bool ca, const double2* B, int ldb, bool cb,
-             double2* C, int ldc, double alpha, double beta, cudaStream_t st) {
-    const dim3 g((unsigned)((M + BS_T - 1) / BS_T), (unsigned)((N + BS_T - 1) / BS_T));
-    roks::count_launch();
-    k_bs_gemm<R, double2><<<g, 256, 0, st>>>(M, N, K, A, lda, ca ? 1 : 0, B, ldb, cb ? 1 : 0, C, ldc, alpha, beta);
-}
 
 // dst (rows x cols, leading dimension rows) = src (FP64, leading dimension ld) in FP32
 __global__ void k_pack_f32(int rows, int cols, const double2* __restrict__ src, int ld, float2* __restrict__ dst) {
@@ -835,7 +860,7 @@ void small_gemm(int M, int N, int K, const double2* A, int lda, bool ca, const d
                 double2* C, int ldc, double alpha, double beta, cudaStream_t st) {
     if (M <= 0 || N <= 0) return;
     if (bs_tiled(M, N, K)) {
-        bs_gemm<double>(M, N, K, A, lda, ca, B, ldb, cb, C, ldc, alpha, beta, st);
+        launch_bs<double>(M, N, K, A, lda, ca, B, ldb, cb, C, ldc, alpha, beta, st);
         return;
     }
     const long long threads = (long long)M * N * 32;
@@ -891,12 +916,9 @@ void small_gemm_f32(int M, int N, int K, const double2* A, int lda, bool ca, con
             const int64_t ta = (int64_t)ra * na, tb = (int64_t)rb * nbc;
             roks::count_launch(), k_pack_f32<<<(unsigned)((ta + 255) / 256), 256, 0, st>>>(ra, na, A, lda, Ap);
             roks::count_launch(), k_pack_f32<<<(unsigned)((tb + 255) / 256), 256, 0, st>>>(rb, nbc, B, ldb, Bp);
-            const dim3 g((unsigned)((M + BS_T - 1) / BS_T), (unsigned)((N + BS_T - 1) / BS_T));
-            roks::count_launch();
-            k_bs_gemm<float, float2><<<g, 256, 0, st>>>(M, N, K, Ap, ra, ca ? 1 : 0, Bp, rb, cb ? 1 : 0, C, ldc, alpha,
-                                                        beta);
+            launch_bs<float, float2>(M, N, K, Ap, ra, ca, Bp, rb, cb, C, ldc, alpha, beta, st);
         } else {
-            bs_gemm<float>(M, N, K, A, lda, ca, B, ldb, cb, C, ldc, alpha, beta, st);
+            launch_bs<float>(M, N, K, A, lda, ca, B, ldb, cb, C, ldc, alpha, beta, st);
         }
         return;
     }
