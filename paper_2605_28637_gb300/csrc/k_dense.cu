@@ -353,7 +353,11 @@ int cn_resident_blocks(int rm, int rn, int threads, size_t smem) {
 }
 
 // Register tile and thread grid with the least padded work (plus the
-// shared-memory loads per multiply-add), then K chunks for whole waves of
+// shared-memory loads per multiply-add; in long FP64 sums, where the pipes of
+// the SM's four parts set the time, threads short of a multiple of four warps
+// count as work: 172 x 42 over 34,265 rows with 210 threads a block 2.67 ms, with
+// 126 1.76; over 1050 rows the partials of smaller tiles cost more: a tiny-16
+// PCG step 569 us, 607 with them), then K chunks for whole waves of
 // resident blocks, each at least two K slices long.  FP64 products are bound
 // by the pipe of the SMs that take part (two multiply-adds a cycle each), so
 // their chunks go down to half a slice, up to as many as there are SMs: 44 x 6
@@ -368,18 +372,24 @@ CnPlan cn_plan(int M, int N, int K, int max_chunks) {
     // faster on these shapes: the kernel is issue-bound at any tile size)
     const int rcand[5] = {1, 2, 3, 4, 6};
     const int nc = 4;
+    const bool pipes = sizeof(T) == 8 && K >= 8192;
     for (int ia = 0; ia < nc; ++ia)
         for (int ib = 0; ib < nc; ++ib) {
             const int rm = rcand[ia], rn = rcand[ib];
-            const int mt = (M + 16 * rm - 1) / (16 * rm), nt = (N + 16 * rn - 1) / (16 * rn);
-            const int ty = (M + mt * rm - 1) / (mt * rm), tx = (N + nt * rn - 1) / (nt * rn);
-            const double covered = (double)mt * ty * rm * nt * tx * rn;
-            double cost = covered * (1.0 + (rm + rn) / (4.0 * rm * rn));
-            if (ty * tx < 64) cost *= 1.5;   // too few threads per block to hide latency
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = CnPlan{rm, rn, ty, tx, mt, nt, 0, 0};
-            }
+            const int mt0 = (M + 16 * rm - 1) / (16 * rm), nt0 = (N + 16 * rn - 1) / (16 * rn);
+            const int more = pipes ? 2 : 0;   // also smaller tiles
+            for (int mt = mt0; mt <= mt0 + more; ++mt)
+                for (int nt = nt0; nt <= nt0 + more; ++nt) {
+                    const int ty = (M + mt * rm - 1) / (mt * rm), tx = (N + nt * rn - 1) / (nt * rn);
+                    const double covered = (double)mt * ty * rm * nt * tx * rn;
+                    double cost = covered * (1.0 + (rm + rn) / (4.0 * rm * rn));
+                    if (ty * tx < 64) cost *= 1.5;   // too few threads per block to hide latency
+                    else if (pipes) cost *= (ty * tx + 127) / 128 * 128.0 / (ty * tx);
+                    if (cost < best_cost) {
+                        best_cost = cost;
+                        best = CnPlan{rm, rn, ty, tx, mt, nt, 0, 0};
+                    }
+                }
         }
     const int tiles = best.mt * best.nt;
     int SA = 0, SB = 0;
@@ -729,8 +739,9 @@ __global__ void k_small_gemm(int M, int N, int K, const double2* __restrict__ A,
 //
 // 2 x 2 outputs per thread.  Tiles of 32 (all of K in the 256 threads' one
 // pass) where they fill the SMs: 430 x 430 x 1288 167 us (178 without loads in
-// flight; 4 x 4 per thread and four groups 283, with one block an SM).  Else tiles of 16 with K split eight
-// ways (four in FP64): 128 x 128 x 376 15.5 us, on 16 blocks of 32 63.
+// flight; 4 x 4 per thread and four groups 283, with one block an SM).  Else
+// tiles of 16 with K split eight ways (four in FP64): 128 x 128 x 376 15.5 us,
+// on 16 blocks of 32 63.
 constexpr int BS_K = 16;
 
 // TD x TD threads a group, RT x RT outputs each
