@@ -258,11 +258,15 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
         const int cg = 64 * ((warp - 4) >> 2);   // complex columns cg .. cg + 63
         const int r = 32 * q + lane;          // tile row
         // What the truncating additions of a stage take from its sum, given
-        // back: A^H B's long sums of like sign lose 2.3e-7 of their size
-        // (measured on the norms of 11,075 plane waves; four additions of
-        // half a unit in the last place each, and those inside an MMA), nearly
-        // 2^-22.  The products with the small B of A B lose no measurable part.
-        constexpr float gain = NN ? 1.f : 1.f + 0x1p-22f;
+        // back (A^H B: alpha is the factor).  The norms of A^H A, sums of
+        // like sign, lose 2.3e-7 of their size (11,075 plane waves; four
+        // additions of half a unit in the last place each, and those inside an
+        // MMA), nearly 2^-22; P^H Psi, whose signs mix, half of it: with 2^-23
+        // the nonlocal energy of organic-96 and mgo-72 is -1.6e-6 and -1.6e-5 Ha
+        // off, with 2^-22 -1.6e-5 and -7.5e-5, without 1.4e-5 and 4.5e-5 (FP32
+        // sums: 1.2e-6 and 4.9e-5).  The products with the small B of A B lose no
+        // measurable part.
+        const float gain = NN ? 1.f : alpha;
         float2 re[32], im[32];                // column pairs
 #pragma unroll
         for (int j = 0; j < 32; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
@@ -663,8 +667,14 @@ bool tcg_keep_images() {
     return on == 1;
 }
 
-bool tcg_cn_takes(int M, int N, int K) { return tcg_enabled() && M >= 128 && N >= 64 && K >= 1024; }
-bool tcg_nn_takes(int M, int N, int K) { return tcg_enabled() && M >= 4096 && N >= 64 && K >= 64; }
+// Where the tensor cores take over from the streamed FP32 kernels: from 32
+// bands on.  An MMA costs little less for 32 columns than for 64, so that is
+// where P^H Psi breaks even (32 bands, 160 projectors, 5600 plane waves 19 us
+// both ways; 42 x 172 x 34,265 62 us streamed, 57 here; 63 bands, 320
+// projectors 43 and 27) and P (D B) gains (26 and 25; 67 and 44; 68 and 33).
+// Fewer than 128 rows (the bands against each other) leave an M tile half empty.
+bool tcg_cn_takes(int M, int N, int K) { return tcg_enabled() && M >= 128 && N >= 32 && K >= 1024; }
+bool tcg_nn_takes(int M, int N, int K) { return tcg_enabled() && M >= 4096 && N >= 32 && K >= 64; }
 
 size_t tcg_image_bytes(int rows, int cols) {
     const size_t Q = (rows + 7) / 8, G = (cols + 7) / 8;
@@ -740,7 +750,8 @@ bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2
     const int T = stages(K);
     float2* part = reinterpret_cast<float2*>(w);
     k_tcgemm<false><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, T, sk, tmA, tmB, nullptr, part, nullptr, 0, nullptr, 0,
-                                                          0.f, 0.f, wait_polls());
+                                                          same ? 1.f + 0x1p-22f : 1.f + 0x1p-23f, 0.f,
+                                                          wait_polls());
     roks::count_launch();
     const int mt = (M + GB_M - 1) / GB_M;
     // many CTAs per tile: their segments shared out over the warps of a block
