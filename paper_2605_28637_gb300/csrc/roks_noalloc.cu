@@ -85,9 +85,12 @@ __global__ void __launch_bounds__(256) k_rows_times_upper(int npw, int nb, c2<T>
 // shared memory in block order, every block takes the Cholesky inverse
 // (chol_inverse_block) and multiplies its rows, unless a pivot failed.  The
 // launch chain of the kernels above, 102 us for 6 bands x 1045 rows in FP64,
-// is the cost it removes: 55 us.  Up to 250,000 multiply-adds (rows x
-// bands^2) in FP64, where eight SMs' FP64 pipes take about as long as that
-// chain; in FP32 the shared memory is the limit.
+// is the cost it removes: 55 us.  Up to 7 bands (8 in FP32), where the kernels
+// above fill few threads and the Cholesky is short (times of the chain and
+// here, in us: FP64 1000 x 6 71 and 44, 3000 x 6 109 and 65, 1000 x 8 58 and 65,
+// 1000 x 12 63 and 99; FP32 1000 x 8 46 and 41, 10000 x 6 72 and 53, 700 x 12 48
+// and 52, 6000 x 10 47 and 77), and in FP64 up to 250,000 multiply-adds (rows x
+// bands^2), beyond which eight SMs' FP64 pipes take longer than the chain.
 constexpr int kNaCluster = 8, kNaThreads = 256;
 constexpr size_t kNaSmem = 200 * 1024;
 template <typename T> size_t cluster_smem(int npw, int nb) {
@@ -95,7 +98,8 @@ template <typename T> size_t cluster_smem(int npw, int nb) {
     return sizeof(double2) * 3 * (size_t)nb * nb + sizeof(c2<T>) * rows * nb;
 }
 template <typename T> bool cluster_takes(int npw, int nb) {
-    return cluster_smem<T>(npw, nb) <= kNaSmem && (int64_t)npw * nb * nb <= (sizeof(T) == 8 ? 250000 : 4000000);
+    return nb <= (sizeof(T) == 8 ? 7 : 8) && cluster_smem<T>(npw, nb) <= kNaSmem &&
+           (sizeof(T) == 4 || (int64_t)npw * nb * nb <= 250000);
 }
 
 template <typename T>

@@ -13,7 +13,7 @@ from tests.gpu_helpers import built, rel
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [(1, 1), (5, 3), (64, 1), (500, 2), (1045, 6), (1000, 15), (975, 16), (977, 16), (6944, 6), (6945, 6),
+SIZES = [(1, 1), (5, 3), (900, 7), (900, 8), (900, 9), (64, 1), (500, 2), (1045, 6), (1000, 15), (975, 16), (977, 16), (6944, 6), (6945, 6),
          (300, 28), (4000, 31), (400, 50), (700, 64)]
 
 
