@@ -257,17 +257,17 @@ def family_work(ctx, cfg, family: str, csize: int, rsize: int, precision: str, t
 def tensor_families(ctx, precision: str, tc_launches: int):
     """Kernel families whose products the library puts on the tcgen05 tensor
     cores at this workload (the shape rule of k_tcgemm.cu: A^H B with
-    M >= 128, N >= 64, K >= 1024; tall products with M >= 4096, N >= 64,
+    M >= 128, N >= 32, K >= 1024; tall products with M >= 4096, N >= 32,
     K >= 64), provided tensor-core launches were counted."""
     if precision != "mixed" or not tc_launches:
         return frozenset()
     nb, npj, npw = ctx.nb, ctx.nproj, ctx.npw
 
     def cn(M, N, K):
-        return M >= 128 and N >= 64 and K >= 1024
+        return M >= 128 and N >= 32 and K >= 1024
 
     def nn(M, N, K):
-        return M >= 4096 and N >= 64 and K >= 64
+        return M >= 4096 and N >= 32 and K >= 64
     fams = set()
     if cn(npj, nb, npw):
         fams.add("proj_PhPsi")
@@ -293,13 +293,13 @@ def bf16_peak():
 
 
 def alu_peak(precision: str, bound: str = "alu"):
-    """Peak of a contraction family.  Tensor cores: the TF32 rate (measured
-    bf16 peak x the nominal TF32/BF16 ratio 1.1/2.25) over the three TF32
-    products each FP32 product takes.  SIMT: FP32 FMA from the unit counts
+    """Peak of a contraction family.  Tensor cores: the measured bf16
+    peak (FP16 runs at the same rate) over the three FP16 products each FP32
+    product takes.  SIMT: FP32 FMA from the unit counts
     and clock (no measured FP32 peak is provided), or the FP64 rate."""
     if bound == "tensor":
         b, kind = bf16_peak()
-        return b * (1.1 / 2.25) / 3.0, (f"{kind} bf16 peak x 1.1/2.25 (TF32) / 3 TF32 products per FP32 product")
+        return b / 3.0, f"{kind} bf16 peak / 3 FP16 products per FP32 product"
     if precision == "fp64":
         if "fp64" in MEASURED_ALU:
             return MEASURED_ALU["fp64"], "measured FP64 (cuBLAS DGEMM on this GPU)"
@@ -663,7 +663,9 @@ def hybrid_leg(args, torch):
     roks.roks_profile_enable(ctx.ctx, 0)
     N = cfg["grid"]
     npairs = ctx.nb * (ctx.nb + 1) // 2
-    alg = npairs * (4 * 8 * N ** 3 + 16 * ctx.npw)
+    # points a side that hold the pair densities and W psi without aliasing
+    M = min(N, 4 * int(np.sqrt(2.0 * cfg["ecut"]) * cfg["L"] / (2.0 * np.pi)) + 1)
+    alg = npairs * (4 * 8 * M ** 3 + 16 * ctx.npw)
     ex = prof.get("exchange")
     roof = None
     if ex:

@@ -535,7 +535,7 @@ struct Impl {
             }
         }
         if (ctx->alpha != 0.0 && ctx->exx_M != N) {
-            PROF("exchange");
+            PROF("exchange_add");
             const double M3 = double(ctx->exx_M) * ctx->exx_M * ctx->exx_M;
             exx_add_fields<T>(exx_sphere(ctx), ccv(ctx->d_twx), ccv(ctx->d_Xx), ctx->nb, cv(ctx->d_Ypx),
                               cv(ctx->d_Zc), cv(F), ldf, T(1.0 / M3), st);
