@@ -23,6 +23,17 @@ __host__ __device__ constexpr int tile_lines(int n) {
     return n == 16 ? 16 : (n == 32 || n == 96 || n == 120) ? 32 : 24;
 }
 constexpr int kThreads = 256;
+
+// Lets launches of a kernel have up to `bytes` of dynamic shared memory (the
+// kernel's largest, so that calls of different sizes do not lower each other's
+// limit).  Asked for at every launch: the limit belongs to the current device's
+// context.  The 48 KB that a launch has without asking hold the kernel's static
+// arrays too, up to 8 KB here: hence 40.
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t bytes) {
+    return bytes <= 40 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 // Threads of the x-stage apply: for N = 96 (radix 12 then 8 over 32 lines:
 // 256 and 384 butterflies) 128 threads take 2 and 3 butterflies each with
 // none idle; other lengths keep kThreads.

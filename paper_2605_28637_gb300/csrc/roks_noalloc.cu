@@ -191,9 +191,7 @@ roks_status run(int npw, int nb, void* psi, int64_t ld, cudaStream_t st, unsigne
     int* flag = reinterpret_cast<int*>(Lw + kNaMat);
     if (cluster_takes<T>(npw, nb)) {
         const size_t sm = cluster_smem<T>(npw, nb);
-        if (sm > 48 * 1024 && cudaFuncSetAttribute(k_orth_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)kNaSmem) != cudaSuccess)
-            return ROKS_ECUDA;
+        if (allow_smem(k_orth_cluster<T>, kNaSmem) != cudaSuccess) return ROKS_ECUDA;
         count_launch();
         k_orth_cluster<T><<<kNaCluster, kNaThreads, sm, st>>>(npw, nb, static_cast<V*>(psi), ld, flag);
         return result(flag, st);
