@@ -1160,8 +1160,7 @@ __global__ void __launch_bounds__(1024) k_cholesky_inverse(int n, const double2*
 void cholesky_inverse(int n, const double2* O, double2* Lw, double2* LinvH, int* flag, cudaStream_t st) {
     if (n <= kSmallN) {
         const size_t sm = sizeof(double2) * 2 * n * n;
-        if (sm > 48 * 1024)
-            cudaFuncSetAttribute(k_cholesky_small<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_smem(k_cholesky_small<1024>, sizeof(double2) * 2 * kSmallN * kSmallN);
         roks::count_launch();
         if (n <= 16) k_cholesky_small<128><<<1, 128, sm, st>>>(n, O, LinvH, flag);
         else k_cholesky_small<1024><<<1, 1024, sm, st>>>(n, O, LinvH, flag);

@@ -5,6 +5,7 @@ for all later ones of the process.
 
 Tolerance: the orthonormality that the suite asks of these calls, 1e-12 in FP64
 and 2e-6 in FP32."""
+import os
 import subprocess
 import sys
 
@@ -32,7 +33,8 @@ assert err < (1e-12 if f64 else 2e-6), err
 
 def alone(code):
     built()
-    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0, r.stderr[-2000:]
 
 
@@ -40,3 +42,29 @@ def alone(code):
 @pytest.mark.parametrize("npw,nb,f64", [(3320, 7, True), (3930, 6, True), (5720, 8, False)])
 def test_orthonormalize_noalloc_cluster(npw, nb, f64):
     alone(FREE.format(npw=npw, nb=nb, f64=f64))
+
+
+# 39 bands: 48,672 bytes of the Cholesky kernel's matrices
+@pytest.mark.parametrize("nb", [38, 39, 40])
+@pytest.mark.parametrize("f64", [True, False])
+def test_orthonormalize_noalloc_chain(nb, f64):
+    alone(FREE.format(npw=1000, nb=nb, f64=f64))
+
+
+STEP = """
+import numpy as np
+from oracle import roks as R
+from paper_2605_28637_gb300 import roks, synthetic as syn
+cfg = syn.with_changes(syn.make_config("tiny-16", 0), n_closed={nb}, grid=24, ecut=12.0, mode=0)
+s = R.System(cfg)
+u = syn.orbital_uniforms(cfg, s.npw)
+ctx = roks.Context(cfg, "fp64")
+psi = ctx.init_orbitals(u)
+x = psi[:, :ctx.npw].cpu().numpy().T
+assert np.abs(s.overlap(x) - np.eye({nb})).max() < 1e-12
+"""
+
+
+@pytest.mark.parametrize("nb", [38, 39, 40])
+def test_orthonormalisation(nb):
+    alone(STEP.format(nb=nb))
