@@ -201,6 +201,9 @@ roks_status run(int npw, int nb, void* psi, int64_t ld, cudaStream_t st, unsigne
     V* X = static_cast<V*>(psi);
     gemm_cn_capped<T>(nb, nb, npw, X, ld, X, ld, O, nb, part, kNaMaxChunks, st);
     cholesky_inverse(nb, O, Lw, LinvH, flag, st);
+    // psi is touched only if all before it was launched: the scratch holds an
+    // earlier call's L^{-H} otherwise
+    if (cudaGetLastError() != cudaSuccess) return ROKS_ECUDA;
     const size_t sm = sizeof(V) * ((size_t)nb * 64 + (size_t)nb * nb);
     if (sm > 48 * 1024 &&
         cudaFuncSetAttribute(k_rows_times_upper<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
