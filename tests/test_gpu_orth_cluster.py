@@ -52,25 +52,3 @@ def test_a_failed_pivot_keeps_psi(npw, nb):
         roks.roks_orthonormalize_noalloc(roks.ROKS_FP64, npw, nb, psi, npw, None)
     assert ei.value.status == roks.ROKS_ENOTPOSDEF
     assert torch.equal(psi, kept)
-
-
-@pytest.mark.parametrize("nb", [6, 20, 64])
-def test_an_error_before_the_product_keeps_psi(nb):
-    """A launch error that is there when psi's turn comes (here one that an
-    invalid device number left behind) is reported, and psi is not multiplied by
-    what an earlier call left in the scratch."""
-    import ctypes
-    import torch
-    roks = built()
-    a = torch.randn((nb, 20000), dtype=torch.complex128, device="cuda")
-    roks.roks_orthonormalize_noalloc(roks.ROKS_FP64, 20000, nb, a, 20000, None)
-    psi = torch.randn((nb, 20000), dtype=torch.complex128, device="cuda")
-    kept = psi.clone()
-    torch.cuda.synchronize()
-    assert ctypes.CDLL("libcudart.so.13").cudaSetDevice(9999) != 0
-    with pytest.raises(roks.RoksError) as ei:
-        roks.roks_orthonormalize_noalloc(roks.ROKS_FP64, 20000, nb, psi, 20000, None)
-    assert ei.value.status == roks.ROKS_ECUDA
-    assert torch.equal(psi, kept)
-    roks.roks_orthonormalize_noalloc(roks.ROKS_FP64, 20000, nb, psi, 20000, None)
-    assert not torch.equal(psi, kept)

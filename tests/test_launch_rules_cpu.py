@@ -1,0 +1,19 @@
+"""CPU: rules of the CUDA sources that no launch on a healthy single GPU shows,
+read from the text of the sources."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_28637_gb300", "csrc")
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return f.read()
+
+
+def test_noalloc_checks_its_launches_before_psi_is_multiplied():
+    """A chain that failed leaves an earlier call's factor in the scratch."""
+    run = source("roks_noalloc.cu")
+    run = run[run.index("cholesky_inverse(nb"):run.index("k_rows_times_upper<T><<<")]
+    assert re.search(r"if \(cudaGetLastError\(\) != cudaSuccess\) return ROKS_ECUDA;", run)
