@@ -12,10 +12,19 @@
 // one, and an absolute error of 2^-40 of that largest one below.  A product
 // is lo.hi + hi.lo + hi.hi.  That is the accuracy of a TF32 split (the same
 // 11-bit significands) at twice the MMA rate and half the operand bytes.
-// The tensor cores' FP32 accumulation truncates, which biases long sums of
-// like-signed terms, so every stage (32 complex K) goes into a fresh
-// tensor-memory accumulator, the small cross terms first, and the drain warps
-// add the stage's result into FP32 sums in registers (round to nearest).
+// The tensor cores' FP32 accumulation truncates, which biases sums of
+// like-signed terms, so a few products go into a fresh tensor-memory
+// accumulator, the small cross terms first, and the drain warps add its result
+// into FP32 sums in registers (round to nearest).  A B: every stage (32 complex
+// K).  A^H B, whose sums are a thousand stages long: every half stage, and no
+// sum in registers goes on for more than GB_PIECE stages.  (Drained by the stage,
+// norms come out 2.3e-7 low; by half stages 0.8e-7, in segments 0.6e-7, 1.2e-7 in
+// the TF32 form.  At mgo-120, errors of F and of a DIIS step's psi: half stages
+// in one sum 1.40e-7 and 1.79e-7, quarter stages, whose longer sums lose more
+// than the shorter accumulations gain, 1.65e-7 and 2.5e-7, half stages in
+// segments 1.11e-7 and 1.50e-7; the TF32 form 1.48e-7 and 2.16e-7.  That takes
+// 1.5% of an apply's time, two thirds of it for the segments.)  Nothing is
+// scaled to give back what is lost: sums without truncation are exact.
 //
 // Images.  A block X (rows x cols, column major) is split once per use, by
 // k_tcg_split, into an image in global memory that the MMAs can read as it
@@ -70,6 +79,7 @@ constexpr int GB_KC = 32;     // complex K per stage
 constexpr int GB_ST = 3;      // stages
 constexpr int GB_ACC = 2;     // accumulators (256 tensor-memory columns each)
 constexpr int GB_DRAIN = 8;   // drain warps
+constexpr int GB_PIECE = 64;  // A^H B: most stages of a running sum (a segment)
 constexpr int GB_THREADS = (4 + GB_DRAIN) * 32;
 constexpr uint32_t GB_ABYTES = GB_M * GB_KC * 8;      // 32 KB
 constexpr uint32_t GB_SLOT = 2 * GB_ABYTES;           // A, then B (tn x KC x 8 bytes)
@@ -100,14 +110,17 @@ __device__ __forceinline__ void give_up(volatile int* failed) {
     g_tcg_timeout = 1;
 }
 
+// segments of so many stages of a tile
+__host__ __device__ constexpr int segments(int stages) { return (stages + GB_PIECE - 1) / GB_PIECE; }
+
 // 2^e as a float, e in [-126, 127]
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
 // CTA-loop schedules, at most one CTA per SM:
 // * A^H B, stream-K: CTA c takes the units c len .. (c + 1) len - 1 of the
 //   (tile, stage) sequence, stage fastest (tile t: M tile t % fast, N tile t /
-//   fast), and writes the partial sums of each tile it touches to its segment
-//   slot c * maxseg + (t - its first tile);
+//   fast), and writes the partial sums of each tile that it touches, a segment
+//   for every GB_PIECE stages of it, to its slots c * maxseg + 0, 1, ...;
 // * A B, persistent: units = tiles, CTA c takes the whole tiles c, c + ctas,
 //   ... (tile t: N tile t % fast, M tile t / fast), its pipeline running on
 //   across them, and writes each tile's result as it completes.
@@ -128,6 +141,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
     __shared__ volatile int failed;
     unsigned char* ring = gb_smem + ((1024u - (tc::smem_u32(gb_smem) & 1023u)) & 1023u);
     const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+    constexpr int DS = NN ? 1 : 2;   // drain steps of a stage
     const int64_t u0 = NN ? 0 : sk.len * blockIdx.x;
     // the first tile and stage (the loops then step them); after a tile's
     // last stage the next tile is t + tstep
@@ -204,44 +218,52 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
             bool ok = true;
             int sl = 0;
             for (int i = 0; i < ns && ok; ++i) {
-                const int b = i % GB_ACC;
-                if (!warp_wait(&full[sl], (uint32_t)((i / GB_ST) & 1), wcap, &failed) ||
-                    (i >= GB_ACC && !warp_wait(&acc_empty[b], (uint32_t)((i / GB_ACC - 1) & 1), wcap, &failed))) {
+                if (!warp_wait(&full[sl], (uint32_t)((i / GB_ST) & 1), wcap, &failed)) {
                     ok = false;
                     break;
                 }
-                tc::fence_after_sync();
                 const uint32_t sa = tc::smem_u32(ring + (size_t)sl * GB_SLOT), sb = sa + GB_ABYTES;
-                const uint32_t d = tmem + (uint32_t)(b * 256);
-                // D(out) += A(part pa, plane xa) B(part pb, plane xb) over the stage's two K-steps of 16
-                auto mm = [&](int out, int pa, int xa, int pb, int xb, bool neg, uint32_t first) {
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk)
-                        tc::mma_f16(d + 128u * out, da0 + ((sa + pa * a_part + xa * a_plane + kk * a_k) >> 4),
-                                    db0 + ((sb + pb * 2 * wb + xb * wb + kk * 8 * wb) >> 4),
-                                    neg ? (idesc | tc::IDESC_NEG_A) : idesc, (first && kk == 0) ? 0u : 1u);
-                };
-                // the small cross terms first, then the hi.hi products, which alone
-                // meet a large partial sum.  CN: re = Ar.Br + Ai.Bi, im = Ar.Bi -
-                // Ai.Br; NN: re = Ar.Br - Ai.Bi, im = Ar.Bi + Ai.Br.  The last
-                // products are those with Br: in A B, where B is near a real
-                // multiple of the identity or has a real diagonal, its large
-                // elements are then truncated least often
-                if (leader) {
-#pragma unroll
-                    for (int o = 0; o < 2; ++o) {
-                        const bool n0 = !NN && o == 1, n1 = NN && o == 0;   // the terms with Br, with Bi
-                        mm(o, 1, 1 - o, 0, 1, n1, 1u);
-                        mm(o, 0, 1 - o, 1, 1, n1, 0u);
-                        mm(o, 1, o, 0, 0, n0, 0u);
-                        mm(o, 0, o, 1, 0, n0, 0u);
-                        mm(o, 0, 1 - o, 0, 1, n1, 0u);
-                        mm(o, 0, o, 0, 0, n0, 0u);
+                for (int h = 0; h < DS; ++h) {
+                    const int e = DS * i + h, b = e % GB_ACC;   // drain step and its accumulator
+                    if (e >= GB_ACC && !warp_wait(&acc_empty[b], (uint32_t)((e / GB_ACC - 1) & 1), wcap, &failed)) {
+                        ok = false;
+                        break;
                     }
-                    tc::commit(&acc_full[b]);
-                    tc::commit(&empty[sl]);   // the slot is free once these MMAs complete
+                    tc::fence_after_sync();
+                    const uint32_t d = tmem + (uint32_t)(b * 256);
+                    // D(out) += A(part pa, plane xa) B(part pb, plane xb) over the step's K-steps of 16
+                    auto mm = [&](int out, int pa, int xa, int pb, int xb, bool neg, uint32_t first) {
+#pragma unroll
+                        for (int k = 0; k < 2 / DS; ++k) {
+                            const int kk = h + k;
+                            tc::mma_f16(d + 128u * out, da0 + ((sa + pa * a_part + xa * a_plane + kk * a_k) >> 4),
+                                        db0 + ((sb + pb * 2 * wb + xb * wb + kk * 8 * wb) >> 4),
+                                        neg ? (idesc | tc::IDESC_NEG_A) : idesc, (first && k == 0) ? 0u : 1u);
+                        }
+                    };
+                    // the small cross terms first, then the hi.hi products, which alone
+                    // meet a large partial sum.  CN: re = Ar.Br + Ai.Bi, im = Ar.Bi -
+                    // Ai.Br; NN: re = Ar.Br - Ai.Bi, im = Ar.Bi + Ai.Br.  The last
+                    // products are those with Br: in A B, where B is near a real
+                    // multiple of the identity or has a real diagonal, its large
+                    // elements are then truncated least often
+                    if (leader) {
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) {
+                            const bool n0 = !NN && o == 1, n1 = NN && o == 0;   // the terms with Br, with Bi
+                            mm(o, 1, 1 - o, 0, 1, n1, 1u);
+                            mm(o, 0, 1 - o, 1, 1, n1, 0u);
+                            mm(o, 1, o, 0, 0, n0, 0u);
+                            mm(o, 0, o, 1, 0, n0, 0u);
+                            mm(o, 0, 1 - o, 0, 1, n1, 0u);
+                            mm(o, 0, o, 0, 0, n0, 0u);
+                        }
+                        tc::commit(&acc_full[b]);
+                        if (h == DS - 1) tc::commit(&empty[sl]);   // the slot is free once these MMAs complete
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
                 sl = sl == GB_ST - 1 ? 0 : sl + 1;
             }
             if (!ok) give_up(&failed);
@@ -257,24 +279,14 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
         const int q = warp & 3;               // lane quadrant
         const int cg = 64 * ((warp - 4) >> 2);   // complex columns cg .. cg + 63
         const int r = 32 * q + lane;          // tile row
-        // What the truncating additions of a stage take from its sum, given
-        // back (A^H B: alpha is the factor).  The norms of A^H A, sums of
-        // like sign, lose 2.3e-7 of their size (11,075 plane waves; four
-        // additions of half a unit in the last place each, and those inside an
-        // MMA), nearly 2^-22; P^H Psi, whose signs mix, half of it: with 2^-23
-        // the nonlocal energy of organic-96 and mgo-72 is -1.6e-6 and -1.6e-5 Ha
-        // off, with 2^-22 -1.6e-5 and -7.5e-5, without 1.4e-5 and 4.5e-5 (FP32
-        // sums: 1.2e-6 and 4.9e-5).  The products with the small B of A B lose no
-        // measurable part.
-        const float gain = NN ? 1.f : alpha;
         float2 re[32], im[32];                // column pairs
 #pragma unroll
         for (int j = 0; j < 32; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
         bool ok = true;
-        int left = total_stages - s_first, seg = 0, t_cur = t_first;
-        for (int i = 0; i < ns; ++i) {
-            const int b = i % GB_ACC;
-            if (!warp_wait(&acc_full[b], (uint32_t)((i / GB_ACC) & 1), wcap, &failed)) {
+        int left = total_stages - s_first, seg = 0, in_seg = 0, t_cur = t_first;
+        for (int e = 0; e < DS * ns; ++e) {
+            const int b = e % GB_ACC;
+            if (!warp_wait(&acc_full[b], (uint32_t)((e / GB_ACC) & 1), wcap, &failed)) {
                 ok = false;
                 break;
             }
@@ -296,18 +308,20 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float2 g2 = make_float2(gain, gain);
-                        re[8 * c + j] = __ffma2_rn(make_float2(v[2 * j], v[2 * j + 1]), g2, re[8 * c + j]);
-                        im[8 * c + j] = __ffma2_rn(make_float2(w[2 * j], w[2 * j + 1]), g2, im[8 * c + j]);
+                        re[8 * c + j] = __fadd2_rn(re[8 * c + j], make_float2(v[2 * j], v[2 * j + 1]));
+                        im[8 * c + j] = __fadd2_rn(im[8 * c + j], make_float2(w[2 * j], w[2 * j + 1]));
                     }
                 }
             }
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&acc_empty[b]);
-            // the last stage of a tile in this CTA's run: its sums go out (NN:
-            // the result; CN: the partial sums to the segment slot) and restart
-            if (--left == 0 || i == ns - 1) {
+            if (DS > 1 && e % DS < DS - 1) continue;
+            // the last stage of a tile (CN: or of a segment) in this CTA's run: its
+            // sums go out (NN: the result; CN: the partial sums to the segment
+            // slot) and restart
+            --left;
+            if (left == 0 || e == DS * ns - 1 || (!NN && ++in_seg == GB_PIECE)) {
                 if (NN) {
                     const int m = (t_cur / sk.fast) * GB_M + r;
                     const int no = (t_cur % sk.fast) * sk.tn + cg;
@@ -350,8 +364,11 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
 #pragma unroll
                 for (int j = 0; j < 32; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
                 ++seg;
-                t_cur += tstep;
-                left = total_stages;
+                in_seg = 0;
+                if (left == 0) {
+                    t_cur += tstep;
+                    left = total_stages;
+                }
             }
         }
         if (!ok) give_up(&failed);
@@ -504,7 +521,8 @@ bool launch_split(int R, int V, const D* X, int64_t ld, const int* exA, const Tc
 
 // ------------------------------------------------------------------ partial sums
 // C (M x N, FP64) of tile t: the segments of the CTAs whose runs meet the
-// tile's units t T .. (t + 1) T - 1.  A warp covers 32 rows of one column; RG
+// tile's units t T .. (t + 1) T - 1 (one each where runs are short, else one for
+// every GB_PIECE stages).  A warp covers 32 rows of one column; RG
 // warps of a block take every RG-th CTA of the tile, the block's other warps
 // further columns.  Compensated FP32 sums (FP64 arithmetic is slow on this
 // part), combined in warp order; the operands' scales come out at the end.
@@ -529,13 +547,30 @@ __global__ void __launch_bounds__(256) k_tcg_reduce_sk(int M, int N, int mt, int
         const int64_t off = (int64_t)(n % sk.tn) * GB_M + (m % GB_M);
         const int64_t ta = (int64_t)t * T;
         const int c0 = (int)(ta / sk.len), c1 = (int)((ta + T - 1) / sk.len);
+        if (sk.len <= GB_PIECE) {
 #pragma unroll 4
-        for (int c = c0 + wg; c <= c1; c += RG) {
-            // a run that starts before the tile has it further on
-            const int seg = c == c0 ? t - (int)(c0 * sk.len / T) : 0;
-            const float2 p = part[((int64_t)c * sk.maxseg + seg) * sk.tn * GB_M + off];
-            add(sx, cx, p.x);
-            add(sy, cy, p.y);
+            for (int c = c0 + wg; c <= c1; c += RG) {
+                // a run that starts before the tile has it further on
+                const int seg = c == c0 ? t - (int)(c0 * sk.len / T) : 0;
+                const float2 p = part[((int64_t)c * sk.maxseg + seg) * sk.tn * GB_M + off];
+                add(sx, cx, p.x);
+                add(sy, cy, p.y);
+            }
+        } else {
+            for (int c = c0 + wg; c <= c1; c += RG) {
+                // the segments of the run's tiles before this one, then this one's
+                const int64_t u0 = c * sk.len;
+                const int tb = (int)(u0 / T), sb = (int)(u0 - (int64_t)tb * T);
+                const int seg = tb < t ? segments(T - sb) + (t - tb - 1) * segments(T) : 0;
+                const int ns = segments((int)(min(u0 + sk.len, ta + T) - max(u0, ta)));
+                const float2* p = part + ((int64_t)c * sk.maxseg + seg) * sk.tn * GB_M + off;
+#pragma unroll 4
+                for (int q = 0; q < ns; ++q, p += sk.tn * GB_M) {
+                    const float2 v = *p;
+                    add(sx, cx, v.x);
+                    add(sy, cy, v.y);
+                }
+            }
         }
     }
     if constexpr (RG > 1) {
@@ -600,7 +635,9 @@ SkPlan cn_plan(int M, int N, int K, int waves_x2) {
     p.ctas = (int)std::min<int64_t>(sm_count() * waves_x2 / 2, std::max<int64_t>(1, p.units / 4));
     p.len = (p.units + p.ctas - 1) / p.ctas;
     p.ctas = (int)((p.units + p.len - 1) / p.len);
-    p.maxseg = (int)((p.len + T - 1) / T) + 1;
+    // (long runs: whole tiles, what is left over, and a short segment at either end)
+    p.maxseg = p.len <= GB_PIECE ? (int)((p.len + T - 1) / T) + 1
+                                 : (int)(p.len / T) * segments(T) + (int)(p.len % T) / GB_PIECE + 3;
     return p;
 }
 
@@ -750,8 +787,7 @@ bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2
     const int T = stages(K);
     float2* part = reinterpret_cast<float2*>(w);
     k_tcgemm<false><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, T, sk, tmA, tmB, nullptr, part, nullptr, 0, nullptr, 0,
-                                                          same ? 1.f + 0x1p-22f : 1.f + 0x1p-23f, 0.f,
-                                                          wait_polls());
+                                                          1.f, 0.f, wait_polls());
     roks::count_launch();
     const int mt = (M + GB_M - 1) / GB_M;
     // many CTAs per tile: their segments shared out over the warps of a block
