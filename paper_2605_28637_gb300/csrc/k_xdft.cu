@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(256, 2) k_xdft_density(int nmax, const __grid_
                                                          DensAcc<float>::S* __restrict__ rho3,
                                                          DensAcc<float>::S* __restrict__ slot,
                                                          const uint4* __restrict__ tab, int b0, int nbb, int gs,
-                                                         int n_closed, float scale, int cls_override,
+                                                         int n_closed, float2 scale, int cls_override,
                                                          int* __restrict__ timeout, uint32_t wcap) {
     using DA = DensAcc<float>;
     constexpr int NN = N * N;
@@ -467,8 +467,8 @@ __global__ void __launch_bounds__(256, 2) k_xdft_density(int nmax, const __grid_
                 for (int k = 0; k < 8; ++k) {
                     const int kk = 4 * q + (k >> 1);
                     const float2 v2 = (k & 1) ? sm[kk >> 1] : sp[kk >> 1];
-                    const float u = (kk & 1) ? v2.y : v2.x, v = u * scale;
-                    const DA::S inc = make_float2(v, fmaf(u, scale, -v) + XD_LOSS * v);
+                    const float u = (kk & 1) ? v2.y : v2.x, v = u * scale.x;
+                    const DA::S inc = make_float2(v, fmaf(u, scale.y, fmaf(u, scale.x, -v)) + XD_LOSS * v);
                     const int e = at(k);
                     if (e >= 0) dst[e * NN] = add ? DA::add2(old[k], inc) : inc;
                 }
@@ -648,8 +648,11 @@ void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, c
 }
 
 void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rho3, double* slot, int gs, int ng,
-                  int b0, int nbb, int n_closed, float scale, int cls_override, cudaStream_t st) {
+                  int b0, int nbb, int n_closed, double scale, int cls_override, cudaStream_t st) {
     using DS = DensAcc<float>::S;
+    // (in two words: rounded to one, it moves every density the same way, by up
+    // to 6e-8; 4.3e-8 at mgo-120)
+    const float2 sc = make_float2((float)scale, (float)(scale - (double)(float)scale));
     const dim3 grid((s.N * s.N + 127) / 128, ng);
     CUtensorMap tm{};
     const bool staged = xd_smem(s.nmax, true) <= XD_SMEM_HALF && plane_map(&tm, s, Yp, nbb);
@@ -658,7 +661,7 @@ void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rh
         xd_attr(kernel, sm);
         roks::count_launch(), kernel<<<grid, 256, sm, st>>>(
                                   s.nmax, tm, Yp, reinterpret_cast<DS*>(rho3), reinterpret_cast<DS*>(slot),
-                                  static_cast<const uint4*>(tab), b0, nbb, gs, n_closed, scale, cls_override,
+                                  static_cast<const uint4*>(tab), b0, nbb, gs, n_closed, sc, cls_override,
                                   tcg_timeout_flag(), wait_polls());
     };
     XD_DISPATCH(s.N, XD_PICK(k_xdft_density));

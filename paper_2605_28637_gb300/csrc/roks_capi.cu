@@ -339,7 +339,7 @@ struct Impl {
         if constexpr (sizeof(T) == 4) {
             if (ctx->d_xtab && part_sel == 0 && nbb > 0) {
                 const int gs = (nbb + ngroups - 1) / ngroups, ng = (nbb + gs - 1) / gs;
-                xdft_density(s, ctx->d_xtab, Yp, rho3, slot, gs, ng, b0, nbb, n_closed, (float)scale, cls_override,
+                xdft_density(s, ctx->d_xtab, Yp, rho3, slot, gs, ng, b0, nbb, n_closed, scale, cls_override,
                              ctx->st);
                 if (slot) band_density_reduce<T>(ctx->N, ng, slot, rho3, ctx->st);
                 return;

@@ -145,7 +145,7 @@ void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, c
                 int n_closed, float scale, cudaStream_t st);
 // band_x_density of |psi|^2 without the sum of the slots; bands in ng groups of gs
 void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rho3, double* slot, int gs, int ng,
-                  int b0, int nbb, int n_closed, float scale, int cls_override, cudaStream_t st);
+                  int b0, int nbb, int n_closed, double scale, int cls_override, cudaStream_t st);
 
 // ------------------------------------------------------------ Gamma point (k_gamma.cu)
 // Real orbitals are stored on the half sphere (G = 0 and the Miller triples
