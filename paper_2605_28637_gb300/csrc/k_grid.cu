@@ -645,7 +645,8 @@ void potentials(int N, double L, const double* rho3, const T* vloc, const PotCoe
     a.partA = part;
     a.partB = part + 4 * kPotBlocks;
     a.partC = a.partB + kPotBlocks;
-    a.vmax = vmax;
+    // (cleared on the way to its maximum: with the potentials it bounds, or not at all)
+    a.vmax = energies_only ? nullptr : vmax;
     c2<T>* gg = gga ? static_cast<c2<T>*>(gga->gg) : nullptr;
     c2<T>* dd = gga ? static_cast<c2<T>*>(gga->dd) : nullptr;
     int na = kPotBlocks;

@@ -17,3 +17,13 @@ def test_noalloc_checks_its_launches_before_psi_is_multiplied():
     run = source("roks_noalloc.cu")
     run = run[run.index("cholesky_inverse(nb"):run.index("k_rows_times_upper<T><<<")]
     assert re.search(r"if \(cudaGetLastError\(\) != cudaSuccess\) return ROKS_ECUDA;", run)
+
+
+def test_the_potentials_bound_is_cleared_only_where_they_are_written():
+    """An energies-only call keeps the potentials, and must keep their bound,
+    from which the apply takes its scale: the plane pass clears it."""
+    grid = source("k_grid.cu")
+    body = grid[grid.index("void potentials(int N"):]
+    body = body[:body.index("\n}\n")]
+    assert re.search(r"a\.vmax = energies_only \? nullptr : vmax;", body)
+    assert len(re.findall(r"\bvmax\b", body)) == 3       # the parameter and that line
