@@ -308,12 +308,7 @@ size_t cn_smem_max() {
 
 template <typename T, int RM, int RN>
 void cn_attr() {
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(k_gemm_cn<T, RM, RN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cn_smem_max<T, RM, RN>());
-        done = true;
-    }
+    allow_smem(k_gemm_cn<T, RM, RN>, cn_smem_max<T, RM, RN>());
 }
 
 // Blocks of the chosen contraction kernel resident on one SM (occupancy API),
@@ -595,11 +590,7 @@ template <typename T, int RN, int RM>
 void launch_nn(int M, int N, int K, int ty, int nt, const c2<T>* A, int64_t lda, const c2<T>* B, int ldb, c2<T>* C,
                int64_t ldc, T alpha, T beta, cudaStream_t st) {
     const size_t smem = sizeof(c2<T>) * (2 * NN_KT * (32 * RM + 8 * RN + 1) + (size_t)(8 * RN) * (32 * RM));
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_gemm_nn<T, RM, RN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    allow_smem(k_gemm_nn<T, RM, RN>, smem);
     dim3 g((M + 32 * RM - 1) / (32 * RM), nt);
     roks::count_launch();
     k_gemm_nn<T, RM, RN><<<g, 32 * ty, smem, st>>>(M, N, K, ty, A, lda, B, ldb, C, ldc, alpha, beta);
@@ -1084,16 +1075,17 @@ __global__ void __launch_bounds__(1024) k_cholesky_dev_f32(int n, const double2*
     }
 }
 
+static constexpr size_t chol_dev_smem(int n) { return sizeof(float2) * 2 * n * n + sizeof(int) * n * (n - 1) / 2; }
+constexpr size_t kCholDevSmem = chol_dev_smem(kSmallN);
+
 void cholesky_dev_f32(int n, const double2* O, double2* XiH, int* flag, cudaStream_t st) {
-    const size_t sm = sizeof(float2) * 2 * n * n + sizeof(int) * n * (n - 1) / 2;
+    const size_t sm = chol_dev_smem(n);
     roks::count_launch();
     if (n * (n - 1) / 2 <= 4 * kCholFactorThreads) {
-        if (sm > 48 * 1024)
-            cudaFuncSetAttribute(k_cholesky_dev_f32<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_smem(k_cholesky_dev_f32<4>, kCholDevSmem);
         k_cholesky_dev_f32<4><<<1, 1024, sm, st>>>(n, O, XiH, flag);
     } else {
-        if (sm > 48 * 1024)
-            cudaFuncSetAttribute(k_cholesky_dev_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_smem(k_cholesky_dev_f32<8>, kCholDevSmem);
         k_cholesky_dev_f32<8><<<1, 1024, sm, st>>>(n, O, XiH, flag);
     }
 }
@@ -1495,12 +1487,7 @@ bool expm_small_f32(int n, const double2* A, const double* scale_dev, double2* E
     if (n > kSmallN) return false;
     const int ldm = (n + 1) & ~1;
     const size_t sm = sizeof(float2) * 5 * ldm * ldm;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_expm_small_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float2) * 5 * kSmallN * kSmallN));
-        attr = true;
-    }
+    allow_smem(k_expm_small_f32, sizeof(float2) * 5 * kSmallN * kSmallN);
     roks::count_launch(), k_expm_small_f32<<<kExpmCluster, kExpmThreads, sm, st>>>(n, A, scale_dev, E);
     return true;
 }
@@ -1509,12 +1496,7 @@ void expm_scaled(int n, const double2* A, const double* scale_dev, double2* E, d
                  double2* w3, double* sdev, cudaStream_t st) {
     if (n <= kExpmF64N) {
         const size_t sm = sizeof(double2) * 6 * n * n;
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(k_expm_small_f64<kExpmCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(double2) * 6 * kExpmF64N * kExpmF64N));
-            attr = true;
-        }
+        allow_smem(k_expm_small_f64<kExpmCluster>, sizeof(double2) * 6 * kExpmF64N * kExpmF64N);
         roks::count_launch();
         if (n <= 12) k_expm_small_f64<1><<<1, kExpmThreads, sm, st>>>(n, A, scale_dev, E);
         else k_expm_small_f64<kExpmCluster><<<kExpmCluster, kExpmThreads, sm, st>>>(n, A, scale_dev, E);

@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(plane_threads(N)) k_grid_plane(const c2<T>* __
 // ------------------------------------------------------------------ launchers
 template <typename K>
 static void set_smem(K kernel, size_t bytes) {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    allow_smem(kernel, bytes);
 }
 
 template <typename T, int N>

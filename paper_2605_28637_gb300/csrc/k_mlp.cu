@@ -584,11 +584,7 @@ void mlp_grad(int n, const float* U, const float* t, const float* w, const float
     const int nblk = (n + GB - 1) / GB;
     if (nblk <= 0) return;
     const size_t sm = grad_smem();
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_mlp_grad_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        attr = true;
-    }
+    allow_smem(k_mlp_grad_partial, sm);
     roks::count_launch(), k_mlp_grad_partial<<<nblk, GT, sm, st>>>(n, U, t, w, params, work);
     roks::count_launch(), k_mlp_grad_reduce<<<(kMlpParams + 1 + 31) / 32, 32 * RW, 0, st>>>(nblk, work, grad, loss);
 }

@@ -494,11 +494,6 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // polls of the work-loop waits of the next launches (set_wait_cap)
 uint32_t g_wait_polls = ST_WAIT;
 
-template <typename F>
-void set_smem(F* f, size_t bytes) {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 // Tiled map of 64-bit words, dims[0] contiguous, strides (bytes) of the others
@@ -609,11 +604,7 @@ bool gemm_cn_stream(int M, int N, int K, const float2* A, int64_t lda, const flo
     float2* part = reinterpret_cast<float2*>(work);
 #define CNS_CASE(RM_, RN_, KS_)                                                                            \
     if (cands[best].rm == RM_ && cands[best].rn == RN_ && ks == KS_) {                                    \
-        static bool attr = false;                                                                          \
-        if (!attr) {                                                                                       \
-            set_smem(k_cn_stream<RM_, RN_, KS_>, ST_SMEM);                                                 \
-            attr = true;                                                                                   \
-        }                                                                                                  \
+        allow_smem(k_cn_stream<RM_, RN_, KS_>, ST_SMEM);                                                   \
         roks::count_launch();                                                                              \
         k_cn_stream<RM_, RN_, KS_><<<G, threads, smem, st>>>(M, N, K, rows, ty, tx, NS, tmA, tmB, part,      \
                                                              g_wait_polls);                                 \
@@ -691,11 +682,7 @@ bool gemm_nn_stream(int M, int N, int K, const float2* A, int64_t lda, const dou
     const int threads = 32 * (W * WS + 1);
 #define NNS_CASE(RR_, RN_, WS_)                                                                              \
     if (RR == RR_ && RN == RN_ && WS == WS_) {                                                              \
-        static bool attr = false;                                                                           \
-        if (!attr) {                                                                                        \
-            set_smem(k_nn_stream<RR_, RN_, WS_>, ST_SMEM);                                                  \
-            attr = true;                                                                                    \
-        }                                                                                                   \
+        allow_smem(k_nn_stream<RR_, RN_, WS_>, ST_SMEM);                                                    \
         roks::count_launch();                                                                               \
         k_nn_stream<RR_, RN_, WS_><<<G, threads, smem, st>>>(M, N, K, KC, nkc, rows, W, NS, load_c ? 1 : 0,  \
                                                              tmA, tmC, Bf, convert_in ? B : nullptr, ldb,   \

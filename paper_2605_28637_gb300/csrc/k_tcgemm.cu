@@ -606,15 +606,6 @@ int sm_count() {
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
-template <bool NN>
-void set_attr() {
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(k_tcgemm<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GB_SMEM);
-        done = true;
-    }
-}
-
 int stages(int k) { return (k + GB_KC - 1) / GB_KC; }
 int tile_cols(int N, int nt) { return ((N + nt - 1) / nt + 15) / 16 * 16; }
 
@@ -783,7 +774,7 @@ bool gemm_cn_tcg(int M, int N, int K, const float2* A, int64_t lda, const float2
     if (!ib && !same && !tcg_split(mb, B, ldb, st)) return false;
     roks::count_launch();
     g_tcg_launches += 1;
-    set_attr<false>();
+    allow_smem(k_tcgemm<false>, GB_SMEM);
     const int T = stages(K);
     float2* part = reinterpret_cast<float2*>(w);
     k_tcgemm<false><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, T, sk, tmA, tmB, nullptr, part, nullptr, 0, nullptr, 0,
@@ -824,7 +815,7 @@ bool gemm_nn_tcg(int M, int N, int K, const float2* A, int64_t lda, const double
     if (!launch_split<double2, false>(K, N, B, ldb, ma.ex, mb, st)) return false;
     roks::count_launch();
     g_tcg_launches += 1;
-    set_attr<true>();
+    allow_smem(k_tcgemm<true>, GB_SMEM);
     k_tcgemm<true><<<sk.ctas, GB_THREADS, GB_SMEM, st>>>(M, N, stages(K), sk, tmA, tmB, mb.ex, nullptr, Cin, ldcin,
                                                          Cout, ldc, alpha, beta, wait_polls());
     return true;

@@ -573,11 +573,6 @@ int xd_sms() {
     return n;
 }
 
-template <typename K>
-void xd_attr(K kernel, size_t bytes) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 // The grids whose kernels are instantiated, as far as their densities fit
@@ -639,7 +634,7 @@ void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, c
     const bool staged = xd_smem(s.nmax, true) <= XD_SMEM_HALF && plane_map(&tm, s, Yp, nbb);
     const size_t sm = xd_smem(s.nmax, staged);
     auto go = [&](auto kernel) {
-        xd_attr(kernel, sm);
+        allow_smem(kernel, XD_SMEM_HALF);
         roks::count_launch(), kernel<<<grid, 256, sm, st>>>(s.nmax, tm, Yp, Vk, vmax, static_cast<const uint4*>(tab),
                                                             b0, nbb, n_closed, scale, tcg_timeout_flag(),
                                                             wait_polls());
@@ -658,7 +653,7 @@ void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rh
     const bool staged = xd_smem(s.nmax, true) <= XD_SMEM_HALF && plane_map(&tm, s, Yp, nbb);
     const size_t sm = xd_smem(s.nmax, staged);
     auto go = [&](auto kernel) {
-        xd_attr(kernel, sm);
+        allow_smem(kernel, XD_SMEM_HALF);
         roks::count_launch(), kernel<<<grid, 256, sm, st>>>(
                                   s.nmax, tm, Yp, reinterpret_cast<DS*>(rho3), reinterpret_cast<DS*>(slot),
                                   static_cast<const uint4*>(tab), b0, nbb, gs, n_closed, sc, cls_override,

@@ -205,10 +205,7 @@ roks_status run(int npw, int nb, void* psi, int64_t ld, cudaStream_t st, unsigne
     // earlier call's L^{-H} otherwise
     if (cudaGetLastError() != cudaSuccess) return ROKS_ECUDA;
     const size_t sm = sizeof(V) * ((size_t)nb * 64 + (size_t)nb * nb);
-    if (sm > 48 * 1024 &&
-        cudaFuncSetAttribute(k_rows_times_upper<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-            cudaSuccess)
-        return ROKS_ECUDA;
+    if (allow_smem(k_rows_times_upper<T>, sizeof(V) * kNaMaxBands * (64 + kNaMaxBands)) != cudaSuccess) return ROKS_ECUDA;
     count_launch();
     k_rows_times_upper<T><<<(npw + 63) / 64, 256, sm, st>>>(npw, nb, X, ld, LinvH, flag);
     return result(flag, st);
