@@ -348,11 +348,14 @@ int cn_resident_blocks(int rm, int rn, int threads, size_t smem) {
 }
 
 // Register tile and thread grid with the least padded work (plus the
-// shared-memory loads per multiply-add; in long FP64 sums, where the pipes of
-// the SM's four parts set the time, threads short of a multiple of four warps
-// count as work: 172 x 42 over 34,265 rows with 210 threads a block 2.67 ms, with
-// 126 1.76; over 1050 rows the partials of smaller tiles cost more: a tiny-16
-// PCG step 569 us, 607 with them), then K chunks for whole waves of
+// shared-memory loads per multiply-add), and no fewer than 64 threads where that
+// can be had.  In long FP64 sums the pipes of the SM's four parts set the time,
+// and a lane that idles in its warp, or a warp in a block's last round of four,
+// costs what a busy one does, as does an SM without a block where the chunks are
+// limited: there the work is charged by lanes issued, and smaller tiles may be
+// taken (172 x 42 over 34,265 rows, 210 threads a block 2.67 ms, 126 1.76; over
+// 1050 rows the partials of smaller tiles cost more: a tiny-16 PCG step 569 us,
+// 607 with them).  Then K chunks for whole waves of
 // resident blocks, each at least two K slices long.  FP64 products are bound
 // by the pipe of the SMs that take part (two multiply-adds a cycle each), so
 // their chunks go down to half a slice, up to as many as there are SMs: 44 x 6
@@ -378,8 +381,14 @@ CnPlan cn_plan(int M, int N, int K, int max_chunks) {
                     const int ty = (M + mt * rm - 1) / (mt * rm), tx = (N + nt * rn - 1) / (nt * rn);
                     const double covered = (double)mt * ty * rm * nt * tx * rn;
                     double cost = covered * (1.0 + (rm + rn) / (4.0 * rm * rn));
-                    if (ty * tx < 64) cost *= 1.5;   // too few threads per block to hide latency
-                    else if (pipes) cost *= (ty * tx + 127) / 128 * 128.0 / (ty * tx);
+                    if (pipes) {
+                        const double per_sm = max_chunks > 0 ? (double)mt * nt * max_chunks / sm_count() : 2.0;
+                        const int step = per_sm >= 1.0 && ty * tx <= 128 ? 32 : 128;
+                        cost *= (double)((ty * tx + step - 1) / step * step) / (ty * tx);
+                        if (per_sm < 1.0) cost /= per_sm;   // SMs without a block
+                    }
+                    // too few threads per block to hide latency
+                    if (ty * tx < 64) cost *= pipes && M * N >= 64 ? 4.0 : 1.5;
                     if (cost < best_cost) {
                         best_cost = cost;
                         best = CnPlan{rm, rn, ty, tx, mt, nt, 0, 0};
