@@ -618,14 +618,16 @@ void gemm_nn(int M, int N, int K, const c2<T>* A, int64_t lda, const double2* B,
             return;
     }
     // Column tiles of at most 64: RN = ceil(tile / 8) columns per thread, TY <= 8
-    // warps.  Where tiles of 128 rows leave SMs idle the rows go down to 32 and
-    // the columns are split, as long as SMs are free (FP64 runs at the pipe of
-    // the SMs that take part: 1050 x 6 x 44 on 9 blocks 16.8 us, on 198 6.6;
-    // 4000 x 48 x 200 785 and 202).  Short FP32 sums are bound by latency either
+    // warps.  Where tiles of 128 rows leave a quarter of the SMs idle the rows go
+    // down to 32 and the columns are split, as long as SMs are free (FP64 runs at
+    // the pipe of the SMs that take part: 1050 x 6 x 44 on 9 blocks 16.8 us, on 198
+    // 6.6; 3407 x 24 x 84 on 27 blocks 600, split 159; 9795 x 24 x 84 on 77 602 and
+    // 450, 12197 on 96 602 and 455; on 119 blocks 601 and 597, and with 8 columns
+    // and 28 terms 81 and 84).  Short FP32 sums are bound by latency either
     // way and keep the fewer blocks (a DIIS step of 12 bands 430 us, 435 split;
     // a PCG step of 53 bands, 150 projectors: 1070 us, 916 split).
     int nt = (N + 63) / 64;
-    const bool low = (sizeof(T) == 8 || K >= 48) && (int64_t)((M + 127) / 128) * nt < sm_count();
+    const bool low = (sizeof(T) == 8 || K >= 48) && (int64_t)((M + 127) / 128) * nt < 3 * sm_count() / 4;
     while (low && nt < N && (int64_t)((M + 31) / 32) * nt < sm_count()) nt = std::min(N, 2 * nt);
     const int tn = (N + nt - 1) / nt;
     nt = (N + tn - 1) / tn;
