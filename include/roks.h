@@ -173,7 +173,7 @@ typedef struct {
                           the band transforms and keeps the fastest          */
     int exx_kernel;    /* ROKS_EXX_TRUNCATED (0) or ROKS_EXX_BARE            */
     int wait_cap;      /* polls of every bounded device wait (mbarrier waits
-                          of the streamed and tensor-core contractions) before
+                          of the streamed and tensor-core kernels) before
                           it gives up with ROKS_ETIMEOUT; 0: 2^26; < 0: no
                           poll at all, so every such wait gives up (a test of
                           the timeout path).  Copies already in flight are

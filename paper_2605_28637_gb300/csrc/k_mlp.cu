@@ -70,7 +70,7 @@ __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 // per SM.  34,265 plane waves x 42 bands: 464 -> 247 us with the column sums.
 constexpr int NT = 128;                       // rows (and threads) of a block
 constexpr uint32_t NET_COLS = 128;            // A hi 0..31, A lo 32..63, D 64..127
-constexpr uint32_t NET_WAIT = 1u << 24;       // polls before a wait gives up
+constexpr uint32_t NET_WAIT = 1u << 26;       // polls before a wait is given up for good
 constexpr size_t NET_PAD = 27 * 1024;         // dynamic shared memory that keeps a fifth block off the SM
 
 struct NetShared {
@@ -124,9 +124,11 @@ __device__ __forceinline__ void net_setup(NetShared& S, const float* __restrict_
 }
 
 // Network output for every thread's row; phase counts the calls.  FULL: W2
-// has a low part.  ok is cleared (for the whole block) if the wait ran out.
+// has a low part.  A wait that runs out (wcap polls) sets the contractions' flag
+// and goes on with the default bound; ok is cleared if that runs out too.
 template <bool FULL>
-__device__ __forceinline__ float net_eval(NetShared& S, float u0, float u1, float u2, uint32_t phase, bool& ok) {
+__device__ __forceinline__ float net_eval(NetShared& S, float u0, float u1, float u2, uint32_t phase, bool& ok,
+                                          int* timeout, uint32_t wcap) {
     const uint32_t tm = S.tmem, lanes = (threadIdx.x & 96u) << 16;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
@@ -167,7 +169,11 @@ __device__ __forceinline__ float net_eval(NetShared& S, float u0, float u1, floa
         for (int kk = 0; kk < 4; ++kk) tc::mma_f16_ta(tm + 64, tm + 8 * kk, bh + 128 * kk, idesc, 1);
         tc::commit(&S.bar);
     }
-    ok = tc::mbar_wait(&S.bar, phase & 1u, NET_WAIT);
+    ok = tc::mbar_wait(&S.bar, phase & 1u, wcap);
+    if (!ok) {
+        if (timeout) *timeout = 1;
+        ok = tc::mbar_wait(&S.bar, phase & 1u, NET_WAIT);
+    }
     tc::fence_after_sync();
     float s = S.b3;
     const float2 un = f2(S.unscale);
@@ -199,7 +205,8 @@ __device__ __forceinline__ void net_done(NetShared& S) {
 
 template <bool FULL>
 __global__ void __launch_bounds__(NT) k_mlp_forward(int n, const float* __restrict__ U,
-                                                    const float* __restrict__ params, float* __restrict__ s) {
+                                                    const float* __restrict__ params, float* __restrict__ s,
+                                                    int* timeout) {
     __shared__ __align__(128) NetShared S;
     net_setup(S, params, !FULL);
     bool ok = true;
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(NT) k_mlp_forward(int n, const float* __restri
     for (int i0 = blockIdx.x * NT; i0 < n; i0 += gridDim.x * NT, ++phase) {
         const int i = i0 + threadIdx.x;
         const float* u = U + 3 * (int64_t)min(i, n - 1);
-        const float v = net_eval<FULL>(S, u[0], u[1], u[2], phase, ok);
+        const float v = net_eval<FULL>(S, u[0], u[1], u[2], phase, ok, timeout, NET_WAIT);
         if (i < n) s[i] = ok ? v : __int_as_float(0x7fffffff);
     }
     net_done(S);
@@ -487,7 +494,8 @@ __global__ void __launch_bounds__(NT) k_precond_mlp(int npw, const c2<T>* __rest
                                                     int nb, const double2* __restrict__ Theta,
                                                     const double* __restrict__ wband,
                                                     const float* __restrict__ params, const PcgScalars* sc,
-                                                    c2<T>* __restrict__ out, int64_t ldo) {
+                                                    c2<T>* __restrict__ out, int64_t ldo, int* timeout,
+                                                    uint32_t wcap) {
     __shared__ __align__(128) NetShared S;
     __shared__ float band[5];   // 1/X, -2/X, 1/T, 1/rms, eps
     const bool use = params != nullptr && (sc == nullptr || sc->mlp_off <= 0.0);
@@ -525,7 +533,8 @@ __global__ void __launch_bounds__(NT) k_precond_mlp(int npw, const c2<T>* __rest
         float K = band[1] * num / (num + 16.f * x * x * x * x);
         if (use) {
             const float amp = sqrtf(float(a.x) * float(a.x) + float(a.y) * float(a.y));
-            const float s = net_eval<false>(S, log1pf(gh * band[2]), log1pf(amp * band[3]), band[4], phase++, ok);
+            const float s = net_eval<false>(S, log1pf(gh * band[2]), log1pf(amp * band[3]), band[4], phase++, ok,
+                                            timeout, wcap);
             K *= ok ? expf(fminf(fmaxf(s, -3.f), 3.f)) : __int_as_float(0x7fffffff);
         }
         if (g < npw) out[(int64_t)n * ldo + g] = mk<T>(T(K) * a.x, T(K) * a.y);
@@ -573,8 +582,8 @@ void mlp_forward(int n, const float* U, const float* params, bool bf16, float* s
     if (n <= 0) return;
     const int blocks = net_blocks((n + NT - 1) / NT);
     roks::count_launch();
-    if (bf16) k_mlp_forward<false><<<blocks, NT, NET_PAD, st>>>(n, U, params, s);
-    else k_mlp_forward<true><<<blocks, NT, NET_PAD, st>>>(n, U, params, s);
+    if (bf16) k_mlp_forward<false><<<blocks, NT, NET_PAD, st>>>(n, U, params, s, tcg_timeout_flag());
+    else k_mlp_forward<true><<<blocks, NT, NET_PAD, st>>>(n, U, params, s, tcg_timeout_flag());
 }
 
 size_t mlp_grad_work_floats(int n) { return (size_t)((n + GB - 1) / GB) * (kMlpParams + 2); }
@@ -602,7 +611,8 @@ void precondition_mlp(int npw, int nb, const c2<T>* gI, int64_t ld, const T* g2h
                       const double2* Theta, const double* wband, const float* params, const PcgScalars* sc,
                       c2<T>* out, int64_t ldo, cudaStream_t st) {
     roks::count_launch(), k_precond_mlp<T><<<net_blocks((int64_t)((npw + NT - 1) / NT) * nb), NT, NET_PAD, st>>>(
-                              npw, gI, ld, g2h, sums, nb, Theta, wband, params, sc, out, ldo);
+                              npw, gI, ld, g2h, sums, nb, Theta, wband, params, sc, out, ldo, tcg_timeout_flag(),
+                              wait_polls());
 }
 
 template <typename T>

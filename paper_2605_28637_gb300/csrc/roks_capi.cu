@@ -1616,10 +1616,10 @@ roks_status roks_setup(const roks_cell* cell, double ecut, int natoms, const rok
         cudaMemcpyAsync(ctx->d_tw, t32.data(), sizeof(float2) * N, cudaMemcpyHostToDevice, ctx->st);
         cudaStreamSynchronize(ctx->st);
     }
+    tcg_timeout_flag();   // (looks its address up outside any capture)
     if (ctx->d_xtab) {
         std::vector<unsigned char> tab(xdft_table_bytes());
         xdft_table(N, n, tab.data());
-        tcg_timeout_flag();   // (looks its address up outside any capture)
         cudaMemcpyAsync(ctx->d_xtab, tab.data(), tab.size(), cudaMemcpyHostToDevice, ctx->st);
         cudaStreamSynchronize(ctx->st);
     }
@@ -2117,6 +2117,7 @@ roks_status roks_set_preconditioner(roks_ctx* ctx, int kind, const float* params
 roks_status roks_precondition(roks_ctx* ctx, const void* grad, int64_t ld, void* out, float* feats) {
     if (!ctx) return ROKS_EINVAL;
     if (!grad || !out || ld < ctx->npw) return fail(ctx, ROKS_EINVAL, "bad gradient or output");
+    enter(ctx);
     const int npw = ctx->npw, nb = ctx->nb;
     cudaStream_t st = ctx->st;
     if (ctx->prec == ROKS_FP64) {
