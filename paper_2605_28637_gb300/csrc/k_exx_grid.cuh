@@ -268,8 +268,10 @@ template <typename T> constexpr size_t exx_acc_smem() {
 template <typename T> struct ExxPairCoef { T c[3][3]; };
 template <typename V>
 __device__ __forceinline__ void exx_async(V* dst, const V* src) {
+    // (memory: the slot's earlier values are read, and X written, before the copy is issued)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "n"(sizeof(V)));
+                 "n"(sizeof(V))
+                 : "memory");
 }
 template <typename T>
 __global__ void __launch_bounds__(kExxAccThreads, sizeof(T) == 4 ? 4 : 2)

@@ -38,3 +38,18 @@ def test_shared_memory_is_asked_for_at_every_launch():
         assert calls == (1 if path.endswith("roks_impl.cuh") else 0), path
         # no flag stands before the asking
         assert not re.search(r"static bool \w+ = false;", text), path
+
+
+def test_copies_in_assembly_are_ordered_with_memory():
+    """Without the clobber the compiler may move the reads of a ring's slot past
+    the copy that overwrites it."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = source(os.path.basename(path))
+        for m in re.finditer(r"asm volatile\(", text):
+            depth, i = 1, m.end()
+            while depth:                                   # to the closing parenthesis
+                depth += {"(": 1, ")": -1}.get(text[i], 0)
+                i += 1
+            body = text[m.end():i]
+            if "cp.async" in body:
+                assert '"memory"' in body, (path, body)
