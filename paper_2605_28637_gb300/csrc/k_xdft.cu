@@ -72,7 +72,10 @@ constexpr uint32_t XD_WAIT = 1u << 26;
 __host__ __device__ constexpr size_t xd_smem(int nmax, bool staged) {
     return xd_abytes(nmax) + XD_TAB + (staged ? 1024 * (2 * nmax + 1) : 0) + 1024;
 }
-constexpr size_t XD_SMEM_HALF = 112 * 1024;          // what lets two blocks share an SM
+// what lets two blocks share an SM's 228 KB: 1 KB of each is the system's, a
+// little more their static arrays
+constexpr size_t XD_SMEM_HALF = 111 * 1024;
+constexpr size_t XD_SMEM_MAX = xd_smem(29, true);    // the largest sphere, 120^3
 // 1 + what a sum of the apply's inverse and forward products loses to the
 // truncating additions, as far as it shows in F (alpha: 2^-23 each; F's
 // error against 64 bits is 1.39e-7 without, 1.21e-7 with, of the register
@@ -225,10 +228,12 @@ __device__ __forceinline__ void stage_planes(float2* raw, const CUtensorMap* tm,
 // place into the forward product's A (each thread overwrites the columns it
 // has read), and the forward sums take the other 128 columns.  ST: the next
 // tile's planes stream into shared memory meanwhile (where two blocks still
-// fit an SM); otherwise they are loaded when their tile begins.  (One block
-// of 512 threads with all x at once and the next tile's input split beside
-// the forward products left every phase's latency in the open: 1.67 ms at
-// mgo-120, against the two blocks' 1.22.)
+// fit an SM, nmax <= 21); otherwise they are loaded when their tile begins
+// (staged in one block per SM 387 us at 160 bands on 96^3, nmax 22; loaded 293;
+// the register transforms 372).  (One block
+// of 512 threads with all x at once and the next tile's input split beside the
+// forward products left every phase's latency in the open: 1.67 ms at mgo-120,
+// against the two blocks' 1.22.)
 template <int N, int KS, bool ST>
 __global__ void __launch_bounds__(256, 2) k_xdft_apply(int nmax, const __grid_constant__ CUtensorMap tm,
                                                        float2* __restrict__ Yp, const float* __restrict__ Vk,
@@ -623,6 +628,13 @@ static bool plane_map(CUtensorMap* tm, const Sphere& s, const float2* Yp, int nb
     (s.nmax < 16 ? (staged ? go(KERNEL<NN_, 1, true>) : go(KERNEL<NN_, 1, false>)) \
                  : (staged ? go(KERNEL<NN_, 2, true>) : go(KERNEL<NN_, 2, false>)))
 
+// Whether the density's planes are staged where only one block then fits an SM
+// (nmax >= 22).  It reads them twice, and on 120^3 those of two blocks don't stay
+// in L1 meanwhile: 160 bands, nmax 22 and 29, 353 and 384 us staged, 404 and 452
+// loaded (register transforms 451 and 474); on 96^3 nmax 22 they do, 230 and 224
+// (230), and loading has no fewer blocks in flight for few bands.
+static bool density_staged(const Sphere& s) { return xd_smem(s.nmax, true) <= XD_SMEM_HALF || s.N >= 120; }
+
 // Bands b0 .. b0 + nbb - 1, in place on their planes Yp; vmax: the largest
 // |V| of each class.
 void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, const float* vmax, int b0, int nbb,
@@ -634,7 +646,7 @@ void xdft_apply(const Sphere& s, const void* tab, float2* Yp, const float* Vk, c
     const bool staged = xd_smem(s.nmax, true) <= XD_SMEM_HALF && plane_map(&tm, s, Yp, nbb);
     const size_t sm = xd_smem(s.nmax, staged);
     auto go = [&](auto kernel) {
-        allow_smem(kernel, XD_SMEM_HALF);
+        allow_smem(kernel, XD_SMEM_MAX);
         roks::count_launch(), kernel<<<grid, 256, sm, st>>>(s.nmax, tm, Yp, Vk, vmax, static_cast<const uint4*>(tab),
                                                             b0, nbb, n_closed, scale, tcg_timeout_flag(),
                                                             wait_polls());
@@ -650,10 +662,10 @@ void xdft_density(const Sphere& s, const void* tab, const float2* Yp, double* rh
     const float2 sc = make_float2((float)scale, (float)(scale - (double)(float)scale));
     const dim3 grid((s.N * s.N + 127) / 128, ng);
     CUtensorMap tm{};
-    const bool staged = xd_smem(s.nmax, true) <= XD_SMEM_HALF && plane_map(&tm, s, Yp, nbb);
+    const bool staged = density_staged(s) && plane_map(&tm, s, Yp, nbb);
     const size_t sm = xd_smem(s.nmax, staged);
     auto go = [&](auto kernel) {
-        allow_smem(kernel, XD_SMEM_HALF);
+        allow_smem(kernel, XD_SMEM_MAX);
         roks::count_launch(), kernel<<<grid, 256, sm, st>>>(
                                   s.nmax, tm, Yp, reinterpret_cast<DS*>(rho3), reinterpret_cast<DS*>(slot),
                                   static_cast<const uint4*>(tab), b0, nbb, gs, n_closed, sc, cls_override,
