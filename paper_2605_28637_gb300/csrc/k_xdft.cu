@@ -588,6 +588,19 @@ bool xdft_takes(int N, int nmax) {
     return tcg_enabled() && (N == 72 || N == 96 || N == 120) && nmax <= sphere_prune_nmax(N);
 }
 
+// Whether so many bands at once take them.  A block sets up its table and
+// tensor memory first, which pays from some 1.7 million grid points on (apply and
+// density in us, registers and tensor cores: 72^3, nmax 17, one band 9.0, 12.1 and
+// 11.2, 15.1, six 14.2, 14.1 and 15.3, 17.3; 96^3, nmax 14, one 10.1, 10.2 and
+// 13.2, 15.4, two 12.0, 11.0 and 17.3, 16.4; 120^3, nmax 20, one 13.3, 12.2 and
+// 18.5, 17.4).  The density of the one sphere of 96^3 whose planes are neither
+// staged nor stay in L1 (nmax 23) takes them up to 32 bands (12 bands 29.8 us,
+// registers 33.8; 42 bands 76.8 and 74.7; 160 bands 242 and 230).
+bool xdft_apply_takes(const Sphere& s, int nbb) { return (int64_t)s.N * s.N * s.N * nbb >= 1700000; }
+bool xdft_density_takes(const Sphere& s, int nbb) {
+    return xdft_apply_takes(s, nbb) && (s.N != 96 || s.nmax < 23 || nbb <= 32);
+}
+
 size_t xdft_table_bytes() { return XD_TAB; }
 
 // Image of cos and sin of 2 pi i x / N, times 2^10, as FP16 hi and lo: element

@@ -337,7 +337,7 @@ struct Impl {
         const Sphere s = sphere(ctx);
         const double scale = 1.0 / ctx->omega;
         if constexpr (sizeof(T) == 4) {
-            if (ctx->d_xtab && part_sel == 0 && nbb > 0) {
+            if (ctx->d_xtab && part_sel == 0 && nbb > 0 && xdft_density_takes(s, nbb)) {
                 const int gs = (nbb + ngroups - 1) / ngroups, ng = (nbb + gs - 1) / gs;
                 xdft_density(s, ctx->d_xtab, Yp, rho3, slot, gs, ng, b0, nbb, n_closed, scale, cls_override,
                              ctx->st);
@@ -355,7 +355,7 @@ struct Impl {
         const T scale = T(1.0 / (double(ctx->N) * ctx->N * ctx->N));
         const T* Vk = static_cast<const T*>(ctx->d_Vk);
         if constexpr (sizeof(T) == 4) {
-            if (ctx->d_xtab && !Xx) {
+            if (ctx->d_xtab && !Xx && xdft_apply_takes(s, nbb)) {
                 auto run = [&](int first, int count) {
                     xdft_apply(s, ctx->d_xtab, Yp + (int64_t)(first - b0) * s.np * s.N * s.N, Vk, ctx->d_vmax, first,
                                count, n_closed, scale, ctx->st);

@@ -137,6 +137,8 @@ void band_density_reduce(int N, int ng, const double* slot, double* rho3, cudaSt
 // FP32, N = 72, 96, 120, spheres that fit the pruned first passes.  tab: the
 // transform's table (xdft_table_bytes(), filled on the host by xdft_table).
 bool xdft_takes(int N, int nmax);
+bool xdft_apply_takes(const Sphere& s, int nbb);
+bool xdft_density_takes(const Sphere& s, int nbb);
 size_t xdft_table_bytes();
 void xdft_table(int N, int nmax, void* host);
 // band_x_apply without exchange fields or a split band; vmax[class]: an upper
