@@ -47,8 +47,8 @@
 //   warp 1      one thread issues the 24 MMAs of a stage (M = 128, N = tn,
 //               K = 16) into one of two accumulators, 128 columns for the
 //               real parts and 128 for the imaginary parts;
-//   warps 4-11  drain: lane quadrant warp % 4, 64 complex columns each (128
-//               sums a thread: the first warpgroup gives them registers).
+//   warps 4-11  drain: lane quadrant warp % 4, up to 64 complex columns each
+//               (128 sums a thread: the first warpgroup gives them registers).
 // Every wait is bounded (the context's wait cap); a wait that gives up sets
 // a device flag and the CTA winds down: copies and MMAs in flight are waited
 // for with the default bound before the tensor memory is freed.
@@ -277,7 +277,11 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         // ------------------------------------------------ drain
         const int q = warp & 3;               // lane quadrant
-        const int cg = 64 * ((warp - 4) >> 2);   // complex columns cg .. cg + 63
+        // complex columns cg .. cg + ncol - 1: the tile's groups of 16 shared out
+        // between the two warpgroups (64 to the first and the rest to the second
+        // made half stages of 80-column tiles wait for the drain)
+        const int half = 16 * ((sk.tn / 16 + 1) / 2);
+        const int cg = warp < 8 ? 0 : half, ncol = warp < 8 ? half : sk.tn - half;
         const int r = 32 * q + lane;          // tile row
         float2 re[32], im[32];                // column pairs
 #pragma unroll
@@ -295,22 +299,21 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
             if (NN && beta != 0.f && left == total_stages && (lane & 15) == 0) {
                 // a tile's first stage: its Cin on the way to L2
                 const int no = (t_cur % sk.fast) * sk.tn + cg, m = (t_cur / sk.fast) * GB_M + r;
-                const int nc = min(sk.tn - cg, N - no);
+                const int nc = min(ncol, N - no);
                 for (int j = 0; j < nc && m < M; ++j)
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(Cin + (int64_t)(no + j) * ldcin + m));
             }
-            if (cg < sk.tn) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float v[16], w[16];
-                    tc::tmem_ld16_nowait(ta + 16 * c, v);
-                    tc::tmem_ld16_nowait(ta + 128 + 16 * c, w);
-                    tc::tmem_wait_ld();
+            for (int c = 0; c < 4; ++c) {
+                if (16 * c >= ncol) break;
+                float v[16], w[16];
+                tc::tmem_ld16_nowait(ta + 16 * c, v);
+                tc::tmem_ld16_nowait(ta + 128 + 16 * c, w);
+                tc::tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        re[8 * c + j] = __fadd2_rn(re[8 * c + j], make_float2(v[2 * j], v[2 * j + 1]));
-                        im[8 * c + j] = __fadd2_rn(im[8 * c + j], make_float2(w[2 * j], w[2 * j + 1]));
-                    }
+                for (int j = 0; j < 8; ++j) {
+                    re[8 * c + j] = __fadd2_rn(re[8 * c + j], make_float2(v[2 * j], v[2 * j + 1]));
+                    im[8 * c + j] = __fadd2_rn(im[8 * c + j], make_float2(w[2 * j], w[2 * j + 1]));
                 }
             }
             tc::fence_before_sync();
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                 if (NN) {
                     const int m = (t_cur / sk.fast) * GB_M + r;
                     const int no = (t_cur % sk.fast) * sk.tn + cg;
-                    const int nc = min(sk.tn - cg, N - no);   // this warp's columns
+                    const int nc = min(ncol, N - no);   // this warp's columns
                     if (m < M) {
                         // 32 columns at a time, every load before the first store
                         // (Cin may be Cout, so the compiler keeps their order: one
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
                     float2* Pp = part + (((int64_t)blockIdx.x * sk.maxseg + seg) * sk.tn + cg) * GB_M + r;
 #pragma unroll
                     for (int j = 0; j < 64; ++j)
-                        if (cg + j < sk.tn)
+                        if (j < ncol)
                             Pp[(int64_t)j * GB_M] = (j & 1) ? make_float2(re[j >> 1].y, im[j >> 1].y)
                                                             : make_float2(re[j >> 1].x, im[j >> 1].x);
                 }
