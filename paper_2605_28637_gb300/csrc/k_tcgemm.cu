@@ -698,13 +698,18 @@ bool tcg_keep_images() {
     return on == 1;
 }
 
-// Where the tensor cores take over from the streamed FP32 kernels: from 32
-// bands on.  An MMA costs little less for 32 columns than for 64, so that is
-// where P^H Psi breaks even (32 bands, 160 projectors, 5600 plane waves 19 us
-// both ways; 42 x 172 x 34,265 62 us streamed, 57 here; 63 bands, 320
-// projectors 43 and 27) and P (D B) gains (26 and 25; 67 and 44; 68 and 33).
+// Where the tensor cores take over from the streamed FP32 kernels.  P (D B) gains
+// from 32 columns on (42 x 172 x 34,265 67 us streamed, 44 here; 63 bands, 320
+// projectors 68 and 33; 32 bands, 160 projectors, 5600 plane waves 25 and 26).
+// P^H Psi splits Psi first, and an MMA costs little less for 32 columns than for
+// 64: from 8000 outputs on (9,795 plane waves, 216 x 42 43 us and 34, 144 x 56 46
+// and 31), in sums of 20,000 from 6000 on (144 x 48 43 and 43 at 21,823, 82 and 74
+// at 52,923); 144 x 36 is 25 and 34 us at 9,795 plane waves, 50 and 54 at 35,033.
 // Fewer than 128 rows (the bands against each other) leave an M tile half empty.
-bool tcg_cn_takes(int M, int N, int K) { return tcg_enabled() && M >= 128 && N >= 32 && K >= 1024; }
+bool tcg_cn_takes(int M, int N, int K) {
+    return tcg_enabled() && M >= 128 && N >= 32 && K >= 1024 &&
+           ((int64_t)M * N >= 8000 || ((int64_t)M * N >= 6000 && K >= 20000));
+}
 bool tcg_nn_takes(int M, int N, int K) { return tcg_enabled() && M >= 4096 && N >= 32 && K >= 64; }
 
 size_t tcg_image_bytes(int rows, int cols) {
