@@ -29,6 +29,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <atomic>
+
 #include <cstdlib>
 #include <mutex>
 
@@ -495,6 +497,47 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 uint32_t g_wait_polls = ST_WAIT;
 
 }  // namespace
+
+// The current context's number, never used twice in a process (0: not to be had)
+static unsigned long long context_id() {
+    static PFN_cuCtxGetId_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PFN_cuCtxGetId_v12000>(p);
+        else
+            cudaGetLastError();
+    });
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// Asking takes 1 to 2 us, a twentieth of a small call's launches; a context's
+// number some 20 ns.  A table of kernels and the context each was last asked for
+// in (another device's, or one made after a reset, asks again); `bytes` is a
+// constant of the kernel.
+cudaError_t ask_smem(const void* kernel, size_t bytes) {
+    struct Entry {
+        std::atomic<const void*> kernel{nullptr};
+        std::atomic<unsigned long long> context{0};
+    };
+    constexpr unsigned N = 1024;
+    static Entry table[N];
+    const unsigned long long id = context_id();
+    Entry* e = nullptr;
+    unsigned h = (unsigned)(reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u >> 22;
+    for (unsigned n = 0; id && !e && n < N; ++n, h = (h + 1) % N) {
+        const void* k = nullptr;
+        if (table[h].kernel.compare_exchange_strong(k, kernel) || k == kernel) e = &table[h];
+    }
+    if (e && e->context.load(std::memory_order_acquire) == id) return cudaSuccess;
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e && err == cudaSuccess) e->context.store(id, std::memory_order_release);
+    return err;
+}
 
 // Tiled map of 64-bit words, dims[0] contiguous, strides (bytes) of the others
 bool tensor_map_words(CUtensorMap* map, const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides,

@@ -26,13 +26,13 @@ constexpr int kThreads = 256;
 
 // Lets launches of a kernel have up to `bytes` of dynamic shared memory (the
 // kernel's largest, so that calls of different sizes do not lower each other's
-// limit).  Asked for at every launch: the limit belongs to the current device's
-// context.  The 48 KB that a launch has without asking hold the kernel's static
-// arrays too, up to 8 KB here: hence 40.
+// limit).  The 48 KB that a launch has without asking hold the kernel's static
+// arrays too, up to 8 KB here: hence 40.  The limit belongs to a context: asked
+// for once in each (k_stream.cu).
+cudaError_t ask_smem(const void* kernel, size_t bytes);
 template <typename K>
 inline cudaError_t allow_smem(K kernel, size_t bytes) {
-    return bytes <= 40 * 1024 ? cudaSuccess
-                              : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return bytes <= 40 * 1024 ? cudaSuccess : ask_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
 // Threads of the x-stage apply: for N = 96 (radix 12 then 8 over 32 lines:
 // 256 and 384 butterflies) 128 threads take 2 and 3 butterflies each with

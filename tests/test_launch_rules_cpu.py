@@ -29,13 +29,13 @@ def test_the_potentials_bound_is_cleared_only_where_they_are_written():
     assert len(re.findall(r"\bvmax\b", body)) == 3       # the parameter and that line
 
 
-def test_shared_memory_is_asked_for_at_every_launch():
+def test_shared_memory_is_asked_for_in_every_context():
     """The limit belongs to the context of the current device: a flag that
     remembers having asked refuses the launches on the next device."""
     for path in glob.glob(os.path.join(CSRC, "*.cu*")):
         text = source(os.path.basename(path))
         calls = len(re.findall(r"cudaFuncSetAttribute\(", text))
-        assert calls == (1 if path.endswith("roks_impl.cuh") else 0), path
+        assert calls == (1 if path.endswith("k_stream.cu") else 0), path
         # no flag stands before the asking
         assert not re.search(r"static bool \w+ = false;", text), path
 
