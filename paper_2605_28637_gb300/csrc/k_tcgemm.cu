@@ -17,14 +17,16 @@
 // accumulator, the small cross terms first, and the drain warps add its result
 // into FP32 sums in registers (round to nearest).  A B: every stage (32 complex
 // K).  A^H B, whose sums are a thousand stages long: every half stage, and no
-// sum in registers goes on for more than GB_PIECE stages.  (Drained by the stage,
-// norms come out 2.3e-7 low; by half stages 0.8e-7, in segments 0.6e-7, 1.2e-7 in
-// the TF32 form.  At mgo-120, errors of F and of a DIIS step's psi: half stages
-// in one sum 1.40e-7 and 1.79e-7, quarter stages, whose longer sums lose more
-// than the shorter accumulations gain, 1.65e-7 and 2.5e-7, half stages in
-// segments 1.11e-7 and 1.50e-7; the TF32 form 1.48e-7 and 2.16e-7.  That takes
-// 1.5% of an apply's time, two thirds of it for the segments.)  Nothing is
-// scaled to give back what is lost: sums without truncation are exact.
+// sum in registers goes on for more than GB_PIECE stages: it ends as a segment,
+// and the segments are added with compensation.  (Drained by the stage, norms
+// come out 2.3e-7 low; by half stages 0.8e-7; 1.2e-7 in the TF32 form this
+// replaces.  At mgo-120, errors of F and of a DIIS step's psi: half stages in one
+// sum 1.40e-7 and 1.79e-7, in segments of at most 128, 96 and 64 stages 1.18e-7
+// and 1.77e-7, 1.15e-7 and 1.52e-7, 1.11e-7 and 1.50e-7; the TF32 form 1.48e-7 and
+// 2.16e-7.  Quarter stages, whose longer sums lose more than the shorter
+// accumulations gain, 1.65e-7 and 2.5e-7.  It takes 0.9% of an apply's time there,
+// 1.4% with segments of 64.)  Nothing is scaled to give back what is lost: sums
+// without truncation are exact.
 //
 // Images.  A block X (rows x cols, column major) is split once per use, by
 // k_tcg_split, into an image in global memory that the MMAs can read as it
@@ -79,7 +81,7 @@ constexpr int GB_KC = 32;     // complex K per stage
 constexpr int GB_ST = 3;      // stages
 constexpr int GB_ACC = 2;     // accumulators (256 tensor-memory columns each)
 constexpr int GB_DRAIN = 8;   // drain warps
-constexpr int GB_PIECE = 64;  // A^H B: most stages of a running sum (a segment)
+constexpr int GB_PIECE = 96;  // A^H B: most stages of a running sum (a segment)
 constexpr int GB_THREADS = (4 + GB_DRAIN) * 32;
 constexpr uint32_t GB_ABYTES = GB_M * GB_KC * 8;      // 32 KB
 constexpr uint32_t GB_SLOT = 2 * GB_ABYTES;           // A, then B (tn x KC x 8 bytes)
@@ -110,9 +112,6 @@ __device__ __forceinline__ void give_up(volatile int* failed) {
     g_tcg_timeout = 1;
 }
 
-// segments of so many stages of a tile
-__host__ __device__ constexpr int segments(int stages) { return (stages + GB_PIECE - 1) / GB_PIECE; }
-
 // 2^e as a float, e in [-126, 127]
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -120,7 +119,7 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) 
 // * A^H B, stream-K: CTA c takes the units c len .. (c + 1) len - 1 of the
 //   (tile, stage) sequence, stage fastest (tile t: M tile t % fast, N tile t /
 //   fast), and writes the partial sums of each tile that it touches, a segment
-//   for every GB_PIECE stages of it, to its slots c * maxseg + 0, 1, ...;
+//   for every `piece` stages of it, to its slots c * maxseg + 0, 1, ...;
 // * A B, persistent: units = tiles, CTA c takes the whole tiles c, c + ctas,
 //   ... (tile t: N tile t % fast, M tile t / fast), its pipeline running on
 //   across them, and writes each tile's result as it completes.
@@ -128,6 +127,9 @@ struct SkPlan {
     int64_t units = 0, len = 0;
     int ctas = 0, maxseg = 0, fast = 0;
     int tn = 0;   // complex columns of a tile (a multiple of 16)
+    int piece = 0;   // A^H B: stages of a segment
+    // segments of so many stages of a tile
+    __host__ __device__ int segments(int stages) const { return (stages + piece - 1) / piece; }
 };
 
 template <bool NN>
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(GB_THREADS, 1)
             // sums go out (NN: the result; CN: the partial sums to the segment
             // slot) and restart
             --left;
-            if (left == 0 || e == DS * ns - 1 || (!NN && ++in_seg == GB_PIECE)) {
+            if (left == 0 || e == DS * ns - 1 || (!NN && ++in_seg == sk.piece)) {
                 if (NN) {
                     const int m = (t_cur / sk.fast) * GB_M + r;
                     const int no = (t_cur % sk.fast) * sk.tn + cg;
@@ -550,7 +552,7 @@ __global__ void __launch_bounds__(256) k_tcg_reduce_sk(int M, int N, int mt, int
         const int64_t off = (int64_t)(n % sk.tn) * GB_M + (m % GB_M);
         const int64_t ta = (int64_t)t * T;
         const int c0 = (int)(ta / sk.len), c1 = (int)((ta + T - 1) / sk.len);
-        if (sk.len <= GB_PIECE) {
+        if (sk.len <= sk.piece) {
 #pragma unroll 4
             for (int c = c0 + wg; c <= c1; c += RG) {
                 // a run that starts before the tile has it further on
@@ -564,8 +566,8 @@ __global__ void __launch_bounds__(256) k_tcg_reduce_sk(int M, int N, int mt, int
                 // the segments of the run's tiles before this one, then this one's
                 const int64_t u0 = c * sk.len;
                 const int tb = (int)(u0 / T), sb = (int)(u0 - (int64_t)tb * T);
-                const int seg = tb < t ? segments(T - sb) + (t - tb - 1) * segments(T) : 0;
-                const int ns = segments((int)(min(u0 + sk.len, ta + T) - max(u0, ta)));
+                const int seg = tb < t ? sk.segments(T - sb) + (t - tb - 1) * sk.segments(T) : 0;
+                const int ns = sk.segments((int)(min(u0 + sk.len, ta + T) - max(u0, ta)));
                 const float2* p = part + ((int64_t)c * sk.maxseg + seg) * sk.tn * GB_M + off;
 #pragma unroll 4
                 for (int q = 0; q < ns; ++q, p += sk.tn * GB_M) {
@@ -629,9 +631,12 @@ SkPlan cn_plan(int M, int N, int K, int waves_x2) {
     p.ctas = (int)std::min<int64_t>(sm_count() * waves_x2 / 2, std::max<int64_t>(1, p.units / 4));
     p.len = (p.units + p.ctas - 1) / p.ctas;
     p.ctas = (int)((p.units + p.len - 1) / p.len);
-    // (long runs: whole tiles, what is left over, and a short segment at either end)
-    p.maxseg = p.len <= GB_PIECE ? (int)((p.len + T - 1) / T) + 1
-                                 : (int)(p.len / T) * segments(T) + (int)(p.len % T) / GB_PIECE + 3;
+    // segments of equal length; long runs: whole tiles, what is left over, and a
+    // short segment at either end
+    const int n = (int)((p.len + GB_PIECE - 1) / GB_PIECE);
+    p.piece = (int)((p.len + n - 1) / n);
+    p.maxseg = n == 1 ? (int)((p.len + T - 1) / T) + 1
+                      : (int)(p.len / T) * p.segments(T) + (int)(p.len % T) / p.piece + 3;
     return p;
 }
 

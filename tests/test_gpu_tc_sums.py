@@ -3,7 +3,7 @@
 * Orbitals that are single plane waves: no product is truncated and no sum
   rounded, the overlap is 1 and the orthonormalisation gives back its input, bit
   for bit.
-* Runs of the (tile, stage) sequence around and beyond the 64 stages of a
+* Runs of the (tile, stage) sequence below and beyond the 96 stages of a
   segment (256 bands: 18 stages a run; 512 and 640: 72 and 113 of a tile's 682,
   tiles cut by runs and runs over two tiles), against FP64 torch.  Tolerance: an element of
   the overlap is a sum of products of 22 significant bits (2^-22, random) in
