@@ -7,7 +7,8 @@
 // fixed order), a second kernel sums the partials in a fixed order with
 // two-sum compensation, and an Adam kernel updates the FP32 master weights.
 // Inference (the fused preconditioner inside the PCG step) takes the weights
-// rounded to BF16 and runs the 64 x 64 layer on the tensor cores.
+// rounded to BF16 and runs the 64 x 64 layer on the tensor cores (FP64 contexts:
+// in FP32).
 //
 // Parameter layout (4481 floats): W1 (64 x 3, row major), b1 (64), W2
 // (64 x 64, row major), b2 (64), w3 (64), b3 (1).
@@ -15,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "roks_grid.cuh"
 #include "roks_mlp.cuh"
@@ -484,32 +486,77 @@ __global__ void k_mlp_adam(int np, float* __restrict__ p, float* __restrict__ m,
     p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
 }
 
+// Network output of one row on the FP32 units, in FP32 throughout (BF16-rounded
+// weights w in shared memory).  FP64 contexts take it: their results hold 1e-9
+// against each other from build to build, and products of 22 significant bits
+// move them by 5e-8 (though no further from 64 bits: 7.2e-8, 7.4e-8 here).  14,000
+// plane waves x 40 bands: 222 us, 138 on the tensor cores.
+struct SimtShared {
+    float w[(kMlpParams + 3) / 4 * 4];
+};
+// rows (and threads) of a block of the fused preconditioner
+template <typename T> __host__ __device__ constexpr int net_rows() { return sizeof(T) == 4 ? NT : 256; }
+__device__ __forceinline__ float simt_eval(const float* w, float u0, float u1, float u2) {
+    float h1[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+        float z = w[OB1 + j];
+        z = fmaf(w[OW1 + 3 * j + 0], u0, z);
+        z = fmaf(w[OW1 + 3 * j + 1], u1, z);
+        z = fmaf(w[OW1 + 3 * j + 2], u2, z);
+        h1[j] = tanhf(z);
+    }
+    float s = w[OB3];
+#pragma unroll 4
+    for (int k = 0; k < H; ++k) {
+        const float4* row = reinterpret_cast<const float4*>(w + OW2 + H * k);
+        float z = w[OB2 + k];
+#pragma unroll
+        for (int q = 0; q < H / 4; ++q) {
+            const float4 c = row[q];
+            z = fmaf(c.x, h1[4 * q + 0], z);
+            z = fmaf(c.y, h1[4 * q + 1], z);
+            z = fmaf(c.z, h1[4 * q + 2], z);
+            z = fmaf(c.w, h1[4 * q + 3], z);
+        }
+        s = fmaf(w[OW3 + k], tanhf(z), s);
+    }
+    return s;
+}
+
 // Fused preconditioner of the PCG step: out = K m g_I with K the TPA factor
 // (X_n = 1.5 T_n, T_n the kinetic energy of the residual) and m the network's
 // multiplier on the features (log1p(x), log1p(|g|/rms_n), eps_n); m = 1 while
-// the correction is suspended (sc->mlp_off > 0) or no weights are set.
+// the correction is suspended (sc->mlp_off > 0) or no weights are set.  The
+// network: on the tensor cores in mixed contexts, simt_eval in FP64 ones.
 template <typename T>
-__global__ void __launch_bounds__(NT) k_precond_mlp(int npw, const c2<T>* __restrict__ gI, int64_t ld,
-                                                    const T* __restrict__ g2h, const double* __restrict__ sums,
-                                                    int nb, const double2* __restrict__ Theta,
-                                                    const double* __restrict__ wband,
-                                                    const float* __restrict__ params, const PcgScalars* sc,
-                                                    c2<T>* __restrict__ out, int64_t ldo, int* timeout,
-                                                    uint32_t wcap) {
-    __shared__ __align__(128) NetShared S;
+__global__ void __launch_bounds__(net_rows<T>())
+    k_precond_mlp(int npw, const c2<T>* __restrict__ gI, int64_t ld,
+                  const T* __restrict__ g2h, const double* __restrict__ sums,
+                  int nb, const double2* __restrict__ Theta,
+                  const double* __restrict__ wband,
+                  const float* __restrict__ params, const PcgScalars* sc,
+                  c2<T>* __restrict__ out, int64_t ldo, int* timeout,
+                  uint32_t wcap) {
+    constexpr bool TC = sizeof(T) == 4;
+    __shared__ __align__(128) std::conditional_t<TC, NetShared, SimtShared> S;
     __shared__ float band[5];   // 1/X, -2/X, 1/T, 1/rms, eps
     const bool use = params != nullptr && (sc == nullptr || sc->mlp_off <= 0.0);
-    if (use) net_setup(S, params, true);
-    // tiles of 128 rows of one band; a block takes a run of them, so that the
-    // band's FP64 divisions are rare
-    const int per = (npw + NT - 1) / NT;
+    if (use) {
+        if constexpr (TC) net_setup(S, params, true);
+        else load_params(params, S.w, true);   // (ordered by the first band's barrier)
+    }
+    // tiles of one row a thread of one band; a block takes a run of them, so that
+    // the band's FP64 divisions are rare (FP64: one tile, like its weights)
+    constexpr int R = net_rows<T>();
+    const int per = (npw + R - 1) / R;
     const int64_t tiles = (int64_t)per * nb;
     const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
     int n = -1;
     bool ok = true;
     uint32_t phase = 0;
     for (int64_t t = t0; t < t1; ++t) {
-        const int nt = (int)(t / per), g = (int)(t - (int64_t)nt * per) * NT + threadIdx.x;
+        const int nt = (int)(t / per), g = (int)(t - (int64_t)nt * per) * R + threadIdx.x;
         if (nt != n) {
             n = nt;
             __syncthreads();
@@ -533,13 +580,16 @@ __global__ void __launch_bounds__(NT) k_precond_mlp(int npw, const c2<T>* __rest
         float K = band[1] * num / (num + 16.f * x * x * x * x);
         if (use) {
             const float amp = sqrtf(float(a.x) * float(a.x) + float(a.y) * float(a.y));
-            const float s = net_eval<false>(S, log1pf(gh * band[2]), log1pf(amp * band[3]), band[4], phase++, ok,
-                                            timeout, wcap);
+            const float u0 = log1pf(gh * band[2]), u1 = log1pf(amp * band[3]);
+            float s;
+            if constexpr (TC) s = net_eval<false>(S, u0, u1, band[4], phase++, ok, timeout, wcap);
+            else s = simt_eval(S.w, u0, u1, band[4]);
             K *= ok ? expf(fminf(fmaxf(s, -3.f), 3.f)) : __int_as_float(0x7fffffff);
         }
         if (g < npw) out[(int64_t)n * ldo + g] = mk<T>(T(K) * a.x, T(K) * a.y);
     }
-    if (use) net_done(S);
+    if constexpr (TC)
+        if (use) net_done(S);
 }
 
 template <typename T>
@@ -610,7 +660,10 @@ template <typename T>
 void precondition_mlp(int npw, int nb, const c2<T>* gI, int64_t ld, const T* g2h, const double* sums,
                       const double2* Theta, const double* wband, const float* params, const PcgScalars* sc,
                       c2<T>* out, int64_t ldo, cudaStream_t st) {
-    roks::count_launch(), k_precond_mlp<T><<<net_blocks((int64_t)((npw + NT - 1) / NT) * nb), NT, NET_PAD, st>>>(
+    constexpr bool TC = sizeof(T) == 4;
+    constexpr int R = net_rows<T>();
+    const int64_t tiles = (int64_t)((npw + R - 1) / R) * nb;
+    roks::count_launch(), k_precond_mlp<T><<<TC ? net_blocks(tiles) : (int)tiles, R, TC ? NET_PAD : 0, st>>>(
                               npw, gI, ld, g2h, sums, nb, Theta, wband, params, sc, out, ldo, tcg_timeout_flag(),
                               wait_polls());
 }
