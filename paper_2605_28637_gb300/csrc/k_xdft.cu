@@ -33,8 +33,7 @@
 // bound, that element times 4 (nmax + 1) times the class's largest |V|) and
 // split as hi + lo, as the table is; a product is lo.hi + hi.lo + hi.hi, and
 // the last additions are those with the lowest frequencies, which are the
-// largest.  What the truncating additions of the tensor cores take is given
-// back by the factor XD_GAIN.
+// largest.
 //
 // A tile is 128 consecutive lines of a band, a thread's line its
 // tensor-memory lane; the warpgroups of a block share out the chunks of 8
@@ -76,13 +75,14 @@ __host__ __device__ constexpr size_t xd_smem(int nmax, bool staged) {
 // little more their static arrays
 constexpr size_t XD_SMEM_HALF = 111 * 1024;
 constexpr size_t XD_SMEM_MAX = xd_smem(29, true);    // the largest sphere, 120^3
-// 1 + what a sum of the apply's inverse and forward products loses to the
-// truncating additions, as far as it shows in F (alpha: 2^-23 each; F's
-// error against 64 bits is 1.39e-7 without, 1.21e-7 with, of the register
-// transforms' 1.50e-7, at 430 bands of mgo-120).  
-constexpr float XD_GAIN = 1.f + 1.1920929e-7f;
-// The same for |psi|^2, which twice an inverse product's loss reaches; it goes
-// into the low word of the sums.
+// What the truncating additions of an inverse product take from |psi|^2, as a
+// part of it, in the mean over orbitals of many plane waves: half a unit in the
+// last place of the sums, 2^-24.  It goes into the low word of the density
+// (without it every density of such orbitals is 6e-8 low, which energies show:
+// a DIIS step of mgo-120 2.6e-7 off 64 bits, 1.6e-7 with, 2.2e-7 with register
+// transforms; an orbital of so few plane waves that nothing is truncated comes
+// out half an FP32 unit high).  The apply's products are left as they are: F's
+// error is 1.39e-7, the register transforms' 1.50e-7 (430 bands of mgo-120).
 constexpr float XD_LOSS = 6e-8f;
 
 __device__ __forceinline__ float xpow2(int e) { return __int_as_float((e + 127) << 23); }
@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(256, 2) k_xdft_apply(int nmax, const __grid_co
             if (8 * (h + 2) <= nmax) store_chunk(A, comp, h + 2, r, s, ap1, am1);
             const float bound = mx * (4.f * (nmax + 1)) * vm[cls] * scale;
             const int e2 = below(bound, 14);
-            c0 = scale * xpow2(-e - XD_TSH) * xpow2(e2) * XD_GAIN;
-            sfw = xpow2(-e2 - XD_TSH) * XD_GAIN;
+            c0 = scale * xpow2(-e - XD_TSH) * xpow2(e2);
+            sfw = xpow2(-e2 - XD_TSH);
         }
         tc::fence_async_smem();
         tc::fence_before_sync();
