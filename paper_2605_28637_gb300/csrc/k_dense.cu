@@ -10,6 +10,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "roks_chol.cuh"
 #include "roks_impl.cuh"
 
@@ -128,11 +130,9 @@ __global__ void __launch_bounds__(256) k_gemm_cn(int M, int N, int K, int kchunk
         __syncthreads();
         const V* as = As + (t & 1) * KT * SA + ty * padgroup<RM>();
         const V* bs = Bs + (t & 1) * KT * SB + tx * padgroup<RN>();
-        // (FP64: a chunk of half a slice does not multiply the other half's zeros)
-        const int kc = sizeof(T) == 8 ? min(KT, kend - kbeg - t * KT) : KT;
-        for (int k8 = 0; k8 < kc; k8 += 8) {
-#pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
+        auto slice = [&](auto steps) {
+#pragma unroll 8
+            for (int kk = 0; kk < steps(); ++kk) {
                 V a[RM], b[RN];
 #pragma unroll
                 for (int i = 0; i < RM; ++i) a[i] = as[i];
@@ -145,7 +145,11 @@ __global__ void __launch_bounds__(256) k_gemm_cn(int M, int N, int K, int kchunk
 #pragma unroll
                     for (int j = 0; j < RN; ++j) mac_cn<T>(acc[i][j], a[i], b[j]);
             }
-        }
+        };
+        // FP64: a chunk of half a slice does not multiply the other half's zeros
+        // (both lengths unrolled: in steps of 8 a slice lost 3% at 8 bands)
+        if (sizeof(T) == 8 && kend - kbeg - t * KT <= KT / 2) slice(std::integral_constant<int, KT / 2>{});
+        else slice(std::integral_constant<int, KT>{});
         __syncthreads();
     }
     // stage the tile (column n at Cs[n TM + r]) and write it out along m
