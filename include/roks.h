@@ -444,9 +444,10 @@ ROKS_API roks_status roks_profile_read(roks_ctx* ctx, roks_profile_entry* out, i
  * current device (cudaGetSymbolAddress) before it launches anything; the
  * call synchronises its stream, so it is not for use under stream capture.
  * All calls share the array
- * and it keeps the last call's contents, so calls that overlap on the GPU
- * (different streams or threads at once) race; serialise them.
- * Limits: nbands <= 64 (ROKS_EINVAL beyond).  Synchronises the stream;
+ * and it keeps the last call's contents, so calls of several threads at once
+ * race; serialise them.  (Calls one after the other may be on any streams.)
+ * Limits: nbands <= 64 (ROKS_EINVAL beyond).  Synchronises the stream for its
+ * status; the last product may still run on it when the call returns.
  * ROKS_ENOTPOSDEF leaves psi unchanged. */
 ROKS_API roks_status roks_orthonormalize_noalloc(int precision, int npw, int nbands,
                                                  void* psi, int64_t ld, void* cuda_stream);

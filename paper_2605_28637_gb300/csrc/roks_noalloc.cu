@@ -10,6 +10,7 @@
 // GPU that loads the library holds it until the process exits.
 #include <cooperative_groups.h>
 
+#include <atomic>
 #include <cstddef>
 
 #include "../../include/roks.h"
@@ -43,12 +44,10 @@ cudaError_t scratch_address(unsigned char** out) {
 }
 
 // psi <- psi U in place, U upper triangular (nb x nb, FP64, column major).
-// A block owns 64 rows: it reads them into shared memory before writing.  A
-// failed pivot (flag) leaves psi as it is: the host learns of it afterwards.
+// A block owns 64 rows: it reads them into shared memory before writing.
 template <typename T>
 __global__ void __launch_bounds__(256) k_rows_times_upper(int npw, int nb, c2<T>* psi, int64_t ld,
-                                                          const double2* __restrict__ U, const int* flag) {
-    if (*flag) return;
+                                                          const double2* __restrict__ U) {
     using V = c2<T>;
     constexpr int RT = 64;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -171,14 +170,33 @@ __global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaThreads)
     }
 }
 
-// the call's status once its work is done
-roks_status result(const int* flag, cudaStream_t st) {
+// The call's status once its work is done.  The flag is zero between calls, as
+// the array is when it is loaded: whatever may have left it set clears it.
+roks_status broken(int* flag, cudaStream_t st) {
+    cudaMemsetAsync(flag, 0, sizeof(int), st);
+    return ROKS_ECUDA;
+}
+roks_status result(int* flag, cudaStream_t st) {
     int h = 0;
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
+        return broken(flag, st);
+    if (!h) return ROKS_OK;
+    if (cudaMemsetAsync(flag, 0, sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return ROKS_ECUDA;
-    return h ? ROKS_ENOTPOSDEF : ROKS_OK;
+    return ROKS_ENOTPOSDEF;
+}
+
+// The product of the last call may still read the scratch when that call has
+// returned.  On the same stream this one comes after it; on another the device
+// is waited for.  (Streams are told apart by their number, never used twice.)
+bool after_earlier_calls(cudaStream_t st) {
+    static std::atomic<unsigned long long> last{0};
+    unsigned long long id = 0;
+    if (cudaStreamGetId(st, &id) != cudaSuccess) return false;
+    const unsigned long long was = last.exchange(id);
+    return was == 0 || was == id || cudaDeviceSynchronize() == cudaSuccess;
 }
 
 template <typename T>
@@ -196,19 +214,23 @@ roks_status run(int npw, int nb, void* psi, int64_t ld, cudaStream_t st, unsigne
         k_orth_cluster<T><<<kNaCluster, kNaThreads, sm, st>>>(npw, nb, static_cast<V*>(psi), ld, flag);
         return result(flag, st);
     }
-    // the flag keeps the previous call's value: clear it first
-    if (cudaMemsetAsync(flag, 0, sizeof(int), st) != cudaSuccess) return ROKS_ECUDA;
+    if (!after_earlier_calls(st)) return ROKS_ECUDA;
     V* X = static_cast<V*>(psi);
     gemm_cn_capped<T>(nb, nb, npw, X, ld, X, ld, O, nb, part, kNaMaxChunks, st);
     cholesky_inverse(nb, O, Lw, LinvH, flag, st);
-    // psi is touched only if all before it was launched: the scratch holds an
-    // earlier call's L^{-H} otherwise
-    if (cudaGetLastError() != cudaSuccess) return ROKS_ECUDA;
+    // psi is touched only if all before it was launched (the scratch holds an
+    // earlier call's L^{-H} otherwise) and no pivot failed.  The status is read
+    // before the product, which runs while the caller goes on (FP64, 8 bands x
+    // 19,672 and 9 x 6245: 110 and 78 us, with the status last 124 and 91).
+    if (cudaGetLastError() != cudaSuccess) return broken(flag, st);
+    const roks_status status = result(flag, st);
+    if (status != ROKS_OK) return status;
     const size_t sm = sizeof(V) * ((size_t)nb * 64 + (size_t)nb * nb);
-    if (allow_smem(k_rows_times_upper<T>, sizeof(V) * kNaMaxBands * (64 + kNaMaxBands)) != cudaSuccess) return ROKS_ECUDA;
+    if (allow_smem(k_rows_times_upper<T>, sizeof(V) * kNaMaxBands * (64 + kNaMaxBands)) != cudaSuccess)
+        return broken(flag, st);
     count_launch();
-    k_rows_times_upper<T><<<(npw + 63) / 64, 256, sm, st>>>(npw, nb, X, ld, LinvH, flag);
-    return result(flag, st);
+    k_rows_times_upper<T><<<(npw + 63) / 64, 256, sm, st>>>(npw, nb, X, ld, LinvH);
+    return cudaGetLastError() == cudaSuccess ? ROKS_OK : ROKS_ECUDA;
 }
 
 }  // namespace

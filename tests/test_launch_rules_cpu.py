@@ -16,7 +16,9 @@ def test_noalloc_checks_its_launches_before_psi_is_multiplied():
     """A chain that failed leaves an earlier call's factor in the scratch."""
     run = source("roks_noalloc.cu")
     run = run[run.index("cholesky_inverse(nb"):run.index("k_rows_times_upper<T><<<")]
-    assert re.search(r"if \(cudaGetLastError\(\) != cudaSuccess\) return ROKS_ECUDA;", run)
+    assert re.search(r"if \(cudaGetLastError\(\) != cudaSuccess\) return broken\(flag, st\);", run)
+    # and no way out between them leaves the status flag set for the next call
+    assert "return ROKS_ECUDA" not in run
 
 
 def test_the_potentials_bound_is_cleared_only_where_they_are_written():
