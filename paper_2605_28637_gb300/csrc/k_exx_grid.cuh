@@ -50,7 +50,10 @@ namespace roks {
     }
 
 // Threads of the passes: with 54 = 9 x 6, tiles of 64 lines hold 384 and 576
-// butterflies, two and three rounds of 192 threads.
+// butterflies, two and three rounds of 192 threads (an apply of 40 bands 2.10 ms,
+// with 256 threads 2.14).  Elsewhere 256 against 192, the same apply: 32 0.56 and
+// 0.57, 72 4.39 and 4.59, 80 6.01 and 6.57, 96 (24 bands) 5.15 and 5.33; 192 would
+// be the better at 16, 24, 48, 60 and 64 by 1 to 4% and at 108 by 13%.
 __host__ __device__ constexpr int exx_threads(int m) { return m == 54 ? 192 : kThreads; }
 // lines of an x tile (consecutive y, z)
 __host__ __device__ constexpr int exx_lines(int m, size_t elem) { return m <= 80 && elem == 8 ? 64 : 32; }
@@ -258,7 +261,9 @@ __global__ void __launch_bounds__(kThreads) k_exx_z_mult(const c2<T>* __restrict
 // own slots of shared memory (W of up to 8 pairs, psi_n and X_n each), so no
 // thread waits for another.  288 threads at up to 56 registers (FP32): four
 // blocks an SM, and all points of M = 54 in one wave: 32 us a tile of 64 pairs
-// (loads into registers, 256 threads at 72, coefficients in FP64: 67).
+// (loads into registers, 256 threads at 72, coefficients in FP64: 67).  An apply
+// of 40 bands with 288 and with 256 threads: M = 54 2.10 ms and 2.14; 16 to 48 1 to
+// 2% longer, 60 to 72 1%, from 80 on the same.
 constexpr int kExxAccThreads = 288;
 template <typename T> constexpr size_t exx_acc_smem() {
     return sizeof(c2<T>) * 2 * (kExxTileMax + 2) * kExxAccThreads;

@@ -37,8 +37,9 @@ __device__ __forceinline__ void load_params(const float* __restrict__ p, float* 
     for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) w[i] = bf16 ? bf16_round(p[i]) : p[i];
 }
 
-// tanh of two values, relative error below 3e-7 (2.5 units in the last place):
-// x + x^3 P(x^2) up to 0.625, P the least-squares polynomial of degree 4
+// tanh of two values, relative error below 3e-7 (2.5 units in the last place), in
+// the form of Moshier's Cephes library, with coefficients of its own: x + x^3
+// P(x^2) up to 0.625, P the least-squares polynomial of degree 4
 // brought to equal ripples by Lawson's iteration (4.4e-9), and
 // 1 - 2 / (1 + e^{2|x|}) beyond, the two reciprocals from one (|x| is cut
 // off at 10, where tanh rounds to 1).  Half the instructions of two tanhf

@@ -583,7 +583,10 @@ int xd_sms() {
 // The grids whose kernels are instantiated, as far as their densities fit
 // them: 32 frequencies and 64 x is what the tables hold, and all of these
 // spheres are within it (nmax <= 29); larger spheres keep the register
-// transforms, as do the exchange's fields and the packed open pair.
+// transforms, as do the exchange's fields and the packed open pair.  48^3, which
+// the tables hold too, is faster in registers: half of its 64 x are empty (40
+// bands, nmax 11: density 18.8 us, 29.1 here, apply 20.4 both; 160 bands 45 and
+// 82, 61 and 59).
 bool xdft_takes(int N, int nmax) {
     return tcg_enabled() && (N == 72 || N == 96 || N == 120) && nmax <= sphere_prune_nmax(N);
 }
