@@ -192,11 +192,11 @@ roks_status result(int* flag, cudaStream_t st) {
 // returned.  On the same stream this one comes after it; on another the device
 // is waited for.  (Streams are told apart by their number, never used twice.)
 bool after_earlier_calls(cudaStream_t st) {
-    static std::atomic<unsigned long long> last{0};
+    static std::atomic<unsigned long long> last{0};   // 1 + the number, 0: no call yet
     unsigned long long id = 0;
     if (cudaStreamGetId(st, &id) != cudaSuccess) return false;
-    const unsigned long long was = last.exchange(id);
-    return was == 0 || was == id || cudaDeviceSynchronize() == cudaSuccess;
+    const unsigned long long was = last.exchange(id + 1);
+    return was == 0 || was == id + 1 || cudaDeviceSynchronize() == cudaSuccess;
 }
 
 template <typename T>

@@ -37,13 +37,13 @@ def test_status_starts_clear(bad, good, f64):
     assert np.abs(G.conj() @ G.T - np.eye(good[1])).max() < (1e-12 if f64 else 2e-6)
 
 
-def test_one_call_after_another_on_two_streams():
+def test_one_call_after_another_on_three_streams():
     """The product of a call may still run when it has returned; the next call, on
     another stream, must not change the scratch under it."""
     import torch
     roks = built()
     sizes = [(40000, 24), (30000, 17), (40000, 24), (900, 9), (40000, 30), (2000, 40)]
-    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    streams = [torch.cuda.Stream().cuda_stream, None, torch.cuda.Stream().cuda_stream]     # (None: the legacy stream)
     blocks = []
     for npw, nb in sizes:
         gen = torch.Generator("cuda").manual_seed(npw + nb)
@@ -51,7 +51,7 @@ def test_one_call_after_another_on_two_streams():
     torch.cuda.synchronize()
     for k, X in enumerate(blocks):
         roks.roks_orthonormalize_noalloc(roks.ROKS_FP64, X.shape[1], X.shape[0], X, X.shape[1],
-                                         streams[k % 2].cuda_stream)
+                                         streams[k % 3])
     torch.cuda.synchronize()
     for X in blocks:
         assert (X.conj() @ X.T - torch.eye(X.shape[0], device="cuda")).abs().max().item() < 1e-12
